@@ -174,11 +174,11 @@ typedef struct {
                        * every target by brute force and compare (tests;
                        * sph_list_info reports the result)                */
   int32_t pi_lanes;   /* threads that share one target in the list walk
-                       * (pi_variant 3-5): 0 (default: 1), 1, 2, 4 or 8;
-                       * thread k of a target takes the candidates at bit
-                       * positions k, k + lanes, ... of each chunk record and
-                       * the partial sums are added at the end, so the sums'
-                       * order (not the pair set) depends on it           */
+                       * (pi_variant 3-5): 0 (default: 8), 1, 2, 4 or 8;
+                       * thread k of a target takes the entries k, k +
+                       * lanes, ... of its list and the partial sums are
+                       * added at the end, so the sums' order (not the
+                       * pair set) depends on it                          */
   int32_t pair_once;  /* 1: the list walk (pi_variant 3-5) of an engine with
                        * the default physics (Eq 18 or no diffusion,
                        * Eq 21 viscosity, DBC) evaluates each pair once:
@@ -191,14 +191,9 @@ typedef struct {
                        * admitted a case with other physics) evaluate as
                        * with 0.  0 (default): every target sums its own
                        * pairs, deterministically                         */
-  int32_t wide_records; /* 1: neighbour-list records with a 32-bit first
-                       * index and no row code (the walk takes a record's
-                       * row from its first candidate's cell) at any size;
-                       * 0: only where the engine needs them, beyond 2^25
-                       * particles.  The default physics only (Eq 18 or no
-                       * diffusion, Eq 21 viscosity, DBC); the pair set and
-                       * the order of the sums are those of the narrow
-                       * records, so results are the same bit for bit    */
+  int32_t wide_records; /* 0 or 1, of no effect: lists hold 32-bit indices
+                       * at every size (it once chose between two record
+                       * forms, with the same results bit for bit)        */
 } sph_options;
 
 /* Last error message of the calling thread ("" if none). */

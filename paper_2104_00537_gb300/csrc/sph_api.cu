@@ -144,6 +144,14 @@ void fill_const(const sph_case_params &p, const sph_particles &parts, const Grid
   C.inv_csf = (float)(1.0 / g.cs);
   C.inv_gamma = (float)(1.0 / p.gamma);
   const double kB = -p.gamma / (p.cs0 * p.cs0);  // -rho0 / B
+  C.unit = (float)(g.cs / 536870912.0);  // cs / 2^29
+  C.inv_unit = (float)(536870912.0 / g.cs);
+  C.fix_hi = C.inv_unit;
+  C.fix_lo = (float)(536870912.0 / g.cs - (double)C.fix_hi);
+  const double iu = 536870912.0 / g.cs;
+  C.walk_r2max = (float)(4.0 * p.h * p.h * iu * iu);
+  C.walk_eta2 = (float)(p.eta2 * iu * iu);
+  C.walk_hih = (float)(0.5 / p.h / iu);
   C.khyd[0] = (float)(kB * p.gravity.x);
   C.khyd[1] = (float)(kB * p.gravity.y);
   C.khyd[2] = (float)(kB * p.gravity.z);
@@ -183,7 +191,8 @@ struct sph_engine_t {
   bool ext = false;    // a case uses Eq 19-20 diffusion or laminar + SPS viscosity
   bool sps = false;    // a case uses laminar + SPS viscosity (tau buffers below)
   bool mdbc = false;   // a case uses the modified dynamic boundary condition
-  // neighbour list (pi_variant 3-5): list_cap chunk records per target
+  // neighbour list (pi_variant 3-5): a segment of list_cap chunk records (2
+  // list_cap candidate indices) per target
   bool list_ok = false;
   bool list_wide = false;  // wide records: beyond 2^25 particles (default physics only)
   bool list_wide_needed = false;  // (then always; else as sph_options.wide_records)
@@ -191,6 +200,8 @@ struct sph_engine_t {
   int64_t list_ld = 0;
   uint2 *nlist = nullptr;
   uint16_t *ncount = nullptr;
+  float4 *walk = nullptr;  // what the list walks gather: 32 bytes per particle of the
+                           // evaluated state (kReadPad entries past the last)
   float4 *posc_ref = nullptr;  // positions at the list's build (pi_variant 5)
   float4 *posc_ref2 = nullptr; //   the same gathered into a rebuild's new order
   bool list_dirty = true;      // the next kept-list step starts with a rebuild event
@@ -410,6 +421,7 @@ int allocate(sph_engine e) {
     e->posc_ref2 = (float4 *)A(16 * N);
     e->ctl = (ListCtl *)A(sizeof(ListCtl));
     e->rb_tmp = (uint32_t *)A(4 * rb_temp_words(N));
+    e->walk = (float4 *)A(32 * NP);
   }
   if (e->sps || e->pool) {
     e->tau4 = (float4 *)A(16 * N);
@@ -426,6 +438,7 @@ int allocate(sph_engine e) {
     CUDA_TRY(cudaMemsetAsync(e->S[b].velrho, 0, 16 * NP, e->s));
   }
   CUDA_TRY(cudaMemsetAsync(e->press, 0, 4 * NP, e->s));
+  if (e->walk) CUDA_TRY(cudaMemsetAsync(e->walk, 0, 32 * NP, e->s));
   CUDA_TRY(cudaMemsetAsync(e->ddyn, 0, sizeof(CaseDyn) * e->cap_cases, e->s));
   if (e->ctl) CUDA_TRY(cudaMemsetAsync(e->ctl, 0, sizeof(ListCtl), e->s));
   CUDA_TRY(cudaMemsetAsync(e->dconst, 0, sizeof(CaseConst) * e->cap_cases, e->s));
@@ -637,11 +650,12 @@ void enqueue_list_nl(sph_engine e) {
   cudaStream_t s = e->s;
   radix_sort(e->keysA, e->keysB, e->perm1, n, e->nbits, e->sort_tmp, s);
   launch_reorder(nl, e->perm1, e->keysB, X.posc, X.velrho, X.id, X.cid, X.code, X.vrprev,
-                 X.ghost, Y, e->press, e->dconst, e->ddyn, e->nbits, s);
+                 X.ghost, Y, e->press, e->dconst, e->ddyn, e->nbits, s, nullptr, nullptr,
+                 e->walk);
   launch_cells(nl, e->keysB, e->cstart, e->cells_hw, e->nbits, e->nvalid, e->cells_tmp, s);
   if (e->mdbc)  // boundary values of Eq 38-39 on state n
     launch_mdbc(e->margin, nl, e->nvalid, e->keysB, Y, e->press, e->cstart, e->nbits, e->dconst,
-                e->ddyn, 0, s);
+                e->ddyn, 0, s, false, e->walk);
 }
 
 // The first evaluation of a list step, on state n (Y, keysB): pi_variant 4
@@ -657,26 +671,22 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
   if (e->opt.pi_variant == 5) {
     if (e->mdbc)  // boundary values of Eq 38-39 on state n (the build's cells)
       launch_mdbc(e->margin, nl, e->nvalid, e->keysB, Y, e->press, e->cstart, e->nbits,
-                  e->dconst, e->ddyn, 0, s, true);
-    launch_interact_list(nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid, e->cstart,
-                         e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist,
-                         e->list_cap, e->ncount, e->ext, tau4, e->tau2, s, mu,
-                         e->opt.pi_block, e->opt.pi_lanes,
-                         sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
-                         e->list_wide ? e->keysB : nullptr);
+                  e->dconst, e->ddyn, 0, s, true, e->walk);
+    launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
+                         e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
+                         e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
+                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
   } else if (e->opt.pi_variant == 4) {  // list alone, then both evaluations over it
     if (ev) cudaEventRecord(ev[0], s);  // the first evaluation's time includes the list
     launch_list_begin(e->cap_cases, e->dconst, e->ddyn, e->ctl, 0.f, 1, e->cstart, e->cells_hw,
                       s);
     launch_build_list(e->margin, nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid,
                       e->cstart, e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, e->nlist,
-                      e->list_cap, e->ncount, nullptr, nullptr, s, sym_on(e), e->list_wide);
-    launch_interact_list(nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid, e->cstart,
-                         e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist,
-                         e->list_cap, e->ncount, e->ext, tau4, e->tau2, s, mu,
-                         e->opt.pi_block, e->opt.pi_lanes,
-                         sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
-                         e->list_wide ? e->keysB : nullptr);
+                      e->list_cap, e->ncount, nullptr, nullptr, s, sym_on(e));
+    launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
+                         e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
+                         e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
+                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
   } else {
     launch_list_begin(e->cap_cases, e->dconst, e->ddyn, e->ctl, 0.f, 1, e->cstart, e->cells_hw,
                       s);
@@ -689,8 +699,7 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
   if (ev) cudaEventRecord(ev[1], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysB, Y.posc, Y.cid, e->dconst, e->nbits, e->nlist,
-                      e->list_cap, e->ncount, e->ctl, s, sym_on(e),
-                      e->list_wide ? e->keysB : nullptr);
+                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk);
 }
 
 // The rest of a list step up to its second evaluation: dt (Eq 35), the half
@@ -703,22 +712,20 @@ void enqueue_list_half(sph_engine e, cudaEvent_t *ev, float *mu) {
   cudaStream_t s = e->s;
   launch_dt(e->cap_cases, e->dconst, e->ddyn, s);
   launch_predictor_list(nl, e->keysB, Y, e->ace, e->dconst, e->ddyn, e->nbits, Z.posc, Z.velrho,
-                        e->keysC, e->press, e->opt.pi_variant == 5 ? e->posc_ref : nullptr, s);
+                        e->keysC, e->press, e->opt.pi_variant == 5 ? e->posc_ref : nullptr, e->walk,
+                        s);
   if (e->mdbc)  // boundary values of Eq 38-39 on state n+1/2 (Y's cells)
     launch_mdbc(e->margin, nl, e->nvalid, e->keysC, half_state(Y, Z), e->press, e->cstart,
-                e->nbits, e->dconst, e->ddyn, 1, s, true);
+                e->nbits, e->dconst, e->ddyn, 1, s, true, e->walk);
   if (ev) cudaEventRecord(ev[2], s);
-  launch_interact_list(nl, e->nvalid, e->keysC, Z.posc, Z.velrho, e->press, Y.cid, e->cstart,
-                       e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, 0, e->nlist,
-                       e->list_cap, e->ncount, e->ext, e->sps ? e->tau4 : nullptr, e->tau2, s,
-                       mu, e->opt.pi_block, e->opt.pi_lanes,
-                         sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
-                         e->list_wide ? e->keysB : nullptr);
+  launch_interact_list(nl, e->nvalid, e->keysC, e->walk, Y.cid, e->cstart, e->cells_hw,
+                       e->nbits, e->dconst, e->ddyn, e->ace, 0, e->nlist, e->list_cap, e->ncount,
+                       e->ext, e->sps ? e->tau4 : nullptr, e->tau2, s, mu, e->opt.pi_block,
+                       e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
   if (ev) cudaEventRecord(ev[3], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysC, Z.posc, Y.cid, e->dconst, e->nbits, e->nlist,
-                      e->list_cap, e->ncount, e->ctl, s, sym_on(e),
-                      e->list_wide ? e->keysB : nullptr);
+                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk);
 }
 
 // One Symplectic step with the per-step neighbour list: NL on state n (Y),
@@ -753,11 +760,11 @@ void enqueue_rebuild_sort(sph_engine e, cudaStream_t q) {
     radix_sort(e->keysA, e->keysB, e->perm1, n, e->nbits, e->sort_tmp, q);
     launch_reorder(nl, e->perm1, e->keysB, X.posc, X.velrho, X.id, X.cid, X.code, X.vrprev,
                    X.ghost, Y, e->press, e->dconst, e->ddyn, e->nbits, q, e->posc_ref,
-                   e->posc_ref2);
+                   e->posc_ref2, e->walk);
   } else {
     launch_select(n, X.cid, e->dconst, e->ddyn, e->keysB, Y.posc, e->keysA, X.posc, e->ctl, q);
     launch_rebuild_sort(n, e->ctl, e->keysA, X, Y, e->keysB, e->press, e->dconst, e->ddyn,
-                        e->nbits, e->posc_ref, e->posc_ref2, e->rb_tmp, e->perm2, e->keysC,
+                        e->nbits, e->posc_ref, e->posc_ref2, e->walk, e->rb_tmp, e->perm2, e->keysC,
                         e->keysD, e->perm1, e->sort_tmp, q);
   }
   launch_cells(nl, e->keysB, e->cstart, e->cells_hw, e->nbits, e->nvalid, e->cells_tmp, q);
@@ -773,8 +780,7 @@ void enqueue_rebuild_list(sph_engine e, float extra, cudaStream_t q) {
                     q);
   launch_build_list(e->margin, nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid,
                     e->cstart, e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, e->nlist,
-                    e->list_cap, e->ncount, e->posc_ref, e->posc_ref2, q, sym_on(e),
-                    e->list_wide);
+                    e->list_cap, e->ncount, e->posc_ref, e->posc_ref2, q, sym_on(e));
 }
 
 // Appends to the graph being captured on e->s a k_decide kernel and an IF
@@ -889,7 +895,7 @@ void enqueue_step_reuse(sph_engine e, cudaEvent_t *ev) {
   enqueue_list_first(e, ev, nullptr);
   enqueue_list_half(e, ev, nullptr);
   launch_corrector_reuse(nl, e->keysB, e->keysC, Y, Z.velrho, e->ace, e->posc_ref, e->dconst,
-                         e->ddyn, e->nbits, X, e->keysA, e->press, e->ctl, e->s);
+                         e->ddyn, e->nbits, X, e->keysA, e->press, e->ctl, e->walk, e->s);
   launch_end_step(e->cap_cases, e->dconst, e->ddyn, e->s);
 }
 
@@ -905,7 +911,7 @@ void enqueue_step_verlet_reuse(sph_engine e, cudaEvent_t *ev) {
   enqueue_list_first(e, ev, nullptr);
   launch_dt(e->cap_cases, e->dconst, e->ddyn, e->s);
   launch_verlet_reuse(nl, e->keysB, Y, e->ace, e->dconst, e->ddyn, e->nbits, X, e->keysA,
-                      e->posc_ref, e->press, e->ctl, e->s);
+                      e->posc_ref, e->press, e->ctl, e->walk, e->s);
   launch_end_step(e->cap_cases, e->dconst, e->ddyn, e->s);
 }
 
@@ -1606,6 +1612,9 @@ int sph_eval_step(sph_engine e, int32_t icase, int32_t stage, double *pos, float
   // restore
   if (nl > 0)
     CUDA_TRY(cudaMemcpyAsync(e->press, press_saved, 4 * (size_t)nl, cudaMemcpyDeviceToDevice, s));
+  if (reuse && stage == 1)  // the walk records of state n again
+    launch_pack_walk(nl, e->keysB, Y.posc, Y.velrho, e->press, Y.cid, e->dconst, e->nbits, e->walk,
+                     s);
   CUDA_TRY(cudaMemcpyAsync(e->ddyn, saved.data(), sizeof(CaseDyn) * e->cap_cases,
                            cudaMemcpyHostToDevice, s));
   if (e->ctl)

@@ -55,6 +55,11 @@ struct CaseConst {
   float sps_cs2;  // (C_S Delta)^2 of Eq 25
   float sps_cl2;  // C_l Delta^2 of Eq 25
   float wk;       // a_D of Eq 11: W = a_D t^4 (5 - 4t), t = 1 - r/(2h)
+  // the list walks' positions: integers in units of unit = cs / 2^29 (1 / unit =
+  // inv_unit = fix_hi + fix_lo in two FP32 parts), and 2h squared, eta^2 and
+  // 1/2h in that unit
+  float unit, inv_unit, fix_hi, fix_lo;
+  float walk_r2max, walk_eta2, walk_hih;
   float list_k;   // 1.25 x the Eq 35 bound on dt (or the fixed dt): skin = list_k |v|max + 1e-3 h
 };
 
@@ -84,19 +89,12 @@ constexpr unsigned kFlagNaN = 1u, kFlagDtMin = 2u, kFlagQuota = 4u;
 // holds; a displacement since the list's build exceeded half its skin (or
 // one step's need exceeded the largest skin the rows cover)
 constexpr unsigned kFlagListFull = 8u, kFlagSkin = 16u;
-// list record: first candidate index (25 bits) | row code << 25, with the
-// row code (dz + 4) * 9 + (dy + 4) for row offsets dy, dz in [-4, 4]
+// A target's list: its candidates' indices (32 bits each; count = their
+// number), or, where they do not fit its segment, chunk records (first
+// candidate index, 32-bit mask) with count = kListRecords | their number.
+constexpr unsigned kListRecords = 0x8000u;
+// engines beyond this size keep lists for the default physics only
 constexpr int kListMaxParticles = 1 << 25;
-constexpr uint32_t kListIndexMask = (1u << 25) - 1u;
-__host__ __device__ inline uint32_t list_row_code(int dy, int dz) {
-  return (uint32_t)((dz + 4) * 9 + (dy + 4)) << 25;
-}
-__host__ __device__ inline void list_row_decode(uint32_t x, int &dy, int &dz) {
-  const int r = (int)(x >> 25);
-  const int q = r / 9;
-  dz = q - 4;
-  dy = r - 9 * q - 4;
-}
 
 // Engine-wide control of the neighbour list kept across steps: rebuild is
 // requested by the corrector (a case needs a new list) or by the host (cases

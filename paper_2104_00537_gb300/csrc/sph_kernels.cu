@@ -68,6 +68,28 @@ __device__ __forceinline__ int shift_axis(float off, double disp, const CaseCons
   return (int)k;
 }
 
+// Position of the list walks along one axis: the cell index modulo 8 and the
+// offset in units of cs / 2^29, as one wrapping 32-bit integer.  The offset's
+// product with 2^29 / cs is formed in two FP32 parts, so the integer is within
+// one unit (2^-29 cs) of it: the FP32 offset itself is rounded to 2^-25 cs.
+__device__ __forceinline__ int walk_coord(const CaseConst &C, int c, float off) {
+  const float p = off * C.fix_hi;
+  const float e = fmaf(off, C.fix_lo, fmaf(off, C.fix_hi, -p));
+  return (int)(((uint32_t)c << 29) + (uint32_t)__float2int_rn(p) + (uint32_t)__float2int_rn(e));
+}
+
+// The record the list walks gather for particle i (32 bytes, one sector):
+// {position as three walk_coord integers, P/rho}, {v, rho}.
+__device__ __forceinline__ void put_walk(float4 *walk, int i, const CaseConst &C, uint32_t key,
+                                         int nbits, const float4 &p, const float4 &v, float Q) {
+  int cx, cy, cz;
+  decode_cell(key_cell(key, nbits) - C.cellbase, C.nx, C.ny, cx, cy, cz);
+  walk[2 * (int64_t)i] = make_float4(__int_as_float(walk_coord(C, cx, p.x)),
+                                     __int_as_float(walk_coord(C, cy, p.y)),
+                                     __int_as_float(walk_coord(C, cz, p.z)), Q);
+  walk[2 * (int64_t)i + 1] = v;
+}
+
 // ---- upload ------------------------------------------------------------------
 
 __global__ void k_upload(int n, const double *__restrict__ pos, const float *__restrict__ vel,
@@ -138,7 +160,8 @@ __global__ void k_reorder(int n, const uint32_t *__restrict__ perm,
                           float *__restrict__ press, const CaseConst *__restrict__ cc,
                           CaseDyn *__restrict__ dyn, int nbits,
                           const float4 *__restrict__ ref_src = nullptr,
-                          float4 *__restrict__ ref_dst = nullptr) {
+                          float4 *__restrict__ ref_dst = nullptr,
+                          float4 *__restrict__ walk = nullptr) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   int cidx = -1;
   unsigned v2 = 0u;
@@ -162,7 +185,9 @@ __global__ void k_reorder(int n, const uint32_t *__restrict__ perm,
     if (vrprev_src) dst.vrprev[i] = vrprev_src[p];
     if (ghost_src) dst.ghost[i] = ghost_src[p];
     if (ref_dst) ref_dst[i] = ref_src[p];  // kept list: build positions follow the order
-    press[i] = tait_pressure(C, vr.w) / vr.w;
+    const float Q = tait_pressure(C, vr.w) / vr.w;
+    press[i] = Q;
+    if (walk && k < key_out(nbits)) put_walk(walk, i, C, k, nbits, pc, vr, Q);
   }
   // max |v|^2 per case (for the neighbour list's skin): one atomic per warp
   // when the warp holds one case
@@ -276,7 +301,7 @@ __global__ void k_rb_scatter(int n, const int *__restrict__ m_p, const uint32_t 
                              uint32_t *__restrict__ keys_dst, float *__restrict__ press,
                              const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
                              int nbits, const float4 *__restrict__ ref_src,
-                             float4 *__restrict__ ref_dst) {
+                             float4 *__restrict__ ref_dst, float4 *__restrict__ walk) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   int cidx = -1;
   unsigned v2 = 0u;
@@ -301,7 +326,9 @@ __global__ void k_rb_scatter(int n, const int *__restrict__ m_p, const uint32_t 
     if (src.vrprev) dst.vrprev[d] = src.vrprev[q];
     if (src.ghost) dst.ghost[d] = src.ghost[q];
     if (ref_dst) ref_dst[d] = ref_src[q];
-    press[d] = tait_pressure(C, vr.w) / vr.w;
+    const float Q = tait_pressure(C, vr.w) / vr.w;
+    press[d] = Q;
+    if (walk && k < key_out(nbits)) put_walk(walk, (int)d, C, k, nbits, pc, vr, Q);
   }
   // max |v|^2 per case (for the skin of the cases that rebuild), as k_reorder
   const unsigned full = 0xffffffffu;
@@ -468,8 +495,10 @@ struct Acc {
 // kernel support |x| is small (|x| <= 2h gamma |g| / cs0^2, about 1e-3 for
 // the usual cs0), where the binomial series to x^4 is used: its first
 // omitted term is below 2e-9 relative for |x| < 1e-2; otherwise log1p/expm1.
-__device__ __forceinline__ float rho_hydro(const CaseConst &C, float rx, float ry, float rz) {
-  const float x = fmaf(C.khyd[0], rx, fmaf(C.khyd[1], ry, C.khyd[2] * rz));  // P^H / B
+// unit: the length unit of r (1 on the cell walks, CaseConst::unit on the list walks).
+__device__ __forceinline__ float rho_hydro(const CaseConst &C, float unit, float rx, float ry,
+                                           float rz) {
+  const float x = unit * fmaf(C.khyd[0], rx, fmaf(C.khyd[1], ry, C.khyd[2] * rz));  // P^H / B
   if (fabsf(x) < 1e-2f) {
     const float s = fmaf(C.hyd_c[0] * x, fmaf(C.hyd_c[1] * x, fmaf(C.hyd_c[2], x, 1.f), 1.f), 1.f);
     return C.rho0 * C.inv_gamma * x * s;
@@ -482,6 +511,7 @@ __device__ __forceinline__ float rho_hydro(const CaseConst &C, float rx, float r
 struct Ext {
   const CaseConst *C;
   bool hyd, sps;
+  float unit;    // length unit of r_ab (m)
   float kl;      // -4 nu0 rho_a (Eq 23, in the units of the momentum sums)
   float ta[6];   // rho_a (tau/rho)_a: xx, yy, zz, xy, xz, yz (Eq 25)
   const float4 *__restrict__ tau4;  // (tau/rho)_b: xx, yy, zz, xy
@@ -510,7 +540,7 @@ __device__ __forceinline__ void pair_fluid(const float4 &va, float Pa, float kv,
   A.s1 = fmaf(w, vr, A.s1);
   if (ddt) {
     float d = vb.w - va.w;
-    if (EXT >= 1 && X->hyd) d -= rho_hydro(*X->C, rx, ry, rz);
+    if (EXT >= 1 && X->hyd) d -= rho_hydro(*X->C, X->unit, rx, ry, rz);
     A.s2 = fmaf(w, d, A.s2);
   }
   const float sab = va.w + vb.w;
@@ -553,47 +583,49 @@ __device__ __forceinline__ void pair_boundary(const float4 &va, float hih, float
   A.s1 = fmaf(t3 * __fdividef(1.f, vb.w), vr, A.s1);
 }
 
-// Final values of target a from its accumulators: dv/dt (Eq 22 with g), drho/dt
-// (Eq 15 with the Eq 17-18 term, or Eq 36), mu_max and the Eq 35 candidate
-// time step; then the warp's per-case reduction of counts, dt and flags.
-// With several lanes per target (all holding the same totals) only the lead
-// lane writes and counts.
+// Final values of target a (of density rho_a) from its accumulators: dv/dt
+// (Eq 22 with g), drho/dt (Eq 15 with the Eq 17-18 term, or Eq 36), mu_max and
+// the Eq 35 candidate time step (dtbits) and the non-finite flag.
+__device__ __forceinline__ void finish_values(const CaseConst &C, int i, bool afluid, float rho_a,
+                                              const Acc &A, int want_dt,
+                                              float4 *__restrict__ ace,
+                                              float *__restrict__ mu_out, unsigned &dtbits,
+                                              bool &bad) {
+  const float mcw = C.m * C.cw;
+  float4 out;
+  float mumax = C.h * A.mur;
+  if (afluid) {
+    const float ca = -mcw / rho_a;
+    out.x = fmaf(ca, A.ax, C.g[0]);
+    out.y = fmaf(ca, A.ay, C.g[1]);
+    out.z = fmaf(ca, A.az, C.g[2]);
+    out.w = mcw * (rho_a * A.s1 - C.kddt * A.s2);
+    const float f = sqrtf(out.x * out.x + out.y * out.y + out.z * out.z);
+    const float dtf = f > 0.f ? sqrtf(C.h / f) : INFINITY;
+    const float dtcv = C.h / (C.cs0f + mumax);
+    bad = !(isfinite(out.x) && isfinite(out.y) && isfinite(out.z) && isfinite(out.w));
+    if (want_dt) dtbits = __float_as_uint(fminf(dtf, dtcv));
+  } else {
+    out = make_float4(0.f, 0.f, 0.f, mcw * rho_a * A.s1);
+    mumax = 0.f;
+    bad = !isfinite(out.w);
+  }
+  ace[i] = out;
+  if (mu_out) mu_out[i] = mumax;
+}
+
+// finish_values, then the warp's per-case reduction of counts, dt and flags.
 __device__ __forceinline__ void finish_target(const CaseConst &C, int i, int n, int cidx, bool has,
                                               bool afluid, const float4 &va, const Acc &A,
                                               int want_dt, float4 *__restrict__ ace,
-                                              float *__restrict__ mu_out, CaseDyn *dyn,
-                                              bool lead = true) {
+                                              float *__restrict__ mu_out, CaseDyn *dyn) {
   unsigned npairs = 0, nfb = 0, nbf = 0, dtbits = kFloatInfBits;
   bool bad = false;
   if (has) {
     npairs = A.cnt + A.cntb;
     nfb = afluid ? A.cntb : 0u;
     nbf = afluid ? 0u : A.cnt;
-    const float mcw = C.m * C.cw;
-    float4 out;
-    float mumax = C.h * A.mur;
-    if (afluid) {
-      const float ca = -mcw / va.w;
-      out.x = fmaf(ca, A.ax, C.g[0]);
-      out.y = fmaf(ca, A.ay, C.g[1]);
-      out.z = fmaf(ca, A.az, C.g[2]);
-      out.w = mcw * (va.w * A.s1 - C.kddt * A.s2);
-      const float f = sqrtf(out.x * out.x + out.y * out.y + out.z * out.z);
-      const float dtf = f > 0.f ? sqrtf(C.h / f) : INFINITY;
-      const float dtcv = C.h / (C.cs0f + mumax);
-      bad = !(isfinite(out.x) && isfinite(out.y) && isfinite(out.z) && isfinite(out.w));
-      if (want_dt) dtbits = __float_as_uint(fminf(dtf, dtcv));
-    } else {
-      out = make_float4(0.f, 0.f, 0.f, mcw * va.w * A.s1);
-      mumax = 0.f;
-      bad = !isfinite(out.w);
-    }
-    if (lead) {
-      ace[i] = out;
-      if (mu_out) mu_out[i] = mumax;
-    } else {
-      npairs = nfb = nbf = 0u;
-    }
+    finish_values(C, i, afluid, va.w, A, want_dt, ace, mu_out, dtbits, bad);
   }
   reduce_case(i < n ? cidx : -1, has, npairs, nfb, nbf, dtbits, bad, dyn);
 }
@@ -662,6 +694,67 @@ __global__ void k_need_all(int ncases, CaseDyn *__restrict__ dyn) {
   if (c < ncases) dyn[c].need = 1u;
 }
 
+// Turns the records (first index, mask) that each lane of the warp wrote for
+// its target into the target's flat list: the candidate indices in record
+// order, 32 bits each, in the same segment (2 cap of them).  The warp takes
+// its 32 targets one by one: the records go to registers, then each record's
+// candidates are written side by side by the lanes whose bit is set.  A target
+// whose candidates do not fit, or with more than 128 records, keeps its records
+// (kListRecords in its count).  Cost: about 11 warp-instructions per record,
+// paid once per build, against a list walk without masks, rows or bit scans.
+constexpr int kFlatRounds = 4;  // of 32 records
+__device__ __forceinline__ void flatten_records(int i, bool build, int nrec,
+                                                uint2 *__restrict__ list, int cap,
+                                                uint16_t *__restrict__ count) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  unsigned todo = __ballot_sync(full, build);
+  int mine = 0;
+  __syncwarp();  // the lanes' records are visible to the warp
+  while (todo) {
+    const int t = __ffs(todo) - 1;
+    todo &= todo - 1u;
+    const int nr = __shfl_sync(full, nrec, t);
+    uint2 *rec = list + (int64_t)(i - lane + t) * cap;
+    uint2 r[kFlatRounds];
+    int off[kFlatRounds], total = 0;
+#pragma unroll
+    for (int h = 0; h < kFlatRounds; h++) {
+      r[h] = make_uint2(0u, 0u);
+      off[h] = total;
+      if (nr <= 32 * h) continue;
+      if (32 * h + lane < nr) r[h] = rec[32 * h + lane];
+      const int c = __popc(r[h].y);
+      int x = c;  // inclusive scan of the records' candidate counts
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(full, x, o);
+        if (lane >= o) x += y;
+      }
+      off[h] = total + x - c;
+      total += __shfl_sync(full, x, 31);
+    }
+    const bool flat = nr <= 32 * kFlatRounds && total <= 2 * cap;
+    if (lane == t) mine = flat ? total : (int)kListRecords | nr;
+    if (!flat) continue;
+    __syncwarp();  // every record is in registers before its memory is overwritten
+    uint32_t *dst = reinterpret_cast<uint32_t *>(rec);
+#pragma unroll
+    for (int h = 0; h < kFlatRounds; h++) {
+      const int m = min(32, nr - 32 * h);
+#pragma unroll 4
+      for (int q = 0; q < m; q++) {
+        const uint32_t b = __shfl_sync(full, r[h].x, q);
+        const unsigned mask = __shfl_sync(full, r[h].y, q);
+        const int o = __shfl_sync(full, off[h], q);
+        if ((mask >> lane) & 1u) dst[o + __popc(mask & lt)] = b + (uint32_t)lane;
+      }
+    }
+  }
+  if (build) count[i] = (uint16_t)mine;
+}
+
 // One thread per particle a in sorted order (all fluid targets first, then
 // boundary targets, so warps rarely mix the two).  The (2M+1)^2 rows of
 // neighbour cells (fixed dy, dz) are visited in lock-step by the warp; in a
@@ -681,19 +774,16 @@ __global__ void k_need_all(int ncases, CaseDyn *__restrict__ dyn) {
 // LIST (VARIANT 0): 1 also writes the target's neighbour list, 2 writes
 // only the list (no pair terms, no outputs besides the list and ref): for
 // every tested chunk with a candidate within 2h + skin, one record (first
-// index | row offset, mask of those candidates) to list[i cap + c] (a target's
-// records side by side, four to a 32-byte sector), at most cap per target.  The
+// index, mask of those candidates) to list[i cap + c], at most cap per target;
+// flatten_records then turns a target's records into candidate indices.  The
 // list's rows reach one cell further than the 2h support (M + 1 cells, so
 // 2h + cs >= 2h + skin), clipped to the case's grid.  ref, if set, receives
 // the target's position at the build (the list kept across steps), and the
-// case's build mode applies (k_list_begin): 0 keeps the target's records, 1
+// case's build mode applies (k_list_begin): 0 keeps the target's list, 1
 // builds from posc, 2 rebuilds from the previous build positions (ref_src,
 // gathered into the new order) with the case's old skin.  3 is 2 with only
 // the candidates of larger index than the target (the half list of the
 // pair-once walk: a boundary target, after every fluid index, gets none).
-// LIST | 4 (6, 7): wide records, the whole 32-bit first index with no row
-// code (engines beyond 2^25 particles; the walks find the row from the
-// first candidate's cell).
 template <int M, int VARIANT, int EXT = 0, int LIST = 0>
 __global__ void __launch_bounds__(128, EXT == 2 ? 6 : 0)
 k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ keys,
@@ -739,10 +829,11 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
   // boundary targets of an mDBC case take their density from Eq 38, not Eq 36;
   // a half list (every boundary index above every fluid one) leaves boundary
   // targets without candidates
-  constexpr bool HALF = (LIST & 3) == 3;
+  constexpr bool HALF = LIST == 3;
   const bool work = has && (afluid || C.bmode == 0) && lmode != 0 && (!HALF || afluid);
   Ext X;
   X.C = &C;
+  X.unit = 1.f;
   X.hyd = EXT >= 1 && C.ddt == 2;
   X.sps = EXT == 2 && C.visc == 1 && afluid;
   X.kl = -4.f * C.nu0 * va.w;
@@ -811,7 +902,6 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
       }
     }
     const float sy = fmaf(-(float)dy, cs, pa.y), sz = fmaf(-(float)dz, cs, pa.z);
-    const uint32_t rowbits = list_row_code(dy, dz);
 #pragma unroll 1
     for (int part = 0; part < 2; part++) {  // fluid neighbours, then boundary neighbours
       const int lo = part ? loB : loF;
@@ -834,14 +924,14 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
               if (LIST && __float_as_uint(r2) - 1u < r2l_u) ml |= 1u << k;
             }
           }
-          if ((LIST & 3) == 3) {  // half list: only candidates of larger index than the target
+          if (HALF) {  // half list: only candidates of larger index than the target
             const int lowk = i - (lo + base) + 1;
             if (lowk > 0) ml = lowk >= 32 ? 0u : ml & (0xffffffffu << lowk);
           }
           if (LIST && ml) {
             if (lcnt < cap)
               list[(int64_t)i * cap + lcnt] =
-                  make_uint2((uint32_t)(lo + base) | (LIST & 4 ? 0u : rowbits), ml);
+                  make_uint2((uint32_t)(lo + base), ml);
             lcnt++;
           }
           if (LIST < 2) {
@@ -907,9 +997,9 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
     }
   }
 
-  if (LIST && i < n && lmode != 0) {
-    count[i] = (uint16_t)min(lcnt, cap);
+  if (LIST) {
     if (has && lcnt > cap) atomicOr(&dyn[cidx].flags, kFlagListFull);
+    flatten_records(i, i < n && lmode != 0, min(lcnt, cap), list, cap, count);
   }
   if (LIST >= 2) return;
   finish_target(C, i, n, cidx, has, afluid, va, A, want_dt, ace, mu_out, dyn);
@@ -1363,7 +1453,8 @@ template <int M, bool LIST>
 __global__ void __launch_bounds__(128)
 k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ keys, State st,
        float *__restrict__ press, const uint32_t *__restrict__ cstart, int nbits,
-       const CaseConst *__restrict__ cc, const CaseDyn *__restrict__ dyn, int stage) {
+       const CaseConst *__restrict__ cc, const CaseDyn *__restrict__ dyn, int stage,
+       float4 *__restrict__ walk) {
   const unsigned full = 0xffffffffu;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int nvalid = *nvalid_p;
@@ -1523,8 +1614,13 @@ k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ key
       out.z = fmaf(k2, nz_, vgz);
     }
   }
+  const float Q = tait_pressure(C, out.w) / out.w;
   st.velrho[i] = out;
-  press[i] = tait_pressure(C, out.w) / out.w;
+  press[i] = Q;
+  if (walk) {  // the record of the list walks
+    walk[2 * (int64_t)i].w = Q;
+    walk[2 * (int64_t)i + 1] = out;
+  }
 }
 
 // ---- time step and motion ----------------------------------------------------
@@ -1769,18 +1865,12 @@ __global__ void k_corrector(int n, const uint32_t *__restrict__ perm2,
 // differs.
 
 
-// The interaction over a target's list (state n or n+1/2, same order and
-// cells): the pair terms of k_interact for the entries inside 2h.  EXT 1
-// adds the Eq 19-20 density diffusion, EXT 2 also laminar + SPS (tau4/tau2
-// from k_strain_list), for the cases that use them.
-// Arguments of the interaction over the neighbour list (one struct, so that
-// the one-target body below serves both launch forms).
+// Arguments of the interaction over the neighbour list.
 struct ListArgs {
   int n;
   const int *nvalid_p;
   const uint32_t *keys;
-  const float4 *posc, *velrho;
-  const float *press;
+  const float4 *walk;  // put_walk records of the evaluated state
   const uint16_t *cid;
   const uint32_t *cstart;
   uint32_t cap1;
@@ -1790,328 +1880,378 @@ struct ListArgs {
   float4 *ace;
   int want_dt;
   const uint2 *list;
-  int cap;  // records per target: record r of target i at list[i cap + r]
+  int cap;  // a target's segment: cap records, or 2 cap candidate indices
   const uint16_t *count;
   const float4 *tau4;
   const float2 *tau2;
   float *mu_out;
-  // wide records (beyond 2^25 particles): the keys of the build's cells,
-  // whose cell gives a record's row (valid for every candidate of a kept
-  // list, also where a particle left at the half step)
-  const uint32_t *row_keys;
+  int per;  // targets that a group of G lanes takes one after another (<= G)
 };
 
-// One target i of the list walk (all 32 lanes of the warp call it together).
-// G lanes share a target (G = 1, 2, 4 or 8; sub = the lane's rank among
-// them): lane sub takes the candidates of each record at the bit positions
-// sub, sub + G, sub + 2G, ..., so the lanes of a target load neighbouring
-// candidates together (fewer L1 wavefronts per gather), and the G partial
-// sums are combined by a butterfly over the G lanes at the end.
-template <int EXT, int G, int W = 0>
-__device__ __forceinline__ void list_target(const int i, const int sub, const ListArgs &a) {
+// Relative position of two walk records, in units of cs / 2^29: the integer
+// differences wrap (period 8 cs), so cells and rows need no bookkeeping.
+// Listed particles lie within 2h + 2 skin < 5 cs of each other on every axis;
+// what aliases (beyond 4 cs) stays beyond 3 cs >= 2h, so it is no pair.
+__device__ __forceinline__ float walk_r2(const float4 &a, const float4 &b, float &rx, float &ry,
+                                         float &rz) {
+  rx = (float)(__float_as_int(a.x) - __float_as_int(b.x));
+  ry = (float)(__float_as_int(a.y) - __float_as_int(b.y));
+  rz = (float)(__float_as_int(a.z) - __float_as_int(b.z));
+  return fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+}
+
+// One 32-byte walk record in one 256-bit load.
+__device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j, float4 &p,
+                                          float4 &b) {
+  asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(p.x), "=f"(p.y), "=f"(p.z), "=f"(p.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+      : "l"(walk + 2 * (int64_t)j));
+}
+
+// The candidates of target i (all 32 lanes of the warp call it together, G
+// lanes with the same i; sub: the lane's rank among them).  Lane sub takes the
+// list entries sub, sub + G, ..., so the lanes of a target read neighbouring
+// entries and, the list being in cell order, mostly neighbouring candidates;
+// two candidates per iteration with their loads issued together, the next two
+// indices loaded ahead.  body(rx, ry, rz, r2, b, j) runs for every candidate
+// inside the support; positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
+// A lane without an entry takes the target itself (r2 = 0: no pair).
+template <int G, class Body>
+__device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const int sub,
+                                          const unsigned cw, const float4 &pa,
+                                          const unsigned r2max_u, Body body) {
   const unsigned full = 0xffffffffu;
-  const int n = a.n;
-  const int *__restrict__ nvalid_p = a.nvalid_p;
-  const uint32_t *__restrict__ keys = a.keys;
-  const float4 *__restrict__ posc = a.posc;
-  const float4 *__restrict__ velrho = a.velrho;
-  const float *__restrict__ press = a.press;
-  const uint16_t *__restrict__ cid = a.cid;
-  const uint32_t *__restrict__ cstart = a.cstart;
-  const uint32_t cap1 = a.cap1;
-  const int nbits = a.nbits;
-  const CaseConst *__restrict__ cc = a.cc;
-  CaseDyn *__restrict__ dyn = a.dyn;
-  float4 *__restrict__ ace = a.ace;
-  const int want_dt = a.want_dt;
-  const uint2 *__restrict__ list = a.list;
-  const int cap = a.cap;
-  const uint16_t *__restrict__ count = a.count;
-  const float4 *__restrict__ tau4 = a.tau4;
-  const float2 *__restrict__ tau2 = a.tau2;
-  float *__restrict__ mu_out = a.mu_out;
-  const int nvalid = *nvalid_p;
-  const uint32_t key = i < nvalid ? keys[i] : key_out(nbits);
-  const bool has = key < key_out(nbits);  // not frozen at this state
-  const int cidx = i < n ? (int)cid[i] : 0;
-  const CaseConst &C = cc[cidx];
-  const bool afluid = has && !key_boundary(key, nbits);
-  const float cs = C.csf, eta2 = C.eta2, hih = C.half_inv_h;
-  const unsigned r2max_u = __float_as_uint(C.r2max) - 1u;
-  const float4 pa = has ? posc[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 va = has ? velrho[i] : make_float4(0.f, 0.f, 0.f, 1.f);
-  const float Pa = has ? press[i] * va.w : 0.f;
-  const float kv = C.kvisc * va.w;
-  const bool ddt_on = C.ddt != 0;
-  Ext X;
-  X.C = &C;
-  X.hyd = EXT >= 1 && C.ddt == 2;
-  X.sps = EXT == 2 && C.visc == 1 && afluid;
-  X.kl = -4.f * C.nu0 * va.w;
-  X.tau4 = tau4;
-  X.tau2 = tau2;
-  {
-    const float4 t4 = X.sps ? tau4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float2 t2 = X.sps ? tau2[i] : make_float2(0.f, 0.f);
-    X.ta[0] = va.w * t4.x;
-    X.ta[1] = va.w * t4.y;
-    X.ta[2] = va.w * t4.z;
-    X.ta[3] = va.w * t4.w;
-    X.ta[4] = va.w * t2.x;
-    X.ta[5] = va.w * t2.y;
-  }
-  const int jb = (int)cstart[cap1 - 1];  // first boundary particle of the key order
-  const int nrec = has ? (int)count[i] : 0;
-  const bool warp_fluid = __all_sync(full, afluid || !has);
-  Acc A = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};
-  const uint2 *__restrict__ mine = list + (int64_t)i * cap;
-  // two candidates per lane per iteration (their loads issued together),
-  // records taken in order: the warp waits only for its lane with the most
-  // candidates in total
-  int r = 0;
-  unsigned cm = 0u;
-  int cbase = 0;
-  float sy = 0.f, sz = 0.f;
-  // the next record of the lane: base index, candidate mask, row offsets
-  // the lane's bit positions within a record
-  const unsigned sel = (G == 1 ? 0xffffffffu : G == 2 ? 0x55555555u : G == 4 ? 0x11111111u
-                                                                    : 0x01010101u) << sub;
-  // wide records: the rows relative to the target's own cell
-  int tcy = 0, tcz = 0;
-  if (W && nrec) {
-    int tcx;
-    decode_cell(key_cell(a.row_keys[i], nbits) - C.cellbase, C.nx, C.ny, tcx, tcy, tcz);
-  }
-  auto next_record = [&]() {
-    const uint2 rec = mine[r++];
-    int rdy, rdz;
-    if (W) {
-      cbase = (int)rec.x;
-      int bx, by, bz;
-      decode_cell(key_cell(a.row_keys[cbase], nbits) - C.cellbase, C.nx, C.ny, bx, by, bz);
-      rdy = by - tcy;
-      rdz = bz - tcz;
-    } else {
-      cbase = (int)(rec.x & kListIndexMask);
-      list_row_decode(rec.x, rdy, rdz);
-    }
-    cm = rec.y & sel;
-    sy = fmaf(-(float)rdy, cs, pa.y);
-    sz = fmaf(-(float)rdz, cs, pa.z);
-  };
+  const float4 *__restrict__ walk = a.walk;
+  const bool rec = (cw & kListRecords) != 0u;
+  const int cnt = rec ? 0 : (int)cw;
+  const int kmax = (int)__reduce_max_sync(full, (unsigned)cnt);
+  const uint32_t *__restrict__ mine =
+      reinterpret_cast<const uint32_t *>(a.list + (int64_t)i * a.cap);
+  int j1 = sub < cnt ? (int)mine[sub] : i;
+  int j2 = sub + G < cnt ? (int)mine[sub + G] : i;
 #pragma unroll 1
-  for (;;) {
-    // (a record holds at least one candidate, but with G > 1 maybe none of
-    // this lane's)
-    if (G == 1) {
-      if (cm == 0u && r < nrec) next_record();
-    } else {
-      while (cm == 0u && r < nrec) next_record();
-    }
-    if (!__any_sync(full, cm != 0u)) break;
-    if (cm) {
-      // the lane's next two candidates in list order; the second may open the
-      // next record, so no slot idles at the end of an odd record
-      const int k1 = 31 - __clz(cm);
-      cm ^= 1u << k1;
-      const int j1 = cbase + k1;
-      const float sy1 = sy, sz1 = sz;
-      if (G == 1) {
-        if (cm == 0u && r < nrec) next_record();
-      } else {
-        while (cm == 0u && r < nrec) next_record();
-      }
-      const bool h2 = cm != 0u;
-      const int k2 = h2 ? 31 - __clz(cm) : k1;
-      if (h2) cm ^= 1u << k2;
-      const int j2 = h2 ? cbase + k2 : j1;
-      const float4 pb1 = posc[j1];
-      const float4 pb2 = posc[j2];
-      const float4 vb1 = velrho[j1];
-      const float4 vb2 = velrho[j2];
-      const float q1 = press[j1], q2 = press[j2];
+  for (int k = sub; k - sub < kmax; k += 2 * G) {
+    float4 p1, b1, p2, b2;
+    load_walk(walk, j1, p1, b1);
+    load_walk(walk, j2, p2, b2);
+    const int i1 = j1, i2 = j2;
+    j1 = k + 2 * G < cnt ? (int)mine[k + 2 * G] : i;
+    j2 = k + 3 * G < cnt ? (int)mine[k + 3 * G] : i;
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const float4 pb = u ? pb2 : pb1;
-        const float4 vb = u ? vb2 : vb1;
-        const int j = u ? j2 : j1;
-        const float rx = fmaf(pa.w - pb.w, cs, pa.x - pb.x);
-        const float ry = (u ? sy : sy1) - pb.y, rz = (u ? sz : sz1) - pb.z;
-        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        if ((u == 0 || h2) && __float_as_uint(r2) - 1u < r2max_u) {
-          const bool bfluid = j < jb;
-          if (warp_fluid || afluid) {
-            pair_fluid<EXT>(va, Pa, kv, hih, eta2, rx, ry, rz, r2, vb, u ? q2 : q1,
-                            ddt_on && bfluid, A, &X, j, bfluid);
-            if (bfluid) A.cnt++; else A.cntb++;
-          } else {
-            pair_boundary(va, hih, rx, ry, rz, r2, vb, A);
-            A.cnt++;
-          }
-        }
-      }
+    for (int u = 0; u < 2; u++) {
+      float rx, ry, rz;
+      const float r2 = walk_r2(pa, u ? p2 : p1, rx, ry, rz);
+      const float4 &b = u ? b2 : b1;
+      // (a particle that left at the half step has no density)
+      if (__float_as_uint(r2) - 1u < r2max_u && b.w > 0.f)
+        body(rx, ry, rz, r2, b, u ? p2.w : p1.w, u ? i2 : i1);
     }
   }
-  if (G > 1) {
-    // the G lanes' partial sums; every lane of the target ends with the same
-    // totals (each addition is commutative: lanes pair the same operands)
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1) {
-      A.ax += __shfl_xor_sync(full, A.ax, o);
-      A.ay += __shfl_xor_sync(full, A.ay, o);
-      A.az += __shfl_xor_sync(full, A.az, o);
-      A.s1 += __shfl_xor_sync(full, A.s1, o);
-      A.s2 += __shfl_xor_sync(full, A.s2, o);
-      A.mur = fmaxf(A.mur, __shfl_xor_sync(full, A.mur, o));
-      A.cnt += __shfl_xor_sync(full, A.cnt, o);
-      A.cntb += __shfl_xor_sync(full, A.cntb, o);
+  // a target that kept its records (too many candidates for its segment):
+  // lane sub takes the bits sub, sub + G, ... of every record
+  if (__any_sync(full, rec)) {
+    const int nr = rec ? (int)(cw & ~kListRecords) : 0;
+    const uint2 *__restrict__ seg = a.list + (int64_t)i * a.cap;
+    for (int r = 0; r < nr; r++) {
+      const uint2 q = seg[r];
+      for (int k = sub; k < 32; k += G) {
+        if (!((q.y >> k) & 1u)) continue;
+        const int j = (int)q.x + k;
+        const float4 p = walk[2 * (int64_t)j], b = walk[2 * (int64_t)j + 1];
+        float rx, ry, rz;
+        const float r2 = walk_r2(pa, p, rx, ry, rz);
+        if (__float_as_uint(r2) - 1u < r2max_u && b.w > 0.f) body(rx, ry, rz, r2, b, p.w, j);
+      }
     }
+    __syncwarp();
   }
-  finish_target(C, i, n, cidx, has, afluid, va, A, want_dt, ace, mu_out, dyn, sub == 0);
 }
 
-// G threads per target, in the key order of the targets (W: wide records).
-template <int EXT, int G, int W = 0>
-__global__ void __launch_bounds__(EXT == 0 ? 1024 : 128, EXT == 2 ? 6 : (EXT == 0 ? 1 : 0))
+// Adds the G lanes' partial sums; every lane ends with the same total.
+template <int G>
+__device__ __forceinline__ float group_sum(float x) {
+#pragma unroll
+  for (int o = 1; o < G; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+template <int G>
+__device__ __forceinline__ float group_max(float x) {
+#pragma unroll
+  for (int o = 1; o < G; o <<= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
+
+// Per-case counts, dt minimum and flags of a block: merged per warp, then per
+// run of warps of one case, so that an interior block reaches the case's words
+// with one atomic each (atomics on one address complete about 2 ns apart).
+// Lanes with cidx < 0 have nothing to add.  Every thread of the block calls it.
+__device__ __forceinline__ void reduce_block(int cidx, unsigned npairs, unsigned nfb,
+                                             unsigned nbf, unsigned dtbits, bool bad,
+                                             CaseDyn *dyn) {
+  __shared__ int s_c[32];
+  __shared__ unsigned s_v[32][5];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned act = __ballot_sync(full, cidx >= 0);
+  const int c0 = __shfl_sync(full, cidx, act ? __ffs(act) - 1 : 0);
+  const bool uniform = __all_sync(full, cidx < 0 || cidx == c0);
+  if (uniform) {
+    const bool on = cidx >= 0;
+    const unsigned p = __reduce_add_sync(full, on ? npairs : 0u);
+    const unsigned fb = __reduce_add_sync(full, on ? nfb : 0u);
+    const unsigned bf = __reduce_add_sync(full, on ? nbf : 0u);
+    const unsigned m = __reduce_min_sync(full, on ? dtbits : kFloatInfBits);
+    const unsigned b = __any_sync(full, on && bad);
+    if (lane == 0) {
+      s_c[w] = act ? c0 : -1;
+      s_v[w][0] = p;
+      s_v[w][1] = fb;
+      s_v[w][2] = bf;
+      s_v[w][3] = m;
+      s_v[w][4] = b;
+    }
+  } else {  // a warp across cases: each lane for itself
+    if (lane == 0) s_c[w] = -1;
+    if (cidx >= 0) {
+      if (npairs) atomicAdd(&dyn[cidx].pairs, (unsigned long long)npairs);
+      if (nfb) atomicAdd(&dyn[cidx].pairs_fb, (unsigned long long)nfb);
+      if (nbf) atomicAdd(&dyn[cidx].pairs_bf, (unsigned long long)nbf);
+      if (dtbits < kFloatInfBits) atomicMin(&dyn[cidx].dtmin_bits, dtbits);
+      if (bad) atomicOr(&dyn[cidx].flags, kFlagNaN);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const int nw = blockDim.x >> 5;
+  for (int k = 0; k < nw;) {
+    const int c = s_c[k];
+    unsigned long long p = 0, fb = 0, bf = 0;
+    unsigned m = kFloatInfBits, b = 0u;
+    for (; k < nw && s_c[k] == c; k++) {
+      if (c < 0) continue;
+      p += s_v[k][0];
+      fb += s_v[k][1];
+      bf += s_v[k][2];
+      m = min(m, s_v[k][3]);
+      b |= s_v[k][4];
+    }
+    if (c < 0) continue;
+    if (p) atomicAdd(&dyn[c].pairs, p);
+    if (fb) atomicAdd(&dyn[c].pairs_fb, fb);
+    if (bf) atomicAdd(&dyn[c].pairs_bf, bf);
+    // (the minimum only falls: a block above the value it reads, maybe an
+    // older one, leaves it)
+    if (m < *(volatile const unsigned *)&dyn[c].dtmin_bits) atomicMin(&dyn[c].dtmin_bits, m);
+    if (b) atomicOr(&dyn[c].flags, kFlagNaN);
+  }
+}
+
+// A target of the list walk as its G lanes see it.
+struct WalkTarget {
+  int cidx;
+  bool has, afluid;
+  unsigned cw;  // count word of its list (0: nothing to walk)
+  float4 pa, va;
+};
+__device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int nvalid) {
+  WalkTarget t;
+  const uint32_t key = i < nvalid ? a.keys[i] : key_out(a.nbits);
+  t.has = key < key_out(a.nbits);  // not frozen at this state
+  t.afluid = t.has && !key_boundary(key, a.nbits);
+  t.cidx = i < a.n ? (int)a.cid[i] : 0;
+  t.cw = t.has ? (unsigned)a.count[i] : 0u;
+  t.pa = a.walk[2 * (int64_t)i];  // (readable past the last particle)
+  t.va = t.has ? a.walk[2 * (int64_t)i + 1] : make_float4(0.f, 0.f, 0.f, 1.f);
+  return t;
+}
+
+// The interaction over the targets' lists (state n or n+1/2, same order and
+// cells): the pair terms of k_interact for the entries inside 2h.  EXT 1
+// adds the Eq 19-20 density diffusion, EXT 2 also laminar + SPS (tau4/tau2
+// from k_strain_list), for the cases that use them.  G lanes share a target;
+// a group takes a.per targets one after another (a warp covers 32 / G x per
+// consecutive targets), then lane q of the group finishes its q-th target, so
+// that the closing arithmetic runs on as many lanes as there are targets.
+template <int EXT, int G>
+__global__ void __launch_bounds__(EXT == 0 ? 1024 : 256, EXT == 0 ? 1 : 0)
 k_interact_list(const ListArgs a) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  list_target<EXT, G, W>(t / G, t % G, a);
+  const int lane = threadIdx.x & 31;
+  const int sub = lane % G;
+  constexpr int NG = 32 / G;
+  const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
+  const int nvalid = *a.nvalid_p;
+  const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
+  Acc K = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};  // sums of the lane's own target
+  unsigned npairs = 0u, nfb = 0u, nbf = 0u;
+  int ccase = -1;  // case of the counts
+#pragma unroll 1
+  for (int q = 0; q < a.per; q++) {
+    const int i = first + q * NG;
+    const WalkTarget t = walk_target(a, i, nvalid);
+    const CaseConst &C = a.cc[t.cidx];
+    const float Pa = t.pa.w * t.va.w;  // the record holds P / rho
+    const float kv = C.kvisc * t.va.w * C.inv_unit;
+    const bool ddt_on = C.ddt != 0;
+    Ext X;
+    X.C = &C;
+    X.unit = C.unit;
+    X.hyd = EXT >= 1 && C.ddt == 2;
+    X.sps = EXT == 2 && C.visc == 1 && t.afluid;
+    X.kl = -4.f * C.nu0 * t.va.w * C.inv_unit;
+    X.tau4 = a.tau4;
+    X.tau2 = a.tau2;
+    {
+      const float4 t4 = X.sps ? a.tau4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float2 t2 = X.sps ? a.tau2[i] : make_float2(0.f, 0.f);
+      X.ta[0] = t.va.w * t4.x;
+      X.ta[1] = t.va.w * t4.y;
+      X.ta[2] = t.va.w * t4.z;
+      X.ta[3] = t.va.w * t4.w;
+      X.ta[4] = t.va.w * t2.x;
+      X.ta[5] = t.va.w * t2.y;
+    }
+    const float hih = C.walk_hih, eta2 = C.walk_eta2;
+    Acc A = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};
+    walk_list<G>(a, i, sub, t.cw, t.pa, __float_as_uint(C.walk_r2max) - 1u,
+                 [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb, int j) {
+                   const bool bfluid = j < jb;
+                   if (t.afluid) {
+                     pair_fluid<EXT>(t.va, Pa, kv, hih, eta2, rx, ry, rz, r2, vb, Qb,
+                                     ddt_on && bfluid, A, &X, j, bfluid);
+                   } else {
+                     pair_boundary(t.va, hih, rx, ry, rz, r2, vb, A);
+                   }
+                   if (bfluid) A.cnt++; else A.cntb++;
+                 });
+    if (ccase != t.cidx) {  // the counts so far belong to another case
+      if (npairs) atomicAdd(&a.dyn[ccase].pairs, (unsigned long long)npairs);
+      if (nfb) atomicAdd(&a.dyn[ccase].pairs_fb, (unsigned long long)nfb);
+      if (nbf) atomicAdd(&a.dyn[ccase].pairs_bf, (unsigned long long)nbf);
+      npairs = nfb = nbf = 0u;
+      ccase = t.cidx;
+    }
+    npairs += A.cnt + A.cntb;
+    nfb += t.afluid ? A.cntb : 0u;
+    nbf += t.afluid ? 0u : A.cnt;
+    // the sums back from units of cs / 2^29
+    const float ax = group_sum<G>(A.ax), ay = group_sum<G>(A.ay), az = group_sum<G>(A.az);
+    const float s1 = group_sum<G>(A.s1), s2 = group_sum<G>(A.s2), mur = group_max<G>(A.mur);
+    if (sub == q) {
+      K.ax = C.unit * ax;
+      K.ay = C.unit * ay;
+      K.az = C.unit * az;
+      K.s1 = C.unit * s1;
+      K.s2 = s2;
+      K.mur = C.inv_unit * mur;
+    }
+  }
+  const int i = first + sub * NG;
+  const bool own = sub < a.per && i < nvalid && a.keys[i] < key_out(a.nbits);
+  unsigned dtbits = kFloatInfBits;
+  bool bad = false;
+  int cidx = ccase;
+  if (own) {
+    cidx = (int)a.cid[i];
+    finish_values(a.cc[cidx], i, !key_boundary(a.keys[i], a.nbits), a.walk[2 * (int64_t)i + 1].w,
+                  K, a.want_dt, a.ace, a.mu_out, dtbits, bad);
+    if (cidx != ccase) {  // the lane's counts and its own target differ in case
+      if (dtbits < kFloatInfBits) atomicMin(&a.dyn[cidx].dtmin_bits, dtbits);
+      if (bad) atomicOr(&a.dyn[cidx].flags, kFlagNaN);
+      dtbits = kFloatInfBits;
+      bad = false;
+      cidx = ccase;
+    }
+  }
+  reduce_block(first < a.n ? cidx : -1, npairs, nfb, nbf, dtbits, bad, a.dyn);
 }
-
-
 
 // Each pair once (the default physics of Eq 15, 17-18, 21-22 and 36, DBC):
 // the momentum term of a pair is antisymmetric, -m cw F r_ab on a and
 // +m cw F r_ab on b with F = t^3 [(P_a + P_b)/(rho_a rho_b) + kvisc
 // min(v_ab.r_ab, 0)/((r^2 + eta^2)(rho_a + rho_b))], and the continuity
-// terms of a and b share t^3 v_ab.r_ab.  A fluid target walks its records
-// and takes only the candidates of larger index (in the fluid-first key
-// order every boundary particle has a larger index than every fluid one, so
-// boundary targets walk nothing); it adds its own terms in registers and the
-// partner's with one vector atomic add into sum[b] = (sum_c F_bc r_bc,
-// continuity / (m cw)), then its own sums the same way.  The order of the
-// atomic additions varies, so the sums are not reproducible bit for bit.
+// terms of a and b share t^3 v_ab.r_ab.  A fluid target walks its half list
+// (candidates of larger index; in the fluid-first key order every boundary
+// particle has a larger index than every fluid one, so boundary targets walk
+// nothing); it adds its own terms in registers and the partner's with one
+// vector atomic add into sum[b] = (sum_c F_bc r_bc, continuity / (m cw)), then
+// its own sums the same way.  Sums and mu are in units of cs / 2^29 (the
+// positions' unit; k_sym_finish converts).  The order of the atomic additions
+// varies, so the sums are not reproducible bit for bit.
 // k_sym_finish turns the sums into dv/dt, drho/dt and the Eq 35 terms.
-template <int W>
-__global__ void __launch_bounds__(128)
+template <int G>
+__global__ void __launch_bounds__(256)
 k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict__ mu_bits) {
-  const unsigned full = 0xffffffffu;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = a.n;
-  const int nbits = a.nbits;
-  const float4 *__restrict__ posc = a.posc;
-  const float4 *__restrict__ velrho = a.velrho;
-  const float *__restrict__ press = a.press;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane % G;
+  constexpr int NG = 32 / G;
+  const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
-  const uint32_t key = i < nvalid ? a.keys[i] : key_out(nbits);
-  const bool has = key < key_out(nbits);
-  const int cidx = i < n ? (int)a.cid[i] : 0;
-  const CaseConst &C = a.cc[cidx];
-  const bool afluid = has && !key_boundary(key, nbits);
-  const float cs = C.csf, eta2 = C.eta2, hih = C.half_inv_h, kvisc = C.kvisc, kddt = C.kddt;
-  const unsigned r2max_u = __float_as_uint(C.r2max) - 1u;
-  const float4 pa = afluid ? posc[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 va = afluid ? velrho[i] : make_float4(0.f, 0.f, 0.f, 1.f);
-  const float Qa = afluid ? press[i] : 0.f;  // P_a / rho_a
-  const float ia = __fdividef(1.f, va.w);
-  const bool ddt_on = C.ddt != 0;
   const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
-  const int nrec = afluid ? (int)a.count[i] : 0;
-  const uint2 *__restrict__ mine = a.list + (int64_t)i * a.cap;
-  float fx = 0.f, fy = 0.f, fz = 0.f, cont = 0.f, mur = 0.f;
-  unsigned nff = 0u, nfb = 0u;
-  int r = 0;
-  unsigned cm = 0u;
-  int cbase = 0;
-  float sy = 0.f, sz = 0.f;
-  // the next record of the lane, keeping only candidates of index > i
-  int tcy = 0, tcz = 0;  // wide records: rows relative to the target's cell
-  if (W && nrec) {
-    int tcx;
-    decode_cell(key_cell(a.row_keys[i], nbits) - C.cellbase, C.nx, C.ny, tcx, tcy, tcz);
-  }
-  auto next_record = [&]() {
-    const uint2 rec = mine[r++];
-    cbase = W ? (int)rec.x : (int)(rec.x & kListIndexMask);
-    const int lowk = i - cbase + 1;  // first bit of a larger index
-    cm = lowk <= 0 ? rec.y : (lowk >= 32 ? 0u : rec.y & (0xffffffffu << lowk));
-    int rdy, rdz;
-    if (W) {
-      int bx, by, bz;
-      decode_cell(key_cell(a.row_keys[cbase], nbits) - C.cellbase, C.nx, C.ny, bx, by, bz);
-      rdy = by - tcy;
-      rdz = bz - tcz;
-    } else {
-      list_row_decode(rec.x, rdy, rdz);
-    }
-    sy = fmaf(-(float)rdy, cs, pa.y);
-    sz = fmaf(-(float)rdz, cs, pa.z);
-  };
+  unsigned nall = 0u, nfb = 0u;
+  int ccase = -1;
 #pragma unroll 1
-  for (;;) {
-    while (cm == 0u && r < nrec) next_record();
-    if (!__any_sync(full, cm != 0u)) break;
-    if (cm) {
-      const int k1 = 31 - __clz(cm);
-      cm ^= 1u << k1;
-      const int j1 = cbase + k1;
-      const float sy1 = sy, sz1 = sz;
-      while (cm == 0u && r < nrec) next_record();
-      const bool h2 = cm != 0u;
-      const int k2 = h2 ? 31 - __clz(cm) : k1;
-      if (h2) cm ^= 1u << k2;
-      const int j2 = h2 ? cbase + k2 : j1;
-      const float4 pb1 = posc[j1];
-      const float4 pb2 = posc[j2];
-      const float4 vb1 = velrho[j1];
-      const float4 vb2 = velrho[j2];
-      const float q1 = press[j1], q2 = press[j2];
-#pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const float4 pb = u ? pb2 : pb1;
-        const float4 vb = u ? vb2 : vb1;
-        const int j = u ? j2 : j1;
-        const float rx = fmaf(pa.w - pb.w, cs, pa.x - pb.x);
-        const float ry = (u ? sy : sy1) - pb.y, rz = (u ? sz : sz1) - pb.z;
-        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        if ((u == 0 || h2) && __float_as_uint(r2) - 1u < r2max_u) {
-          const bool bfluid = j < jb;
-          const float rr = r2 * rsqrtf(r2);
-          const float t = fmaf(-hih, rr, 1.f);
-          const float t3 = t * t * t;
-          const float vx = va.x - vb.x, vy = va.y - vb.y, vz = va.z - vb.z;
-          const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
-          const float ib = __fdividef(1.f, vb.w);
-          const float sab = va.w + vb.w;
-          const float ie = __fdividef(1.f, (r2 + eta2) * sab);
-          mur = fmaxf(mur, fabsf(vr * ie * sab));
-          const float pi = fminf(vr, 0.f) * ie;
-          const float F = t3 * fmaf(kvisc, pi, fmaf(Qa, ib, (u ? q2 : q1) * ia));
-          fx = fmaf(F, rx, fx);
-          fy = fmaf(F, ry, fy);
-          fz = fmaf(F, rz, fz);
-          // Eq 17-18 between fluid particles: d = rho_b - rho_a
-          const float d = (ddt_on && bfluid) ? vb.w - va.w : 0.f;
-          cont = fmaf(t3 * ib, fmaf(va.w, vr, -kddt * d), cont);
-          // b: -F r_ab (its r_ba = -r_ab), t^3/rho_a (rho_b v.r + kddt d)
-          const float cb = t3 * ia * fmaf(vb.w, vr, kddt * d);
-          atomicAdd(&sum[j], make_float4(-F * rx, -F * ry, -F * rz, cb));
-          // each particle's own mu_max (an output only when asked for; the
-          // Eq 35 minimum needs only the largest over all pairs)
-          if (a.mu_out) atomicMax(&mu_bits[j], __float_as_uint(fabsf(vr * ie * sab)));
-          if (bfluid) nff++; else nfb++;
-        }
+  for (int q = 0; q < a.per; q++) {
+    const int i = first + q * NG;
+    const WalkTarget t = walk_target(a, i, nvalid);
+    const CaseConst &C = a.cc[t.cidx];
+    if (ccase != t.cidx) {  // the counts so far belong to another case
+      if (nall) atomicAdd(&a.dyn[ccase].pairs, 2ull * nall);
+      if (nfb) {
+        atomicAdd(&a.dyn[ccase].pairs_fb, (unsigned long long)nfb);
+        atomicAdd(&a.dyn[ccase].pairs_bf, (unsigned long long)nfb);
       }
+      nall = nfb = 0u;
+      ccase = t.cidx;
     }
-  }
-  if (afluid) {
-    atomicAdd(&sum[i], make_float4(fx, fy, fz, cont));
-    atomicMax(&mu_bits[i], __float_as_uint(mur));
+    const float eta2 = C.walk_eta2, hih = C.walk_hih;
+    const float kvisc = C.kvisc * C.inv_unit, kddt = C.kddt * C.inv_unit;
+    const float Qa = t.pa.w;  // P_a / rho_a
+    const float ia = __fdividef(1.f, t.va.w);
+    const bool ddt_on = C.ddt != 0;
+    float fx = 0.f, fy = 0.f, fz = 0.f, cont = 0.f, mur = 0.f;
+    walk_list<G>(a, i, sub, t.afluid ? t.cw : 0u, t.pa, __float_as_uint(C.walk_r2max) - 1u,
+                 [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb, int j) {
+                   const bool bfluid = j < jb;
+                   const float rr = r2 * rsqrtf(r2);
+                   const float t1 = fmaf(-hih, rr, 1.f);
+                   const float t3 = t1 * t1 * t1;
+                   const float vx = t.va.x - vb.x, vy = t.va.y - vb.y, vz = t.va.z - vb.z;
+                   const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
+                   const float ib = __fdividef(1.f, vb.w);
+                   const float sab = t.va.w + vb.w;
+                   const float ie = __fdividef(1.f, (r2 + eta2) * sab);
+                   const float mu = fabsf(vr * ie * sab);
+                   mur = fmaxf(mur, mu);
+                   const float pi = fminf(vr, 0.f) * ie;
+                   const float F = t3 * fmaf(kvisc, pi, fmaf(Qa, ib, Qb * ia));
+                   fx = fmaf(F, rx, fx);
+                   fy = fmaf(F, ry, fy);
+                   fz = fmaf(F, rz, fz);
+                   // Eq 17-18 between fluid particles: d = rho_b - rho_a
+                   const float d = (ddt_on && bfluid) ? vb.w - t.va.w : 0.f;
+                   cont = fmaf(t3 * ib, fmaf(t.va.w, vr, -kddt * d), cont);
+                   // b: -F r_ab (its r_ba = -r_ab), t^3/rho_a (rho_b v.r + kddt d)
+                   const float cb = t3 * ia * fmaf(vb.w, vr, kddt * d);
+                   atomicAdd(&sum[j], make_float4(-F * rx, -F * ry, -F * rz, cb));
+                   // each particle's own mu_max (an output only when asked for;
+                   // the Eq 35 minimum needs only the largest over all pairs)
+                   if (a.mu_out) atomicMax(&mu_bits[j], __float_as_uint(mu));
+                   nall++;
+                   if (!bfluid) nfb++;
+                 });
+    fx = group_sum<G>(fx);
+    fy = group_sum<G>(fy);
+    fz = group_sum<G>(fz);
+    cont = group_sum<G>(cont);
+    mur = group_max<G>(mur);
+    if (sub == 0 && t.afluid) {
+      atomicAdd(&sum[i], make_float4(fx, fy, fz, cont));
+      atomicMax(&mu_bits[i], __float_as_uint(mur));
+    }
   }
   // directed pairs: an unordered fluid pair is two, a fluid-boundary pair is
   // one of each kind
-  reduce_case(i < n ? cidx : -1, has, 2u * nff + 2u * nfb, nfb, nfb, kFloatInfBits, false,
-              a.dyn);
+  reduce_block(first < a.n ? ccase : -1, 2u * nall, nfb, nfb, kFloatInfBits, false, a.dyn);
 }
 
 // dv/dt = g - m cw sum.xyz for fluid particles (0 for boundary ones), drho/dt
@@ -2170,9 +2310,9 @@ k_sym_finish(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict__ 
     if (has) {
       const CaseConst &C = a.cc[cidx];
       const bool afluid = !key_boundary(key[k], nbits);
-      const float mcw = C.m * C.cw;
+      const float mcw = C.m * C.cw * C.unit;  // the walk's sums are in units of C.unit
       float4 out;
-      float mumax = C.h * __uint_as_float(mb[k]);
+      float mumax = C.h * C.inv_unit * __uint_as_float(mb[k]);
       if (afluid) {
         out.x = fmaf(-mcw, sm[k].x, C.g[0]);
         out.y = fmaf(-mcw, sm[k].y, C.g[1]);
@@ -2245,79 +2385,51 @@ k_sym_finish(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict__ 
 }
 
 // The strain pass of the laminar + SPS model (as k_strain) over the target's
-// list records, for the half-step state kept in the order and cells of state n.
-__global__ void __launch_bounds__(128)
-k_strain_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ keys,
-              const float4 *__restrict__ posc, const float4 *__restrict__ velrho,
-              const uint16_t *__restrict__ cid, int nbits, const CaseConst *__restrict__ cc,
-              const uint2 *__restrict__ list, int cap, const uint16_t *__restrict__ count,
-              float4 *__restrict__ tau4, float2 *__restrict__ tau2) {
-  const unsigned full = 0xffffffffu;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nvalid = *nvalid_p;
-  const uint32_t key = i < nvalid ? keys[i] : key_out(nbits);
-  const int cidx = i < n ? (int)cid[i] : 0;
-  const CaseConst &C = cc[cidx];
-  const bool act = key < key_out(nbits) && !key_boundary(key, nbits) && C.visc == 1;
-  if (__all_sync(full, !act)) {
-    if (i < n) {
+// list, for the half-step state kept in the order and cells of state n; lanes
+// and targets as in k_interact_list.
+template <int G>
+__global__ void __launch_bounds__(256)
+k_strain_list(const ListArgs a, float4 *__restrict__ tau4, float2 *__restrict__ tau2) {
+  const int lane = threadIdx.x & 31;
+  const int sub = lane % G;
+  constexpr int NG = 32 / G;
+  const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
+  const int nvalid = *a.nvalid_p;
+#pragma unroll 1
+  for (int q = 0; q < a.per; q++) {
+    const int i = first + q * NG;
+    const WalkTarget t = walk_target(a, i, nvalid);
+    const CaseConst &C = a.cc[t.cidx];
+    const bool act = t.afluid && C.visc == 1;
+    const float hih = C.walk_hih;
+    float gxx = 0.f, gyy = 0.f, gzz = 0.f, gxy = 0.f, gxz = 0.f, gyz = 0.f;
+    walk_list<G>(a, i, sub, act ? t.cw : 0u, t.pa, __float_as_uint(C.walk_r2max) - 1u,
+                 [&](float rx, float ry, float rz, float r2, const float4 &vb, float, int) {
+                   const float t1 = fmaf(-hih, r2 * rsqrtf(r2), 1.f);
+                   const float w = t1 * t1 * t1 * __fdividef(1.f, vb.w);
+                   const float dvx = vb.x - t.va.x, dvy = vb.y - t.va.y, dvz = vb.z - t.va.z;
+                   gxx = fmaf(w * dvx, rx, gxx);
+                   gyy = fmaf(w * dvy, ry, gyy);
+                   gzz = fmaf(w * dvz, rz, gzz);
+                   gxy = fmaf(w, fmaf(dvx, ry, dvy * rx), gxy);
+                   gxz = fmaf(w, fmaf(dvx, rz, dvz * rx), gxz);
+                   gyz = fmaf(w, fmaf(dvy, rz, dvz * ry), gyz);
+                 });
+    const float u = C.unit;  // the sums back from units of cs / 2^29
+    gxx = u * group_sum<G>(gxx);
+    gyy = u * group_sum<G>(gyy);
+    gzz = u * group_sum<G>(gzz);
+    gxy = u * group_sum<G>(gxy);
+    gxz = u * group_sum<G>(gxz);
+    gyz = u * group_sum<G>(gyz);
+    if (sub != 0 || i >= a.n) continue;
+    if (!act) {
       tau4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       tau2[i] = make_float2(0.f, 0.f);
-    }
-    return;
-  }
-  const float cs = C.csf, hih = C.half_inv_h;
-  const unsigned r2max_u = __float_as_uint(C.r2max) - 1u;
-  const float4 pa = act ? posc[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 va = act ? velrho[i] : make_float4(0.f, 0.f, 0.f, 1.f);
-  const int nrec = act ? (int)count[i] : 0;
-  const uint2 *__restrict__ mine = list + (int64_t)i * cap;
-  float gxx = 0.f, gyy = 0.f, gzz = 0.f, gxy = 0.f, gxz = 0.f, gyz = 0.f;
-  int r = 0;
-  unsigned cm = 0u;
-  int cbase = 0;
-  float sy = 0.f, sz = 0.f;
-#pragma unroll 1
-  for (;;) {
-    if (cm == 0u && r < nrec) {
-      const uint2 rec = mine[r++];
-      cbase = (int)(rec.x & kListIndexMask);
-      cm = rec.y;
-      int rdy, rdz;
-      list_row_decode(rec.x, rdy, rdz);
-      sy = fmaf(-(float)rdy, cs, pa.y);
-      sz = fmaf(-(float)rdz, cs, pa.z);
-    }
-    if (!__any_sync(full, cm != 0u)) break;
-    if (cm) {
-      const int k = 31 - __clz(cm);
-      cm ^= 1u << k;
-      const int j = cbase + k;
-      const float4 pb = posc[j];
-      const float rx = fmaf(pa.w - pb.w, cs, pa.x - pb.x);
-      const float ry = sy - pb.y, rz = sz - pb.z;
-      const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-      if (__float_as_uint(r2) - 1u < r2max_u) {
-        const float4 vb = velrho[j];
-        const float t = fmaf(-hih, r2 * rsqrtf(r2), 1.f);
-        const float w = t * t * t * __fdividef(1.f, vb.w);
-        const float dvx = vb.x - va.x, dvy = vb.y - va.y, dvz = vb.z - va.z;
-        gxx = fmaf(w * dvx, rx, gxx);
-        gyy = fmaf(w * dvy, ry, gyy);
-        gzz = fmaf(w * dvz, rz, gzz);
-        gxy = fmaf(w, fmaf(dvx, ry, dvy * rx), gxy);
-        gxz = fmaf(w, fmaf(dvx, rz, dvz * rx), gxz);
-        gyz = fmaf(w, fmaf(dvy, rz, dvz * ry), gyz);
-      }
+    } else {
+      sps_tau_from_gradient(C, gxx, gyy, gzz, gxy, gxz, gyz, tau4[i], tau2[i]);
     }
   }
-  if (i >= n) return;
-  if (!act) {
-    tau4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    tau2[i] = make_float2(0.f, 0.f);
-    return;
-  }
-  sps_tau_from_gradient(C, gxx, gyy, gzz, gxy, gxz, gyz, tau4[i], tau2[i]);
 }
 
 // Half step for the list path: state n+1/2 in the same order and the same
@@ -2331,7 +2443,8 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
                                  const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
                                  int nbits, float4 *__restrict__ posc_out,
                                  float4 *__restrict__ velrho_out, uint32_t *__restrict__ keys_out,
-                                 float *__restrict__ press, const float4 *__restrict__ ref) {
+                                 float *__restrict__ press, const float4 *__restrict__ ref,
+                                 float4 *__restrict__ walk) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   // every load of the particle first (independent: one memory latency)
@@ -2368,14 +2481,18 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
     posc_out[i] = make_float4(1e30f, 1e30f, 1e30f, p.w);
     velrho_out[i] = v;
     keys_out[i] = key_out(nbits);
+    walk[2 * (int64_t)i + 1] = make_float4(0.f, 0.f, 0.f, -1.f);  // no density: in no pair
     atomicAdd(&dyn[cidx].n_out, 1);
     return;
   }
-  posc_out[i] = make_float4((float)((double)p.x + disp[0]), (float)((double)p.y + disp[1]),
-                            (float)((double)p.z + disp[2]), p.w);
+  const float4 ph = make_float4((float)((double)p.x + disp[0]), (float)((double)p.y + disp[1]),
+                                (float)((double)p.z + disp[2]), p.w);
+  const float Q = tait_pressure(C, vn.w) / vn.w;  // P/rho of Eq 28 at n+1/2
+  posc_out[i] = ph;
   velrho_out[i] = vn;
   keys_out[i] = k;
-  press[i] = tait_pressure(C, vn.w) / vn.w;  // P/rho of Eq 28 at n+1/2
+  press[i] = Q;
+  put_walk(walk, i, C, k, nbits, ph, vn, Q);
 }
 
 // Full step for the list path, in the order of state n (sn): writes state n+1
@@ -2436,7 +2553,8 @@ __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
                                   const float4 *__restrict__ ace, const float4 *__restrict__ ref,
                                   const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
                                   int nbits, State x, uint32_t *__restrict__ keys_next,
-                                  float *__restrict__ press, ListCtl *__restrict__ ctl) {
+                                  float *__restrict__ press, ListCtl *__restrict__ ctl,
+                                  float4 *__restrict__ walk) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   // every load of the particle first (independent: one memory latency)
@@ -2490,7 +2608,9 @@ __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
                                 (float)((double)pn.z + disp[2]), pn.w);
   y.posc[i] = pu;
   y.velrho[i] = vnew;
-  press[i] = tait_pressure(C, vnew.w) / vnew.w;
+  const float Q = tait_pressure(C, vnew.w) / vnew.w;
+  press[i] = Q;
+  put_walk(walk, i, C, k, nbits, pu, vnew, Q);
   const float dx = pu.x - r.x, dy = pu.y - r.y, dz = pu.z - r.z;
   const float v = sqrtf(fmaf(vnew.x, vnew.x, fmaf(vnew.y, vnew.y, vnew.z * vnew.z)));
   const float e = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) + 0.5f * C.list_k * v;
@@ -2509,16 +2629,16 @@ __global__ void k_decide(cudaGraphConditionalHandle h, const ListCtl *__restrict
 // Brute-force check of a neighbour list (an option for tests, off by
 // default): for every target of the evaluated state, the pairs inside 2h over
 // all particles of its case (boundary targets: fluid neighbours only, Eq 36)
-// are counted with the list walk's own arithmetic (cells of the keys, FP32
-// offsets) and compared with the pairs its list records yield.  Adds the
-// brute-force pairs to ctl->check_pairs and every mismatching target to
-// ctl->check_bad.
+// are counted with the list walk's own arithmetic (walk_r2; the cells of the
+// keys rule out what its wrapping positions alias) and compared with the pairs
+// its list yields.  Adds the brute-force pairs to ctl->check_pairs and every
+// mismatching target to ctl->check_bad.
 __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
                              const uint32_t *__restrict__ keys, const float4 *__restrict__ posc,
                              const uint16_t *__restrict__ cid, const CaseConst *__restrict__ cc,
                              int nbits, const uint2 *__restrict__ list, int cap,
                              const uint16_t *__restrict__ count, ListCtl *__restrict__ ctl,
-                             int half, const uint32_t *__restrict__ row_keys) {
+                             int half, const float4 *__restrict__ walk) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int nvalid = *nvalid_p;
   if (i >= nvalid || i >= n) return;
@@ -2529,11 +2649,16 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
   const CaseConst &C = cc[cidx];
   if (!afluid && C.bmode == 1) return;  // mDBC boundary: no pair terms (Eq 38 instead)
   const float cs = C.csf;
-  const unsigned r2max_u = __float_as_uint(C.r2max) - 1u;
-  const float4 pa = posc[i];
+  const unsigned r2max_u = __float_as_uint(C.walk_r2max) - 1u;
+  const float4 pa = posc[i], wa = walk[2 * (int64_t)i];
   int cx, cy, cz;
   decode_cell(key_cell(k, nbits) - C.cellbase, C.nx, C.ny, cx, cy, cz);
   unsigned nb = 0u, nl = 0u;
+  auto inside = [&](int j) {
+    float rx, ry, rz;
+    const float r2 = walk_r2(wa, walk[2 * (int64_t)j], rx, ry, rz);
+    return __float_as_uint(r2) - 1u < r2max_u && walk[2 * (int64_t)j + 1].w > 0.f;
+  };
   for (int j = 0; j < nvalid; j++) {
     const uint32_t kj = keys[j];
     if (cid[j] != cidx || kj >= key_out(nbits) || (!afluid && key_boundary(kj, nbits))) continue;
@@ -2541,34 +2666,20 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
     int jx, jy, jz;
     decode_cell(key_cell(kj, nbits) - C.cellbase, C.nx, C.ny, jx, jy, jz);
     const float4 pb = posc[j];
-    const float rx = fmaf(pa.w - pb.w, cs, pa.x - pb.x);
-    const float ry = fmaf(-(float)(jy - cy), cs, pa.y) - pb.y;
-    const float rz = fmaf(-(float)(jz - cz), cs, pa.z) - pb.z;
-    const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-    if (__float_as_uint(r2) - 1u < r2max_u) nb++;
+    const float rx = fmaf((float)(cx - jx), cs, pa.x - pb.x);
+    const float ry = fmaf((float)(cy - jy), cs, pa.y - pb.y);
+    const float rz = fmaf((float)(cz - jz), cs, pa.z - pb.z);
+    if (fmaxf(fabsf(rx), fmaxf(fabsf(ry), fabsf(rz))) < 4.f * cs && inside(j)) nb++;
   }
-  for (int r = 0; r < (int)count[i]; r++) {
-    const uint2 rec = list[(int64_t)i * cap + r];
-    const int cbase = row_keys ? (int)rec.x : (int)(rec.x & kListIndexMask);
-    int rdy, rdz;
-    if (row_keys) {  // wide records: the row from the first candidate's cell
-      int bx, by, bz, tx, ty, tz;
-      decode_cell(key_cell(row_keys[cbase], nbits) - C.cellbase, C.nx, C.ny, bx, by, bz);
-      decode_cell(key_cell(row_keys[i], nbits) - C.cellbase, C.nx, C.ny, tx, ty, tz);
-      rdy = by - ty;
-      rdz = bz - tz;
-    } else {
-      list_row_decode(rec.x, rdy, rdz);
-    }
-    const float sy = fmaf(-(float)rdy, cs, pa.y);
-    const float sz = fmaf(-(float)rdz, cs, pa.z);
-    for (unsigned m = rec.y; m; m &= m - 1u) {
-      const float4 pb = posc[cbase + __ffs(m) - 1];
-      const float rx = fmaf(pa.w - pb.w, cs, pa.x - pb.x);
-      const float ry = sy - pb.y, rz = sz - pb.z;
-      const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-      if (__float_as_uint(r2) - 1u < r2max_u) nl++;
-    }
+  const unsigned cw = count[i];
+  const uint2 *seg = list + (int64_t)i * cap;
+  if (cw & kListRecords) {
+    for (int r = 0; r < (int)(cw & ~kListRecords); r++)
+      for (unsigned m = seg[r].y; m; m &= m - 1u)
+        if (inside((int)seg[r].x + __ffs(m) - 1)) nl++;
+  } else {
+    for (int r = 0; r < (int)cw; r++)
+      if (inside((int)reinterpret_cast<const uint32_t *>(seg)[r])) nl++;
   }
   atomicAdd(&ctl->check_pairs, (unsigned long long)nb);
   if (nb != nl) atomicAdd(&ctl->check_bad, 1ull);
@@ -2594,7 +2705,8 @@ __global__ void k_verlet(int n, const uint32_t *__restrict__ keys_in, State src,
                          const float4 *__restrict__ ace, const CaseConst *__restrict__ cc,
                          CaseDyn *__restrict__ dyn, int nbits, State dst,
                          uint32_t *__restrict__ keys_out, const float4 *__restrict__ ref = nullptr,
-                         float *__restrict__ press = nullptr, ListCtl *__restrict__ ctl = nullptr) {
+                         float *__restrict__ press = nullptr, ListCtl *__restrict__ ctl = nullptr,
+                         float4 *__restrict__ walk = nullptr) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t k = keys_in[i];
@@ -2667,7 +2779,9 @@ __global__ void k_verlet(int n, const uint32_t *__restrict__ keys_in, State src,
     src.posc[i] = pu;
     src.velrho[i] = vnew;
     src.vrprev[i] = v;
-    press[i] = tait_pressure(C, vnew.w) / vnew.w;
+    const float Q = tait_pressure(C, vnew.w) / vnew.w;
+    press[i] = Q;
+    put_walk(walk, i, C, k, nbits, pu, vnew, Q);
     const float4 r = ref[i];
     const float dx = pu.x - r.x, dy = pu.y - r.y, dz = pu.z - r.z;
     if (sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) > 0.5f * (D.skin - 1e-3f * C.h)) {
@@ -2908,11 +3022,11 @@ void launch_reorder(int n, const uint32_t *perm, const uint32_t *keys_sorted,
                     const uint16_t *cid, const uint8_t *code, const float4 *vrprev,
                     const float4 *ghost, State dst, float *press, const CaseConst *cc,
                     CaseDyn *dyn, int nbits, cudaStream_t s, const float4 *ref_src,
-                    float4 *ref_dst) {
+                    float4 *ref_dst, float4 *walk) {
   if (n > 0)
     k_reorder<<<nblk(n, 256), 256, 0, s>>>(n, perm, keys_sorted, posc, velrho, id, cid, code,
                                            vrprev, ghost, dst, press, cc, dyn, nbits, ref_src,
-                                           ref_dst);
+                                           ref_dst, walk);
 }
 
 size_t cells_temp_words(int64_t cap_cells) {
@@ -3025,11 +3139,11 @@ void launch_corrector(int n, const uint32_t *perm2, const uint32_t *keys_half,
 
 void launch_mdbc(int margin, int n, const int *nvalid, const uint32_t *keys, State st,
                  float *press, const uint32_t *cstart, int nbits, const CaseConst *cc,
-                 const CaseDyn *dyn, int stage, cudaStream_t s, bool list) {
+                 const CaseDyn *dyn, int stage, cudaStream_t s, bool list, float4 *walk) {
   if (n <= 0) return;
 #define SPH_MD(MM, LL)                                                                    \
   k_mdbc<MM, LL><<<nblk(n, 128), 128, 0, s>>>(n, nvalid, keys, st, press, cstart, nbits, cc, \
-                                              dyn, stage)
+                                              dyn, stage, walk)
   if (margin == 1) {
     if (list) SPH_MD(1, true); else SPH_MD(1, false);
   } else if (margin == 3) {
@@ -3040,58 +3154,65 @@ void launch_mdbc(int margin, int n, const int *nvalid, const uint32_t *keys, Sta
 #undef SPH_MD
 }
 
-void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
-                          const float4 *velrho, const float *press, const uint16_t *cid,
-                          const uint32_t *cstart, int64_t cap_cells, int nbits,
-                          const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
+// Targets that a group of G lanes takes one after another: as many (at most G)
+// as leave 128 warps per SM, some five rounds of its resident ones.  More
+// targets per group share the closing arithmetic, but fewer, longer warps leave
+// the last round emptier.  Measured per evaluation at 1 / 2 / 4 / 8 targets
+// (G = 8): 28k particles 12 / 16 / 27 / 47 us, 167k 91 / 81 / 82 / 91, batch of
+// 420k 305 / 260 / 246 / 248, 1.5M 736 / 635 / 598 / 586.
+static inline int walk_targets(int n, int G) {
+  int per = 1;
+  while (per < G && (int64_t)n * G / 32 / (2 * per) >= 152 * 128) per *= 2;
+  return per;
+}
+
+void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *walk,
+                          const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,
+                          int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
                           float4 *tau4, float2 *tau2, cudaStream_t s, float *mu, int block,
-                          int lanes, float4 *sym_sum, unsigned *sym_mu,
-                          const uint32_t *wide_keys) {
+                          int lanes, float4 *sym_sum, unsigned *sym_mu) {
   if (n <= 0) return;
-  if (lanes != 2 && lanes != 4 && lanes != 8) lanes = 1;
-  const ListArgs a{n,     nvalid, keys,  posc,  velrho, press,  cid,  cstart,
-                   (uint32_t)(cap_cells + 1), nbits, cc, dyn,  ace,  want_dt, list,
-                   cap,   count,  tau4,  tau2,  mu,     wide_keys};
-  if (wide_keys) {  // wide records: the default physics only, one thread per target
-    if (sym_sum) {
-      k_interact_sym<1><<<nblk(n, 128), 128, 0, s>>>(a, sym_sum, sym_mu);
-      k_sym_finish<<<nblk(n, kFinishThreads * kFinishPer), kFinishThreads, 0, s>>>(
-          a, sym_sum, sym_mu);
-    } else {
-      k_interact_list<0, 1, 1><<<nblk(n, 128), 128, 0, s>>>(a);
-    }
-    return;
+  const int G = lanes == 1 || lanes == 2 || lanes == 4 ? lanes : 8;
+  const int per = walk_targets(n, G);
+  const ListArgs a{n,    nvalid, keys, walk, cid,   cstart, (uint32_t)(cap_cells + 1),
+                   nbits, cc,    dyn,  ace,  want_dt, list, cap, count, tau4, tau2, mu, per};
+  // block size of the default kernel as asked for (pi_block); its default 256,
+  // and always for the others (registers)
+  const int b0 = block >= 128 && block <= 1024 && block % 32 == 0 ? block : 256;
+  const int64_t threads = (n + (int64_t)per * (32 / G) - 1) / (per * (32 / G)) * 32;
+#define SPH_LANES(CALL) \
+  switch (G) {          \
+    case 1: CALL(1); break; \
+    case 2: CALL(2); break; \
+    case 4: CALL(4); break; \
+    default: CALL(8); break; \
   }
   if (sym_sum && !ext && !tau4) {  // each pair once, then the per-particle values
-    k_interact_sym<0><<<nblk(n, 128), 128, 0, s>>>(a, sym_sum, sym_mu);
+#define SPH_SYM(GG) k_interact_sym<GG><<<nblk(threads, 256), 256, 0, s>>>(a, sym_sum, sym_mu)
+    SPH_LANES(SPH_SYM)
+#undef SPH_SYM
     k_sym_finish<<<nblk(n, kFinishThreads * kFinishPer), kFinishThreads, 0, s>>>(a, sym_sum,
                                                                                  sym_mu);
     return;
   }
-  if (tau4)  // laminar + SPS cases present: strain pass over the list first
-    k_strain_list<<<nblk(n, 128), 128, 0, s>>>(n, nvalid, keys, posc, velrho, cid, nbits, cc,
-                                               list, cap, count, tau4, tau2);
-  // G = lanes threads per target; block size 128 (default) to 1024 for the
-  // default kernel (EXT 1 and 2: 128, by their registers)
-  const int b0 = block >= 128 && block <= 1024 && block % 32 == 0 ? block : 128;
-  const int64_t nt = (int64_t)n * lanes;
-  const int g1 = (int)((nt + 127) / 128), g0 = (int)((nt + b0 - 1) / b0);
-#define SPH_LIST(EXT, GRID, BLK)                                                      \
-  switch (lanes) {                                                                  \
-    case 2: k_interact_list<EXT, 2><<<GRID, BLK, 0, s>>>(a); break;                 \
-    case 4: k_interact_list<EXT, 4><<<GRID, BLK, 0, s>>>(a); break;                 \
-    case 8: k_interact_list<EXT, 8><<<GRID, BLK, 0, s>>>(a); break;                 \
-    default: k_interact_list<EXT, 1><<<GRID, BLK, 0, s>>>(a); break;                \
-  }
-  if (tau4) {
-    SPH_LIST(2, g1, 128)
+  if (tau4) {  // laminar + SPS cases present: strain pass over the list first
+#define SPH_STR(GG) k_strain_list<GG><<<nblk(threads, 256), 256, 0, s>>>(a, tau4, tau2)
+    SPH_LANES(SPH_STR)
+#undef SPH_STR
+#define SPH_L2(GG) k_interact_list<2, GG><<<nblk(threads, 256), 256, 0, s>>>(a)
+    SPH_LANES(SPH_L2)
+#undef SPH_L2
   } else if (ext) {
-    SPH_LIST(1, g1, 128)
+#define SPH_L1(GG) k_interact_list<1, GG><<<nblk(threads, 256), 256, 0, s>>>(a)
+    SPH_LANES(SPH_L1)
+#undef SPH_L1
   } else {
-    SPH_LIST(0, g0, b0)
+#define SPH_L0(GG) k_interact_list<0, GG><<<nblk(threads, b0), b0, 0, s>>>(a)
+    SPH_LANES(SPH_L0)
+#undef SPH_L0
   }
-#undef SPH_LIST
+#undef SPH_LANES
 }
 
 void launch_list_begin(int ncases, const CaseConst *cc, CaseDyn *dyn, ListCtl *ctl,
@@ -3113,8 +3234,8 @@ size_t rb_temp_words(int64_t n) { return (size_t)((n + kRbTile - 1) / kRbTile) +
 
 void launch_rebuild_sort(int n, const ListCtl *ctl, const uint32_t *keys, State src, State dst,
                          uint32_t *keys_dst, float *press, const CaseConst *cc, CaseDyn *dyn,
-                         int nbits, const float4 *ref_src, float4 *ref_dst, uint32_t *tmp,
-                         uint32_t *idx, uint32_t *kc, uint32_t *kc_sorted, uint32_t *perm,
+                         int nbits, const float4 *ref_src, float4 *ref_dst, float4 *walk,
+                         uint32_t *tmp, uint32_t *idx, uint32_t *kc, uint32_t *kc_sorted, uint32_t *perm,
                          void *sort_tmp, cudaStream_t s) {
   if (n <= 0) return;
   const int ntiles = (n + kRbTile - 1) / kRbTile;
@@ -3124,7 +3245,7 @@ void launch_rebuild_sort(int n, const ListCtl *ctl, const uint32_t *keys, State 
   k_rb_compact<<<ntiles, kRbTile, 0, s>>>(n, src.cid, dyn, ctl, tmp, keys, idx, kc);
   radix_sort(kc, kc_sorted, perm, n, nbits, sort_tmp, s, m);
   k_rb_scatter<<<nblk(n, 256), 256, 0, s>>>(n, m, idx, perm, kc_sorted, src, dst, keys_dst,
-                                             press, cc, dyn, nbits, ref_src, ref_dst);
+                                             press, cc, dyn, nbits, ref_src, ref_dst, walk);
 }
 
 void launch_need_all(int ncases, CaseDyn *dyn, cudaStream_t s) {
@@ -3136,33 +3257,21 @@ void launch_build_list(int margin, int n, const int *nvalid, const uint32_t *key
                        const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells, int nbits,
                        const CaseConst *cc, CaseDyn *dyn, float4 *ace, uint2 *list, int cap,
                        uint16_t *count, float4 *ref, const float4 *ref_src, cudaStream_t s,
-                       bool half, bool wide) {
+                       bool half) {
   if (n <= 0) return;
   const uint32_t cap1 = (uint32_t)(cap_cells + 1);
-#define SPH_BL_ARGS                                                                        \
-  n, nvalid, keys, posc, velrho, press, cid, cstart, cap1, nbits, cc, dyn, ace, nullptr, 0, \
-      nullptr, nullptr, list, cap, count, ref, ref_src
-#define SPH_BL(L)                                                                \
-  if (margin == 1)                                                               \
-    k_interact<1, 0, 0, L><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);           \
-  else if (margin == 3)                                                          \
-    k_interact<3, 0, 0, L><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);           \
-  else                                                                           \
-    k_interact<2, 0, 0, L><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);
-  if (wide && half) {
-    SPH_BL(7)
-  } else if (wide) {
-    SPH_BL(6)
-  } else if (half) {
-    SPH_BL(3)
-  } else if (margin == 1)
-    k_interact<1, 0, 0, 2><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);
-  else if (margin == 3)
-    k_interact<3, 0, 0, 2><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);
-  else
-    k_interact<2, 0, 0, 2><<<nblk(n, 128), 128, 0, s>>>(SPH_BL_ARGS);
+#define SPH_BL(MM, LL)                                                                        \
+  k_interact<MM, 0, 0, LL><<<nblk(n, 128), 128, 0, s>>>(                                      \
+      n, nvalid, keys, posc, velrho, press, cid, cstart, cap1, nbits, cc, dyn, ace, nullptr, 0, \
+      nullptr, nullptr, list, cap, count, ref, ref_src)
+  if (margin == 1) {
+    if (half) SPH_BL(1, 3); else SPH_BL(1, 2);
+  } else if (margin == 3) {
+    if (half) SPH_BL(3, 3); else SPH_BL(3, 2);
+  } else {
+    if (half) SPH_BL(2, 3); else SPH_BL(2, 2);
+  }
 #undef SPH_BL
-#undef SPH_BL_ARGS
 }
 
 void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t *keys,
@@ -3210,25 +3319,27 @@ void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t 
 void launch_predictor_list(int n, const uint32_t *keys_in, State src, const float4 *ace,
                            const CaseConst *cc, CaseDyn *dyn, int nbits, float4 *posc_out,
                            float4 *velrho_out, uint32_t *keys_out, float *press,
-                           const float4 *ref, cudaStream_t s) {
+                           const float4 *ref, float4 *walk, cudaStream_t s) {
   if (n <= 0) return;
   if (ref)
     k_predictor_list<true><<<nblk(n, 256), 256, 0, s>>>(n, keys_in, src, ace, cc, dyn, nbits,
-                                                        posc_out, velrho_out, keys_out, press, ref);
+                                                        posc_out, velrho_out, keys_out, press, ref,
+                                                        walk);
   else
     k_predictor_list<false><<<nblk(n, 256), 256, 0, s>>>(n, keys_in, src, ace, cc, dyn, nbits,
                                                          posc_out, velrho_out, keys_out, press,
-                                                         ref);
+                                                         ref, walk);
 }
 
 void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_half, State y,
                             const float4 *velrho_half, const float4 *ace, const float4 *ref,
                             const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
-                            uint32_t *keys_next, float *press, ListCtl *ctl, cudaStream_t s) {
+                            uint32_t *keys_next, float *press, ListCtl *ctl, float4 *walk,
+                            cudaStream_t s) {
   if (n > 0)
     k_corrector_reuse<<<nblk(n, 256), 256, 0, s>>>(n, keys_n, keys_half, y, velrho_half, ace,
                                                    ref, cc, dyn, nbits, x, keys_next, press,
-                                                   ctl);
+                                                   ctl, walk);
 }
 
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s) {
@@ -3238,10 +3349,10 @@ void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_
 void launch_list_check(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
                        const uint16_t *cid, const CaseConst *cc, int nbits, const uint2 *list,
                        int cap, const uint16_t *count, ListCtl *ctl, cudaStream_t s, bool half,
-                       const uint32_t *wide_keys) {
+                       const float4 *walk) {
   if (n > 0)
     k_list_check<<<nblk(n, 128), 128, 0, s>>>(n, nvalid, keys, posc, cid, cc, nbits, list, cap,
-                                              count, ctl, half ? 1 : 0, wide_keys);
+                                              count, ctl, half ? 1 : 0, walk);
 }
 
 void launch_corrector_list(int n, const uint32_t *keys_n, const uint32_t *keys_half, State sn,
@@ -3264,10 +3375,10 @@ void launch_verlet(int n, const uint32_t *keys_in, State src, const float4 *ace,
 void launch_verlet_reuse(int n, const uint32_t *keys_in, State y, const float4 *ace,
                          const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
                          uint32_t *keys_out, const float4 *ref, float *press, ListCtl *ctl,
-                         cudaStream_t s) {
+                         float4 *walk, cudaStream_t s) {
   if (n > 0)
     k_verlet<true><<<nblk(n, 256), 256, 0, s>>>(n, keys_in, y, ace, cc, dyn, nbits, x, keys_out,
-                                                ref, press, ctl);
+                                                ref, press, ctl, walk);
 }
 
 void launch_export(int n, const uint32_t *keys, State st, const CaseConst *cc, int slot,
@@ -3330,6 +3441,24 @@ void launch_strain(int margin, int n, const int *nvalid, const uint32_t *keys,
   else
     k_strain<2><<<nblk(n, 128), 128, 0, s>>>(n, nvalid, keys, posc, velrho, cid, cstart, cap1,
                                              nbits, cc, tau4, tau2);
+}
+
+// The walk records of the state in posc, velrho and press (cells of keys).
+__global__ void k_pack_walk(int n, const uint32_t *__restrict__ keys,
+                            const float4 *__restrict__ posc, const float4 *__restrict__ velrho,
+                            const float *__restrict__ press, const uint16_t *__restrict__ cid,
+                            const CaseConst *__restrict__ cc, int nbits,
+                            float4 *__restrict__ walk) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n || keys[i] >= key_out(nbits)) return;
+  put_walk(walk, i, cc[cid[i]], keys[i], nbits, posc[i], velrho[i], press[i]);
+}
+
+void launch_pack_walk(int n, const uint32_t *keys, const float4 *posc, const float4 *velrho,
+                      const float *press, const uint16_t *cid, const CaseConst *cc, int nbits,
+                      float4 *walk, cudaStream_t s) {
+  if (n > 0)
+    k_pack_walk<<<nblk(n, 256), 256, 0, s>>>(n, keys, posc, velrho, press, cid, cc, nbits, walk);
 }
 
 void launch_scatter_tau(int n, const uint16_t *cid, const uint32_t *id, int slot,

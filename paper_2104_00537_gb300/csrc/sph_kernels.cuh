@@ -8,13 +8,14 @@ void launch_upload(int n, const double *pos, const float *vel, const float *rho,
                    const uint8_t *type, const int32_t *group, int slot, uint32_t id_base,
                    const CaseConst *cc, CaseDyn *dyn, int nbits, State st, uint32_t *keys,
                    int dst0, const float *ghost, cudaStream_t s);
-// ref_src / ref_dst (or null): also gather the kept list's build positions.
+// ref_src / ref_dst (or null): also gather the kept list's build positions;
+// walk (or null): also write the list walks' records.
 void launch_reorder(int n, const uint32_t *perm, const uint32_t *keys_sorted,
                     const float4 *posc, const float4 *velrho, const uint32_t *id,
                     const uint16_t *cid, const uint8_t *code, const float4 *vrprev,
                     const float4 *ghost, State dst, float *press, const CaseConst *cc,
                     CaseDyn *dyn, int nbits, cudaStream_t s, const float4 *ref_src = nullptr,
-                    float4 *ref_dst = nullptr);
+                    float4 *ref_dst = nullptr, float4 *walk = nullptr);
 // Words of temporary storage launch_cells needs for cap_cells cells.
 size_t cells_temp_words(int64_t cap_cells);
 // Cell start table of the sorted keys (and nvalid); returns kernels launched.
@@ -40,10 +41,12 @@ void launch_predictor(int n, const uint32_t *keys_in, State src, const float4 *a
                       float4 *velrho_out, uint32_t *keys_out, cudaStream_t s);
 // mDBC boundary values (Eq 38-39) on the sorted state st, before an
 // interaction; stage 0: wall velocity at t, 1: at t + dt/2.  list: st is in
-// the cells of a neighbour list's build (offsets up to skin/2 outside them).
+// the cells of a neighbour list's build (offsets up to skin/2 outside them);
+// walk (or null): also update the list walks' records of the particles set.
 void launch_mdbc(int margin, int n, const int *nvalid, const uint32_t *keys, State st,
                  float *press, const uint32_t *cstart, int nbits, const CaseConst *cc,
-                 const CaseDyn *dyn, int stage, cudaStream_t s, bool list = false);
+                 const CaseDyn *dyn, int stage, cudaStream_t s, bool list = false,
+                 float4 *walk = nullptr);
 // Neighbour list (Symplectic scheme, boundary_mode 0): build on state n
 // with radius 2h + skin; interaction over the list; predictor and corrector
 // that keep the order and the cells of the build.
@@ -67,8 +70,8 @@ void launch_select(int n, const uint16_t *cid, const CaseConst *cc, const CaseDy
 size_t rb_temp_words(int64_t n);
 void launch_rebuild_sort(int n, const ListCtl *ctl, const uint32_t *keys, State src, State dst,
                          uint32_t *keys_dst, float *press, const CaseConst *cc, CaseDyn *dyn,
-                         int nbits, const float4 *ref_src, float4 *ref_dst, uint32_t *tmp,
-                         uint32_t *idx, uint32_t *kc, uint32_t *kc_sorted, uint32_t *perm,
+                         int nbits, const float4 *ref_src, float4 *ref_dst, float4 *walk,
+                         uint32_t *tmp, uint32_t *idx, uint32_t *kc, uint32_t *kc_sorted, uint32_t *perm,
                          void *sort_tmp, cudaStream_t s);
 // Marks every case's kept list for a rebuild.
 void launch_need_all(int ncases, CaseDyn *dyn, cudaStream_t s);
@@ -80,7 +83,7 @@ void launch_build_list(int margin, int n, const int *nvalid, const uint32_t *key
                        const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells, int nbits,
                        const CaseConst *cc, CaseDyn *dyn, float4 *ace, uint2 *list, int cap,
                        uint16_t *count, float4 *ref, const float4 *ref_src, cudaStream_t s,
-                       bool half = false, bool wide = false);
+                       bool half = false);
 // First evaluation of the list step: the compacted pair loop on state n that
 // also writes every target's list (chunk records, radius 2h + skin) and count.
 void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t *keys,
@@ -89,32 +92,37 @@ void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t 
                            int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace,
                            uint2 *list, int cap, uint16_t *count, bool ext, float4 *tau4,
                            float2 *tau2, cudaStream_t s, float *mu = nullptr);
-void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
-                          const float4 *velrho, const float *press, const uint16_t *cid,
-                          const uint32_t *cstart, int64_t cap_cells, int nbits,
-                          const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
+// The interaction over the lists of the state whose records are in walk.
+void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *walk,
+                          const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,
+                          int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
                           float4 *tau4, float2 *tau2, cudaStream_t s, float *mu = nullptr,
-                          int block = 128, int lanes = 1, float4 *sym_sum = nullptr,
-                          unsigned *sym_mu = nullptr, const uint32_t *wide_keys = nullptr);
+                          int block = 0, int lanes = 0, float4 *sym_sum = nullptr,
+                          unsigned *sym_mu = nullptr);
+// The walk records of a state (posc, velrho, press in the cells of keys).
+void launch_pack_walk(int n, const uint32_t *keys, const float4 *posc, const float4 *velrho,
+                      const float *press, const uint16_t *cid, const CaseConst *cc, int nbits,
+                      float4 *walk, cudaStream_t s);
 void launch_predictor_list(int n, const uint32_t *keys_in, State src, const float4 *ace,
                            const CaseConst *cc, CaseDyn *dyn, int nbits, float4 *posc_out,
                            float4 *velrho_out, uint32_t *keys_out, float *press,
-                           const float4 *ref, cudaStream_t s);
+                           const float4 *ref, float4 *walk, cudaStream_t s);
 // Corrector of the list kept across steps: state n+1 to x (normalised, keys)
 // and in place to y (the build's cells, P/rho to press); requests a rebuild
 // through ctl when the next step could leave the skin.
 void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_half, State y,
                             const float4 *velrho_half, const float4 *ace, const float4 *ref,
                             const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
-                            uint32_t *keys_next, float *press, ListCtl *ctl, cudaStream_t s);
+                            uint32_t *keys_next, float *press, ListCtl *ctl, float4 *walk,
+                            cudaStream_t s);
 // One-thread kernel: sets conditional handle h to ctl->rebuild != 0.
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s);
 // Brute-force check of the list against the evaluated state (tests).
 void launch_list_check(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
                        const uint16_t *cid, const CaseConst *cc, int nbits, const uint2 *list,
                        int cap, const uint16_t *count, ListCtl *ctl, cudaStream_t s,
-                       bool half = false, const uint32_t *wide_keys = nullptr);
+                       bool half, const float4 *walk);
 void launch_corrector_list(int n, const uint32_t *keys_n, const uint32_t *keys_half, State sn,
                            const float4 *velrho_half, const float4 *ace, const CaseConst *cc,
                            CaseDyn *dyn, int nbits, State x, uint32_t *keys_next,
@@ -128,7 +136,7 @@ void launch_verlet(int n, const uint32_t *keys_in, State src, const float4 *ace,
 void launch_verlet_reuse(int n, const uint32_t *keys_in, State y, const float4 *ace,
                          const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
                          uint32_t *keys_out, const float4 *ref, float *press, ListCtl *ctl,
-                         cudaStream_t s);
+                         float4 *walk, cudaStream_t s);
 void launch_corrector(int n, const uint32_t *perm2, const uint32_t *keys_half,
                       const uint32_t *keys_n, State sn, State x, const float4 *ace,
                       const CaseConst *cc, CaseDyn *dyn, int nbits, uint32_t *keys_next,

@@ -36,6 +36,13 @@ __device__ __forceinline__ void decode_cell(uint32_t lin, int nx, int ny, int &c
   cy = t - cz * ny;
 }
 
+// 1 / x in one instruction (1 ulp; the pair terms' reciprocals).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 __device__ __forceinline__ float below(float cs) {  // largest float < cs
   return __int_as_float(__float_as_int(cs) - 1);
 }
@@ -535,7 +542,7 @@ __device__ __forceinline__ void pair_fluid(const float4 &va, float Pa, float kv,
   const float t3 = t * t * t;
   const float vx = va.x - vb.x, vy = va.y - vb.y, vz = va.z - vb.z;
   const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
-  const float ib = __fdividef(1.f, vb.w);
+  const float ib = rcp_approx(vb.w);
   const float w = t3 * ib;
   A.s1 = fmaf(w, vr, A.s1);
   if (ddt) {
@@ -544,7 +551,7 @@ __device__ __forceinline__ void pair_fluid(const float4 &va, float Pa, float kv,
     A.s2 = fmaf(w, d, A.s2);
   }
   const float sab = va.w + vb.w;
-  const float ie = __fdividef(1.f, (r2 + eta2) * sab);
+  const float ie = rcp_approx((r2 + eta2) * sab);
   const float mu = vr * ie * sab;  // v_ab.r_ab / (r^2 + eta^2)
   A.mur = fmaxf(A.mur, fabsf(mu));
   const float pi = fminf(vr, 0.f) * ie;
@@ -580,7 +587,7 @@ __device__ __forceinline__ void pair_boundary(const float4 &va, float hih, float
   const float t3 = t * t * t;
   const float vx = va.x - vb.x, vy = va.y - vb.y, vz = va.z - vb.z;
   const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
-  A.s1 = fmaf(t3 * __fdividef(1.f, vb.w), vr, A.s1);
+  A.s1 = fmaf(t3 * rcp_approx(vb.w), vr, A.s1);
 }
 
 // Final values of target a (of density rho_a) from its accumulators: dv/dt
@@ -1372,7 +1379,7 @@ k_strain(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ k
             const float ry = sy - pb.y, rz = sz - pb.z;
             const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
             const float t = fmaf(-hih, r2 * rsqrtf(r2), 1.f);
-            const float w = t * t * t * __fdividef(1.f, vb.w);  // V_b grad W / (m cw r_ab)
+            const float w = t * t * t * rcp_approx(vb.w);  // V_b grad W / (m cw r_ab)
             const float dvx = vb.x - va.x, dvy = vb.y - va.y, dvz = vb.z - va.z;
             gxx = fmaf(w * dvx, rx, gxx);
             gyy = fmaf(w * dvy, ry, gyy);
@@ -1526,7 +1533,7 @@ k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ key
         const float rr2 = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz));
         if (rr2 < r2max) {
           const float4 vb = st.velrho[j];
-          const float ib = __fdividef(1.f, vb.w);
+          const float ib = rcp_approx(vb.w);
           const float t = fmaf(-hih, rr2 * rsqrtf(rr2 + 1e-30f), 1.f);
           const float t3 = t * t * t;
           const float w = C.wk * t3 * t * fmaf(-4.f, t, 5.f);  // W (Eq 11)
@@ -2078,71 +2085,98 @@ k_interact_list(const ListArgs a) {
   const int lane = threadIdx.x & 31;
   const int sub = lane % G;
   constexpr int NG = 32 / G;
+  const unsigned full = 0xffffffffu;
   const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
   const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
   Acc K = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};  // sums of the lane's own target
   unsigned npairs = 0u, nfb = 0u, nbf = 0u;
-  int ccase = -1;  // case of the counts
+  int ccase = -1;  // case of the counts and of the constants below
+  float hih = 0.f, eta2 = 0.f, kvc = 0.f, unit = 0.f, inv_unit = 0.f;
+  unsigned r2max_u = 0u;
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
     const WalkTarget t = walk_target(a, i, nvalid);
     const CaseConst &C = a.cc[t.cidx];
-    const float Pa = t.pa.w * t.va.w;  // the record holds P / rho
-    const float kv = C.kvisc * t.va.w * C.inv_unit;
-    const bool ddt_on = C.ddt != 0;
-    Ext X;
-    X.C = &C;
-    X.unit = C.unit;
-    X.hyd = EXT >= 1 && C.ddt == 2;
-    X.sps = EXT == 2 && C.visc == 1 && t.afluid;
-    X.kl = -4.f * C.nu0 * t.va.w * C.inv_unit;
-    X.tau4 = a.tau4;
-    X.tau2 = a.tau2;
-    {
-      const float4 t4 = X.sps ? a.tau4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float2 t2 = X.sps ? a.tau2[i] : make_float2(0.f, 0.f);
-      X.ta[0] = t.va.w * t4.x;
-      X.ta[1] = t.va.w * t4.y;
-      X.ta[2] = t.va.w * t4.z;
-      X.ta[3] = t.va.w * t4.w;
-      X.ta[4] = t.va.w * t2.x;
-      X.ta[5] = t.va.w * t2.y;
-    }
-    const float hih = C.walk_hih, eta2 = C.walk_eta2;
-    Acc A = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};
-    walk_list<G>(a, i, sub, t.cw, t.pa, __float_as_uint(C.walk_r2max) - 1u,
-                 [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb, int j) {
-                   const bool bfluid = j < jb;
-                   if (t.afluid) {
-                     pair_fluid<EXT>(t.va, Pa, kv, hih, eta2, rx, ry, rz, r2, vb, Qb,
-                                     ddt_on && bfluid, A, &X, j, bfluid);
-                   } else {
-                     pair_boundary(t.va, hih, rx, ry, rz, r2, vb, A);
-                   }
-                   if (bfluid) A.cnt++; else A.cntb++;
-                 });
     if (ccase != t.cidx) {  // the counts so far belong to another case
       if (npairs) atomicAdd(&a.dyn[ccase].pairs, (unsigned long long)npairs);
       if (nfb) atomicAdd(&a.dyn[ccase].pairs_fb, (unsigned long long)nfb);
       if (nbf) atomicAdd(&a.dyn[ccase].pairs_bf, (unsigned long long)nbf);
       npairs = nfb = nbf = 0u;
       ccase = t.cidx;
+      hih = C.walk_hih;
+      eta2 = C.walk_eta2;
+      unit = C.unit;
+      inv_unit = C.inv_unit;
+      kvc = C.kvisc * inv_unit;
+      r2max_u = __float_as_uint(C.walk_r2max) - 1u;
     }
-    npairs += A.cnt + A.cntb;
-    nfb += t.afluid ? A.cntb : 0u;
-    nbf += t.afluid ? 0u : A.cnt;
-    // the sums back from units of cs / 2^29
-    const float ax = group_sum<G>(A.ax), ay = group_sum<G>(A.ay), az = group_sum<G>(A.az);
-    const float s1 = group_sum<G>(A.s1), s2 = group_sum<G>(A.s2), mur = group_max<G>(A.mur);
-    if (sub == q) {
-      K.ax = C.unit * ax;
-      K.ay = C.unit * ay;
-      K.az = C.unit * az;
-      K.s1 = C.unit * s1;
-      K.s2 = s2;
-      K.mur = C.inv_unit * mur;
+    Acc A = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};
+    if (__any_sync(full, t.cw != 0u)) {
+      const float Pa = t.pa.w * t.va.w;  // the record holds P / rho
+      const float kv = kvc * t.va.w;
+      Ext X;
+      if (EXT >= 1) {
+        X.C = &C;
+        X.unit = unit;
+        X.hyd = C.ddt == 2;
+        X.sps = EXT == 2 && C.visc == 1 && t.afluid;
+        X.kl = -4.f * C.nu0 * t.va.w * inv_unit;
+        X.tau4 = a.tau4;
+        X.tau2 = a.tau2;
+        const float4 t4 = X.sps ? a.tau4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float2 t2 = X.sps ? a.tau2[i] : make_float2(0.f, 0.f);
+        X.ta[0] = t.va.w * t4.x;
+        X.ta[1] = t.va.w * t4.y;
+        X.ta[2] = t.va.w * t4.z;
+        X.ta[3] = t.va.w * t4.w;
+        X.ta[4] = t.va.w * t2.x;
+        X.ta[5] = t.va.w * t2.y;
+      }
+      // (no test of the case's diffusion mode: without one kddt is 0)
+      unsigned cnt = 0u, cb = 0u;  // pairs; those with a boundary candidate
+      if (__all_sync(full, t.afluid || t.cw == 0u)) {
+        walk_list<G>(a, i, sub, t.cw, t.pa, r2max_u,
+                     [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb,
+                         int j) {
+                       const bool bfluid = j < jb;
+                       pair_fluid<EXT>(t.va, Pa, kv, hih, eta2, rx, ry, rz, r2, vb, Qb, bfluid,
+                                       A, &X, j, bfluid);
+                       cnt++;
+                       if (!bfluid) cb++;
+                     });
+      } else {
+        walk_list<G>(a, i, sub, t.cw, t.pa, r2max_u,
+                     [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb,
+                         int j) {
+                       const bool bfluid = j < jb;
+                       if (t.afluid)
+                         pair_fluid<EXT>(t.va, Pa, kv, hih, eta2, rx, ry, rz, r2, vb, Qb, bfluid,
+                                         A, &X, j, bfluid);
+                       else
+                         pair_boundary(t.va, hih, rx, ry, rz, r2, vb, A);
+                       cnt++;
+                       if (!bfluid) cb++;
+                     });
+      }
+      npairs += cnt;
+      nfb += t.afluid ? cb : 0u;
+      nbf += t.afluid ? 0u : cnt - cb;
+      A.ax = group_sum<G>(A.ax);
+      A.ay = group_sum<G>(A.ay);
+      A.az = group_sum<G>(A.az);
+      A.s1 = group_sum<G>(A.s1);
+      A.s2 = group_sum<G>(A.s2);
+      A.mur = group_max<G>(A.mur);
+    }
+    if (sub == q) {  // the sums back from units of cs / 2^29
+      K.ax = unit * A.ax;
+      K.ay = unit * A.ay;
+      K.az = unit * A.az;
+      K.s1 = unit * A.s1;
+      K.s2 = A.s2;
+      K.mur = inv_unit * A.mur;
     }
   }
   const int i = first + sub * NG;
@@ -2184,16 +2218,18 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
   const int lane = threadIdx.x & 31;
   const int sub = lane % G;
   constexpr int NG = 32 / G;
+  const unsigned full = 0xffffffffu;
   const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
   const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
   unsigned nall = 0u, nfb = 0u;
-  int ccase = -1;
+  int ccase = -1;  // case of the counts and of the constants below
+  float hih = 0.f, eta2 = 0.f, kvisc = 0.f, kddt = 0.f;
+  unsigned r2max_u = 0u;
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
     const WalkTarget t = walk_target(a, i, nvalid);
-    const CaseConst &C = a.cc[t.cidx];
     if (ccase != t.cidx) {  // the counts so far belong to another case
       if (nall) atomicAdd(&a.dyn[ccase].pairs, 2ull * nall);
       if (nfb) {
@@ -2202,14 +2238,19 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
       }
       nall = nfb = 0u;
       ccase = t.cidx;
+      const CaseConst &C = a.cc[ccase];
+      hih = C.walk_hih;
+      eta2 = C.walk_eta2;
+      kvisc = C.kvisc * C.inv_unit;
+      kddt = C.kddt * C.inv_unit;  // (0 without diffusion)
+      r2max_u = __float_as_uint(C.walk_r2max) - 1u;
     }
-    const float eta2 = C.walk_eta2, hih = C.walk_hih;
-    const float kvisc = C.kvisc * C.inv_unit, kddt = C.kddt * C.inv_unit;
+    const unsigned cw = t.afluid ? t.cw : 0u;
+    if (!__any_sync(full, cw != 0u)) continue;
     const float Qa = t.pa.w;  // P_a / rho_a
-    const float ia = __fdividef(1.f, t.va.w);
-    const bool ddt_on = C.ddt != 0;
+    const float ia = rcp_approx(t.va.w);
     float fx = 0.f, fy = 0.f, fz = 0.f, cont = 0.f, mur = 0.f;
-    walk_list<G>(a, i, sub, t.afluid ? t.cw : 0u, t.pa, __float_as_uint(C.walk_r2max) - 1u,
+    walk_list<G>(a, i, sub, cw, t.pa, r2max_u,
                  [&](float rx, float ry, float rz, float r2, const float4 &vb, float Qb, int j) {
                    const bool bfluid = j < jb;
                    const float rr = r2 * rsqrtf(r2);
@@ -2217,9 +2258,9 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
                    const float t3 = t1 * t1 * t1;
                    const float vx = t.va.x - vb.x, vy = t.va.y - vb.y, vz = t.va.z - vb.z;
                    const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
-                   const float ib = __fdividef(1.f, vb.w);
+                   const float ib = rcp_approx(vb.w);
                    const float sab = t.va.w + vb.w;
-                   const float ie = __fdividef(1.f, (r2 + eta2) * sab);
+                   const float ie = rcp_approx((r2 + eta2) * sab);
                    const float mu = fabsf(vr * ie * sab);
                    mur = fmaxf(mur, mu);
                    const float pi = fminf(vr, 0.f) * ie;
@@ -2228,7 +2269,7 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
                    fy = fmaf(F, ry, fy);
                    fz = fmaf(F, rz, fz);
                    // Eq 17-18 between fluid particles: d = rho_b - rho_a
-                   const float d = (ddt_on && bfluid) ? vb.w - t.va.w : 0.f;
+                   const float d = bfluid ? vb.w - t.va.w : 0.f;
                    cont = fmaf(t3 * ib, fmaf(t.va.w, vr, -kddt * d), cont);
                    // b: -F r_ab (its r_ba = -r_ab), t^3/rho_a (rho_b v.r + kddt d)
                    const float cb = t3 * ia * fmaf(vb.w, vr, kddt * d);
@@ -2244,7 +2285,7 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
     fz = group_sum<G>(fz);
     cont = group_sum<G>(cont);
     mur = group_max<G>(mur);
-    if (sub == 0 && t.afluid) {
+    if (sub == 0 && cw) {
       atomicAdd(&sum[i], make_float4(fx, fy, fz, cont));
       atomicMax(&mu_bits[i], __float_as_uint(mur));
     }
@@ -2406,7 +2447,7 @@ k_strain_list(const ListArgs a, float4 *__restrict__ tau4, float2 *__restrict__ 
     walk_list<G>(a, i, sub, act ? t.cw : 0u, t.pa, __float_as_uint(C.walk_r2max) - 1u,
                  [&](float rx, float ry, float rz, float r2, const float4 &vb, float, int) {
                    const float t1 = fmaf(-hih, r2 * rsqrtf(r2), 1.f);
-                   const float w = t1 * t1 * t1 * __fdividef(1.f, vb.w);
+                   const float w = t1 * t1 * t1 * rcp_approx(vb.w);
                    const float dvx = vb.x - t.va.x, dvy = vb.y - t.va.y, dvz = vb.z - t.va.z;
                    gxx = fmaf(w * dvx, rx, gxx);
                    gyy = fmaf(w * dvy, ry, gyy);

@@ -670,8 +670,8 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
   float4 *tau4 = e->sps ? e->tau4 : nullptr;
   if (e->opt.pi_variant == 5) {
     if (e->mdbc)  // boundary values of Eq 38-39 on state n (the build's cells)
-      launch_mdbc(e->margin, nl, e->nvalid, e->keysB, Y, e->press, e->cstart, e->nbits,
-                  e->dconst, e->ddyn, 0, s, true, e->walk);
+      launch_mdbc_list(nl, e->nvalid, e->keysB, Y, e->press, e->cstart, e->cells_hw, e->nbits,
+                       e->dconst, e->ddyn, 0, e->walk, e->nlist, e->list_cap, e->ncount, s);
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
                          e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
@@ -682,7 +682,8 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
                       s);
     launch_build_list(e->margin, nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid,
                       e->cstart, e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, e->nlist,
-                      e->list_cap, e->ncount, nullptr, nullptr, s, sym_on(e));
+                      e->list_cap, e->ncount, nullptr, nullptr, s, sym_on(e),
+                      e->mdbc ? Y.ghost : nullptr);
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
                          e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
@@ -714,9 +715,15 @@ void enqueue_list_half(sph_engine e, cudaEvent_t *ev, float *mu) {
   launch_predictor_list(nl, e->keysB, Y, e->ace, e->dconst, e->ddyn, e->nbits, Z.posc, Z.velrho,
                         e->keysC, e->press, e->opt.pi_variant == 5 ? e->posc_ref : nullptr, e->walk,
                         s);
-  if (e->mdbc)  // boundary values of Eq 38-39 on state n+1/2 (Y's cells)
-    launch_mdbc(e->margin, nl, e->nvalid, e->keysC, half_state(Y, Z), e->press, e->cstart,
-                e->nbits, e->dconst, e->ddyn, 1, s, true, e->walk);
+  if (e->mdbc) {  // boundary values of Eq 38-39 on state n+1/2 (Y's cells)
+    if (e->opt.pi_variant == 3)  // (its list has no ghost nodes: the cells' rows instead)
+      launch_mdbc(e->margin, nl, e->nvalid, e->keysC, half_state(Y, Z), e->press, e->cstart,
+                  e->nbits, e->dconst, e->ddyn, 1, s, true, e->walk);
+    else
+      launch_mdbc_list(nl, e->nvalid, e->keysC, half_state(Y, Z), e->press, e->cstart,
+                       e->cells_hw, e->nbits, e->dconst, e->ddyn, 1, e->walk, e->nlist,
+                       e->list_cap, e->ncount, s);
+  }
   if (ev) cudaEventRecord(ev[2], s);
   launch_interact_list(nl, e->nvalid, e->keysC, e->walk, Y.cid, e->cstart, e->cells_hw,
                        e->nbits, e->dconst, e->ddyn, e->ace, 0, e->nlist, e->list_cap, e->ncount,
@@ -780,7 +787,8 @@ void enqueue_rebuild_list(sph_engine e, float extra, cudaStream_t q) {
                     q);
   launch_build_list(e->margin, nl, e->nvalid, e->keysB, Y.posc, Y.velrho, e->press, Y.cid,
                     e->cstart, e->cells_hw, e->nbits, e->dconst, e->ddyn, e->ace, e->nlist,
-                    e->list_cap, e->ncount, e->posc_ref, e->posc_ref2, q, sym_on(e));
+                    e->list_cap, e->ncount, e->posc_ref, e->posc_ref2, q, sym_on(e),
+                    e->mdbc ? Y.ghost : nullptr);
 }
 
 // Appends to the graph being captured on e->s a k_decide kernel and an IF

@@ -802,7 +802,8 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
            const float4 *__restrict__ tau4 = nullptr, const float2 *__restrict__ tau2 = nullptr,
            uint2 *__restrict__ list = nullptr, int cap = 0,
            uint16_t *__restrict__ count = nullptr, float4 *__restrict__ ref = nullptr,
-           const float4 *__restrict__ ref_src = nullptr) {
+           const float4 *__restrict__ ref_src = nullptr,
+           const float4 *__restrict__ ghost = nullptr) {
   const unsigned full = 0xffffffffu;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int nvalid = *nvalid_p;
@@ -811,7 +812,7 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
   const CaseConst &C = cc[cidx];
   const uint32_t key = has ? keys[i] : 0u;
   const bool afluid = has && !key_boundary(key, nbits);
-  const int gc = (int)key_cell(key, nbits);
+  int gc = (int)key_cell(key, nbits);
   const int nx = C.nx, nxy = C.nx * C.ny;
   const float cs = C.csf, ics = C.inv_csf, r2max = C.r2max, eta2 = C.eta2, hih = C.half_inv_h;
   // 0 < r2 < r2max as one unsigned compare (r2 >= 0; +0 wraps to UINT_MAX)
@@ -828,16 +829,18 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
   int lcnt = 0;                          // LIST: records written
   const int lmode = (LIST >= 2 && ref) ? (int)dyn[cidx].lmode : 1;
   const float4 *__restrict__ P = lmode == 2 ? ref_src : posc;  // positions walked
-  const float4 pa = has ? P[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 pa = has ? P[i] : make_float4(0.f, 0.f, 0.f, 0.f);
   const float4 va = has ? velrho[i] : make_float4(0.f, 0.f, 0.f, 1.f);
   const float Pa = has ? press[i] * va.w : 0.f;  // press holds P / rho
   const float kv = C.kvisc * va.w;
   const bool ddt_on = C.ddt != 0;
-  // boundary targets of an mDBC case take their density from Eq 38, not Eq 36;
-  // a half list (every boundary index above every fluid one) leaves boundary
-  // targets without candidates
+  // boundary targets of an mDBC case take their density from Eq 38, not Eq 36:
+  // no pairs, but a list built alone (LIST 2, ghost set) holds the fluid around
+  // their ghost node; a half list (every boundary index above every fluid one)
+  // leaves boundary targets without candidates
   constexpr bool HALF = LIST == 3;
-  const bool work = has && (afluid || C.bmode == 0) && lmode != 0 && (!HALF || afluid);
+  const bool node = LIST == 2 && ghost && has && !afluid && C.bmode == 1 && lmode != 0;
+  const bool work = (has && (afluid || C.bmode == 0) && lmode != 0 && (!HALF || afluid)) || node;
   Ext X;
   X.C = &C;
   X.unit = 1.f;
@@ -862,6 +865,17 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
   // the build position: taken now (mode 1), gathered into the new order by
   // the sort (mode 2), or kept where it is (mode 0: the target did not move)
   if (LIST && ref && i < n && lmode != 0) ref[i] = lmode == 1 ? pa : ref_src[i];
+  if (LIST == 2 && node) {  // from here on the target is the ghost node, in its own cell
+    const float4 g = ghost[i];
+    const float qx = pa.x + g.x, qy = pa.y + g.y, qz = pa.z + g.z;
+    const int ux = (int)floorf(qx * ics), uy = (int)floorf(qy * ics), uz = (int)floorf(qz * ics);
+    tcx += ux;
+    tcy += uy;
+    tcz += uz;
+    gc += uz * nxy + uy * nx + ux;
+    pa = make_float4(fmaf(-(float)ux, cs, qx), fmaf(-(float)uy, cs, qy), fmaf(-(float)uz, cs, qz),
+                     (float)tcx);
+  }
   // rows dy, dz in [-M, M]; a list build adds row -(M+1) (M+1) for the
   // targets within the skin of their cell's lower (upper) face, over the
   // warp's union of those ranges
@@ -894,18 +908,21 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
         kx0 = max(kx0, -tcx);
         kx1 = min(kx1, nx - 1 - tcx);
       }
-      const int c0 = gc + dz * nxy + dy * nx + kx0;
-      const int c1 = gc + dz * nxy + dy * nx + kx1 + 1;
-      // half list: the fluid particles of the rows below the target's and of
-      // the cells before its own in its row have smaller indices (cell order)
-      const bool below = HALF && (dz < 0 || (dz == 0 && dy < 0));
-      if (!below) {
-        loF = (int)cstart[HALF && dz == 0 && dy == 0 ? gc + max(kx0, 0) : c0];
-        hiF = (int)cstart[c1];
-      }
-      if (afluid) {
-        loB = (int)cstart[cap1 + c0];
-        hiB = (int)cstart[cap1 + c1];
+      // (a ghost node beside the grid may reach no cell of the row)
+      if (LIST != 2 || kx1 >= kx0) {
+        const int c0 = gc + dz * nxy + dy * nx + kx0;
+        const int c1 = gc + dz * nxy + dy * nx + kx1 + 1;
+        // half list: the fluid particles of the rows below the target's and of
+        // the cells before its own in its row have smaller indices (cell order)
+        const bool below = HALF && (dz < 0 || (dz == 0 && dy < 0));
+        if (!below) {
+          loF = (int)cstart[HALF && dz == 0 && dy == 0 ? gc + max(kx0, 0) : c0];
+          hiF = (int)cstart[c1];
+        }
+        if (afluid) {
+          loB = (int)cstart[cap1 + c0];
+          hiB = (int)cstart[cap1 + c1];
+        }
       }
     }
     const float sy = fmaf(-(float)dy, cs, pa.y), sz = fmaf(-(float)dz, cs, pa.z);
@@ -1447,6 +1464,123 @@ __device__ double solve4(double A[4][4], double b[4], double x[4]) {
 
 constexpr double kMdbcDetMin = 1e-3;  // |det| below: Shepard value, zero gradient
 
+// Moment sums of Eq 38-39 at a ghost node (per unit particle mass): A00 = sum
+// W / rho_b, A0k = sum e_k W / rho_b, Ak0 = sum F d_k / rho_b, Akl = sum F d_k
+// e_l / rho_b (e = -d = r_b - r_G), vs = sum v W / rho_b, and the right-hand
+// side for (rho_G - rho0, grad rho_G): r0 = sum W (rho_b - rho0) / rho_b, rk =
+// sum F d_k (rho_b - rho0) / rho_b.  The same system as for rho_G itself (A
+// (rho0, 0) is rho0 times A's first column), but its right-hand side has no
+// FP32 cancellation of rho0-sized terms.
+struct Moments {
+  float a00 = 0.f, a01 = 0.f, a02 = 0.f, a03 = 0.f, a10 = 0.f, a20 = 0.f, a30 = 0.f;
+  float dxx = 0.f, dyy = 0.f, dzz = 0.f, dxy = 0.f, dxz = 0.f, dyz = 0.f;
+  float r0 = 0.f, r1 = 0.f, r2s = 0.f, r3 = 0.f, vsx = 0.f, vsy = 0.f, vsz = 0.f;
+
+  // d = r_G - r_b (m), rr2 = d . d, vb = {v, rho} of b
+  __device__ __forceinline__ void add(const CaseConst &C, float hih, float ddx, float ddy,
+                                      float ddz, float rr2, const float4 &vb) {
+    const float ib = rcp_approx(vb.w);
+    const float t = fmaf(-hih, rr2 * rsqrtf(rr2 + 1e-30f), 1.f);
+    const float t3 = t * t * t;
+    const float w = C.wk * t3 * t * fmaf(-4.f, t, 5.f);  // W (Eq 11)
+    const float f = C.cw * t3;                            // grad_G W = f d
+    const float wv = w * ib, fv = f * ib;
+    const float dr = (vb.w - C.rho0) * ib;  // (rho_b - rho0) / rho_b
+    a00 += wv;
+    a01 = fmaf(-wv, ddx, a01);
+    a02 = fmaf(-wv, ddy, a02);
+    a03 = fmaf(-wv, ddz, a03);
+    a10 = fmaf(fv, ddx, a10);
+    a20 = fmaf(fv, ddy, a20);
+    a30 = fmaf(fv, ddz, a30);
+    dxx = fmaf(fv * ddx, ddx, dxx);
+    dyy = fmaf(fv * ddy, ddy, dyy);
+    dzz = fmaf(fv * ddz, ddz, dzz);
+    dxy = fmaf(fv * ddx, ddy, dxy);
+    dxz = fmaf(fv * ddx, ddz, dxz);
+    dyz = fmaf(fv * ddy, ddz, dyz);
+    r0 = fmaf(w, dr, r0);
+    r1 = fmaf(f * dr, ddx, r1);
+    r2s = fmaf(f * dr, ddy, r2s);
+    r3 = fmaf(f * dr, ddz, r3);
+    vsx = fmaf(wv, vb.x, vsx);
+    vsy = fmaf(wv, vb.y, vsy);
+    vsz = fmaf(wv, vb.z, vsz);
+  }
+};
+constexpr int kMoments = sizeof(Moments) / sizeof(float);
+
+// Density and velocity of boundary particle i from its ghost node's sums (Eq 38
+// and, with mdbc_slip, Eq 39), written to its state, P/rho and walk record.
+__device__ __forceinline__ void mdbc_value(const CaseConst &C, const CaseDyn *__restrict__ dyn,
+                                           int i, int cidx, const float4 &g, const Moments &S,
+                                           int stage, const State &st, float *__restrict__ press,
+                                           float4 *__restrict__ walk) {
+  // imposed velocity of B at the evaluation time (Eq 37)
+  float vw[3] = {0.f, 0.f, 0.f};
+  const uint8_t code = st.code[i];
+  if (code >= 2) {
+    const int gi = code - 2;
+    const CaseDyn &D = dyn[cidx];
+    const double te = D.t + (stage ? 0.5 * D.dt : 0.0);
+    const float v = (float)(C.mot_amp[gi] * C.mot_omega[gi] *
+                            cos(C.mot_omega[gi] * te + C.mot_phase[gi]));
+    vw[0] = v * C.mot_axis[gi][0];
+    vw[1] = v * C.mot_axis[gi][1];
+    vw[2] = v * C.mot_axis[gi][2];
+  }
+  float4 out = st.velrho[i];
+  if (!(S.a00 > 0.f)) {  // no fluid near the ghost
+    out.w = C.rho0;
+    if (C.mdbc_slip) {
+      out.x = vw[0];
+      out.y = vw[1];
+      out.z = vw[2];
+    }
+  } else {
+    double A[4][4] = {{S.a00, S.a01, S.a02, S.a03},
+                      {S.a10, -S.dxx, -S.dxy, -S.dxz},
+                      {S.a20, -S.dxy, -S.dyy, -S.dyz},
+                      {S.a30, -S.dxz, -S.dyz, -S.dzz}};
+    double b[4] = {S.r0, S.r1, S.r2s, S.r3}, x[4] = {0.0, 0.0, 0.0, 0.0};
+    // the sums are per unit particle mass: the determinant of the moment
+    // matrix with volumes V_b = m / rho_b is m^4 times this one
+    const double m2 = C.m_d * C.m_d;
+    const double det = solve4(A, b, x) * (m2 * m2);
+    const double shep = (double)C.rho0 + (double)S.r0 / (double)S.a00;  // Shepard value
+    double rhoB = shep;
+    if (fabs(det) >= kMdbcDetMin) {
+      // Eq 38 with r_B - r_G = -ghost
+      rhoB = (double)C.rho0 + x[0] - ((double)g.x * x[1] + (double)g.y * x[2] + (double)g.z * x[3]);
+      if (!(rhoB > 0.0 && rhoB < 1e30)) rhoB = shep;  // not a usable density
+    }
+    out.w = (float)rhoB;
+    const float vgx = S.vsx / S.a00, vgy = S.vsy / S.a00, vgz = S.vsz / S.a00;  // Eq 39
+    if (C.mdbc_slip == 1) {
+      out.x = 2.f * vw[0] - vgx;
+      out.y = 2.f * vw[1] - vgy;
+      out.z = 2.f * vw[2] - vgz;
+    } else if (C.mdbc_slip == 2) {
+      const float gn = sqrtf(g.x * g.x + g.y * g.y + g.z * g.z);
+      const float inv = gn > 0.f ? 1.f / gn : 0.f;
+      const float nx_ = g.x * inv, ny_ = g.y * inv, nz_ = g.z * inv;
+      const float vn = vgx * nx_ + vgy * ny_ + vgz * nz_;
+      const float wn = vw[0] * nx_ + vw[1] * ny_ + vw[2] * nz_;
+      const float k2 = 2.f * (wn - vn);
+      out.x = fmaf(k2, nx_, vgx);
+      out.y = fmaf(k2, ny_, vgy);
+      out.z = fmaf(k2, nz_, vgz);
+    }
+  }
+  const float Q = tait_pressure(C, out.w) / out.w;
+  st.velrho[i] = out;
+  press[i] = Q;
+  if (walk) {  // the record of the list walks
+    walk[2 * (int64_t)i].w = Q;
+    walk[2 * (int64_t)i + 1] = out;
+  }
+}
+
 // One thread per particle (sorted order); boundary particles of mDBC cases
 // get their density from the ghost node r_G = r_B + ghost (Eq 38) and, with
 // mdbc_slip, their velocity from the Shepard sum of Eq 39.  The moment sums
@@ -1493,15 +1627,7 @@ k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ key
               oz = fmaf(-(float)sz, cs, qz0);                               // offset in it
   const int nx = C.nx, ny = C.ny, nz = C.nz, nxy = nx * ny;
   const int base0 = (int)C.cellbase;
-  // moment sums (per unit particle mass): A00 = sum W / rho_b, A0k = sum e_k W / rho_b,
-  // Ak0 = sum F d_k / rho_b, Akl = sum F d_k e_l / rho_b (e = -d = r_b - r_G),
-  // vs = sum v W / rho_b, and the right-hand side for (rho_G - rho0, grad rho_G):
-  // r0 = sum W (rho_b - rho0) / rho_b, rk = sum F d_k (rho_b - rho0) / rho_b.  The
-  // same system as for rho_G itself (A (rho0, 0) is rho0 times A's first column),
-  // but its right-hand side has no FP32 cancellation of rho0-sized terms.
-  float a00 = 0.f, a01 = 0.f, a02 = 0.f, a03 = 0.f, a10 = 0.f, a20 = 0.f, a30 = 0.f;
-  float dxx = 0.f, dyy = 0.f, dzz = 0.f, dxy = 0.f, dxz = 0.f, dyz = 0.f;
-  float r0 = 0.f, r1 = 0.f, r2s = 0.f, r3 = 0.f, vsx = 0.f, vsy = 0.f, vsz = 0.f;
+  Moments S;
   constexpr int W = 2 * MR + 1;
 #pragma unroll 1
   for (int row = 0; row < W * W; row++) {
@@ -1532,102 +1658,13 @@ k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ key
         const float ddy = ry0 - pf.y, ddz = rz0 - pf.z;
         const float rr2 = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz));
         if (rr2 < r2max) {
-          const float4 vb = st.velrho[j];
-          const float ib = rcp_approx(vb.w);
-          const float t = fmaf(-hih, rr2 * rsqrtf(rr2 + 1e-30f), 1.f);
-          const float t3 = t * t * t;
-          const float w = C.wk * t3 * t * fmaf(-4.f, t, 5.f);  // W (Eq 11)
-          const float f = C.cw * t3;                            // grad_G W = f d
-          const float wv = w * ib, fv = f * ib;
-          const float dr = (vb.w - C.rho0) * ib;  // (rho_b - rho0) / rho_b
-          a00 += wv;
-          a01 = fmaf(-wv, ddx, a01);
-          a02 = fmaf(-wv, ddy, a02);
-          a03 = fmaf(-wv, ddz, a03);
-          a10 = fmaf(fv, ddx, a10);
-          a20 = fmaf(fv, ddy, a20);
-          a30 = fmaf(fv, ddz, a30);
-          dxx = fmaf(fv * ddx, ddx, dxx);
-          dyy = fmaf(fv * ddy, ddy, dyy);
-          dzz = fmaf(fv * ddz, ddz, dzz);
-          dxy = fmaf(fv * ddx, ddy, dxy);
-          dxz = fmaf(fv * ddx, ddz, dxz);
-          dyz = fmaf(fv * ddy, ddz, dyz);
-          r0 = fmaf(w, dr, r0);
-          r1 = fmaf(f * dr, ddx, r1);
-          r2s = fmaf(f * dr, ddy, r2s);
-          r3 = fmaf(f * dr, ddz, r3);
-          vsx = fmaf(wv, vb.x, vsx);
-          vsy = fmaf(wv, vb.y, vsy);
-          vsz = fmaf(wv, vb.z, vsz);
+          S.add(C, hih, ddx, ddy, ddz, rr2, st.velrho[j]);
         }
       }
     }
   }
   if (!act) return;
-  // imposed velocity of B at the evaluation time (Eq 37)
-  float vw[3] = {0.f, 0.f, 0.f};
-  const uint8_t code = st.code[i];
-  if (code >= 2) {
-    const int gi = code - 2;
-    const CaseDyn &D = dyn[cidx];
-    const double te = D.t + (stage ? 0.5 * D.dt : 0.0);
-    const float v = (float)(C.mot_amp[gi] * C.mot_omega[gi] *
-                            cos(C.mot_omega[gi] * te + C.mot_phase[gi]));
-    vw[0] = v * C.mot_axis[gi][0];
-    vw[1] = v * C.mot_axis[gi][1];
-    vw[2] = v * C.mot_axis[gi][2];
-  }
-  float4 out = st.velrho[i];
-  if (!(a00 > 0.f)) {  // no fluid near the ghost
-    out.w = C.rho0;
-    if (C.mdbc_slip) {
-      out.x = vw[0];
-      out.y = vw[1];
-      out.z = vw[2];
-    }
-  } else {
-    double A[4][4] = {{a00, a01, a02, a03},
-                      {a10, -dxx, -dxy, -dxz},
-                      {a20, -dxy, -dyy, -dyz},
-                      {a30, -dxz, -dyz, -dzz}};
-    double b[4] = {r0, r1, r2s, r3}, x[4] = {0.0, 0.0, 0.0, 0.0};
-    // the sums are per unit particle mass: the determinant of the moment
-    // matrix with volumes V_b = m / rho_b is m^4 times this one
-    const double m2 = C.m_d * C.m_d;
-    const double det = solve4(A, b, x) * (m2 * m2);
-    const double shep = (double)C.rho0 + (double)r0 / (double)a00;  // Shepard value
-    double rhoB = shep;
-    if (fabs(det) >= kMdbcDetMin) {
-      // Eq 38 with r_B - r_G = -ghost
-      rhoB = (double)C.rho0 + x[0] - ((double)g.x * x[1] + (double)g.y * x[2] + (double)g.z * x[3]);
-      if (!(rhoB > 0.0 && rhoB < 1e30)) rhoB = shep;  // not a usable density
-    }
-    out.w = (float)rhoB;
-    const float vgx = vsx / a00, vgy = vsy / a00, vgz = vsz / a00;  // Eq 39
-    if (C.mdbc_slip == 1) {
-      out.x = 2.f * vw[0] - vgx;
-      out.y = 2.f * vw[1] - vgy;
-      out.z = 2.f * vw[2] - vgz;
-    } else if (C.mdbc_slip == 2) {
-      const float gn = sqrtf(g.x * g.x + g.y * g.y + g.z * g.z);
-      const float inv = gn > 0.f ? 1.f / gn : 0.f;
-      const float nx_ = g.x * inv, ny_ = g.y * inv, nz_ = g.z * inv;
-      const float vn = vgx * nx_ + vgy * ny_ + vgz * nz_;
-      const float wn = vw[0] * nx_ + vw[1] * ny_ + vw[2] * nz_;
-      const float k2 = 2.f * (wn - vn);
-      out.x = fmaf(k2, nx_, vgx);
-      out.y = fmaf(k2, ny_, vgy);
-      out.z = fmaf(k2, nz_, vgz);
-    }
-  }
-  const float Q = tait_pressure(C, out.w) / out.w;
-  st.velrho[i] = out;
-  press[i] = Q;
-  if (walk) {  // the record of the list walks
-    walk[2 * (int64_t)i].w = Q;
-    walk[2 * (int64_t)i + 1] = out;
-  }
+  mdbc_value(C, dyn, i, cidx, g, S, stage, st, press, walk);
 }
 
 // ---- time step and motion ----------------------------------------------------
@@ -2097,8 +2134,10 @@ k_interact_list(const ListArgs a) {
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
-    const WalkTarget t = walk_target(a, i, nvalid);
+    WalkTarget t = walk_target(a, i, nvalid);
     const CaseConst &C = a.cc[t.cidx];
+    // (the list of an mDBC boundary particle is its ghost node's)
+    if (!t.afluid && C.bmode == 1) t.cw = 0u;
     if (ccase != t.cidx) {  // the counts so far belong to another case
       if (npairs) atomicAdd(&a.dyn[ccase].pairs, (unsigned long long)npairs);
       if (nfb) atomicAdd(&a.dyn[ccase].pairs_fb, (unsigned long long)nfb);
@@ -2471,6 +2510,83 @@ k_strain_list(const ListArgs a, float4 *__restrict__ tau4, float2 *__restrict__ 
       sps_tau_from_gradient(C, gxx, gyy, gzz, gxy, gxz, gyz, tau4[i], tau2[i]);
     }
   }
+}
+
+// The mDBC boundary values (as k_mdbc) over the ghost nodes' lists, which the
+// list build wrote into the boundary particles' segments: no search of rows and
+// cells, only the fluid within 2h + skin of the node.  G lanes share a node and
+// take neighbouring list entries; a block's 256 / G nodes then leave their sums
+// in shared memory, and one thread each solves the 4x4 systems, so that the
+// FP64 elimination runs on full warps.
+template <int G>
+__global__ void __launch_bounds__(256)
+k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ keys, State st,
+            float *__restrict__ press, const uint32_t *__restrict__ cstart, uint32_t cap1,
+            int nbits, const CaseConst *__restrict__ cc, const CaseDyn *__restrict__ dyn,
+            int stage, float4 *__restrict__ walk, const uint2 *__restrict__ list, int cap,
+            const uint16_t *__restrict__ count) {
+  constexpr int NB = 256 / G;  // nodes per block
+  __shared__ float s_m[kMoments][NB + 1];
+  const int first = (int)cstart[cap1 - 1] + blockIdx.x * NB;  // boundary particles are last
+  const int nvalid = *nvalid_p;
+  if (first >= nvalid) return;
+  const int sub = threadIdx.x % G, node = threadIdx.x / G;
+  const int i = first + node;
+  const uint32_t key = i < nvalid ? keys[i] : key_out(nbits);
+  const int cidx = i < nvalid ? (int)st.cid[i] : 0;
+  const CaseConst &C = cc[cidx];
+  const bool act = key < key_out(nbits) && C.bmode == 1;
+  Moments S;
+  if (act) {
+    // the node's position in walk coordinates
+    const float4 pb = walk[2 * (int64_t)i], g = st.ghost[i];
+    auto coord = [&](float p, float d) {  // (whole cells first: d may exceed 4 of them)
+      const float u = floorf(d * C.inv_csf);
+      return (int)((unsigned)__float_as_int(p) + (unsigned)walk_coord(C, (int)u, fmaf(-u, C.csf, d)));
+    };
+    const int qx = coord(pb.x, g.x), qy = coord(pb.y, g.y), qz = coord(pb.z, g.z);
+    const float unit = C.unit, r2max = C.r2max, hih = C.half_inv_h;
+    auto visit = [&](int j) {
+      float4 p, b;
+      load_walk(walk, j, p, b);
+      const float dx = unit * (float)(qx - __float_as_int(p.x));
+      const float dy = unit * (float)(qy - __float_as_int(p.y));
+      const float dz = unit * (float)(qz - __float_as_int(p.z));
+      const float rr2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      if (rr2 < r2max && b.w > 0.f) S.add(C, hih, dx, dy, dz, rr2, b);
+    };
+    const unsigned cw = count[i];
+    const uint2 *__restrict__ seg = list + (int64_t)i * cap;
+    if (cw & kListRecords) {
+      for (int r = 0; r < (int)(cw & ~kListRecords); r++) {
+        const uint2 q = seg[r];
+        for (int k = sub; k < 32; k += G)
+          if ((q.y >> k) & 1u) visit((int)q.x + k);
+      }
+    } else {
+      const uint32_t *__restrict__ mine = reinterpret_cast<const uint32_t *>(seg);
+#pragma unroll 2
+      for (int k = sub; k < (int)cw; k += G) visit((int)mine[k]);
+    }
+  }
+  __syncwarp();
+  float *m = reinterpret_cast<float *>(&S);
+#pragma unroll
+  for (int q = 0; q < kMoments; q++) {
+    const float v = group_sum<G>(m[q]);
+    if (sub == 0) s_m[q][node] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x >= NB) return;
+  const int i2 = first + threadIdx.x;
+  if (i2 >= nvalid || keys[i2] >= key_out(nbits)) return;
+  const int c2 = (int)st.cid[i2];
+  if (cc[c2].bmode != 1) return;
+  Moments R;
+  float *r = reinterpret_cast<float *>(&R);
+#pragma unroll
+  for (int q = 0; q < kMoments; q++) r[q] = s_m[q][threadIdx.x];
+  mdbc_value(cc[c2], dyn, i2, c2, st.ghost[i2], R, stage, st, press, walk);
 }
 
 // Half step for the list path: state n+1/2 in the same order and the same
@@ -3207,6 +3323,16 @@ static inline int walk_targets(int n, int G) {
   return per;
 }
 
+void launch_mdbc_list(int n, const int *nvalid, const uint32_t *keys, State st, float *press,
+                      const uint32_t *cstart, int64_t cap_cells, int nbits, const CaseConst *cc,
+                      const CaseDyn *dyn, int stage, float4 *walk, const uint2 *list, int cap,
+                      const uint16_t *count, cudaStream_t s) {
+  if (n > 0)
+    k_mdbc_list<8><<<nblk(n, 32), 256, 0, s>>>(n, nvalid, keys, st, press, cstart,
+                                               (uint32_t)(cap_cells + 1), nbits, cc, dyn, stage,
+                                               walk, list, cap, count);
+}
+
 void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *walk,
                           const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,
                           int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
@@ -3298,13 +3424,13 @@ void launch_build_list(int margin, int n, const int *nvalid, const uint32_t *key
                        const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells, int nbits,
                        const CaseConst *cc, CaseDyn *dyn, float4 *ace, uint2 *list, int cap,
                        uint16_t *count, float4 *ref, const float4 *ref_src, cudaStream_t s,
-                       bool half) {
+                       bool half, const float4 *ghost) {
   if (n <= 0) return;
   const uint32_t cap1 = (uint32_t)(cap_cells + 1);
 #define SPH_BL(MM, LL)                                                                        \
   k_interact<MM, 0, 0, LL><<<nblk(n, 128), 128, 0, s>>>(                                      \
       n, nvalid, keys, posc, velrho, press, cid, cstart, cap1, nbits, cc, dyn, ace, nullptr, 0, \
-      nullptr, nullptr, list, cap, count, ref, ref_src)
+      nullptr, nullptr, list, cap, count, ref, ref_src, ghost)
   if (margin == 1) {
     if (half) SPH_BL(1, 3); else SPH_BL(1, 2);
   } else if (margin == 3) {

@@ -83,7 +83,13 @@ void launch_build_list(int margin, int n, const int *nvalid, const uint32_t *key
                        const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells, int nbits,
                        const CaseConst *cc, CaseDyn *dyn, float4 *ace, uint2 *list, int cap,
                        uint16_t *count, float4 *ref, const float4 *ref_src, cudaStream_t s,
-                       bool half = false);
+                       bool half = false, const float4 *ghost = nullptr);
+// mDBC boundary values over the lists a build with ghost set wrote (the
+// boundary particles' ghost offsets: their lists are their ghost nodes').
+void launch_mdbc_list(int n, const int *nvalid, const uint32_t *keys, State st, float *press,
+                      const uint32_t *cstart, int64_t cap_cells, int nbits, const CaseConst *cc,
+                      const CaseDyn *dyn, int stage, float4 *walk, const uint2 *list, int cap,
+                      const uint16_t *count, cudaStream_t s);
 // First evaluation of the list step: the compacted pair loop on state n that
 // also writes every target's list (chunk records, radius 2h + skin) and count.
 void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t *keys,

@@ -47,3 +47,28 @@ def test_targets_per_group(dp):
     eng.step(2)
     check_step_eval(case, eng, 0, exact_pairs=False)
     eng.destroy()
+
+
+@pytest.mark.parametrize("cell_mode", [0, 1, 2])
+@pytest.mark.parametrize("slip", [0, 2])
+def test_ghost_node_lists(cell_mode, slip):
+    """mDBC boundary values from the ghost nodes' lists (variant 5) against the
+    search of the cells' rows (variant 0), 20 steps of a moving tank.  Ghost
+    offsets reach seven cells at cell_mode 2 (the lists' positions wrap at
+    eight).  The sums are the same up to FP32 rounding (about 1e-6, times ten
+    for the extrapolation to the wall); a missed neighbour shows at 1e-2."""
+    c = cases.sloshing_tank(3000, 0.3, 0.03, 1.2, boundary_mode=1, mdbc_slip=slip,
+                            cell_mode=cell_mode)
+    out = []
+    for variant in (5, 0):
+        eng = sph.Engine.create(c)
+        eng.set_options(pi_variant=variant)
+        eng.step(20)
+        out.append(eng.get_state())
+        eng.destroy()
+    a, b = out
+    b_ = c.ptype != 0
+    d = np.abs(a["rho"][b_] - b["rho"][b_]).max()
+    assert d < 1e-3 * np.abs(b["rho"] - c.params["rho0"]).max(), d
+    assert np.abs(a["vel"] - b["vel"]).max() < 1e-3 * np.abs(b["vel"]).max()
+    assert np.abs(a["pos"] - b["pos"]).max() < 1e-3 * c.params["dp"]

@@ -675,7 +675,8 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
                          e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
-                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
+                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
+                         e->cap_cases == 1);
   } else if (e->opt.pi_variant == 4) {  // list alone, then both evaluations over it
     if (ev) cudaEventRecord(ev[0], s);  // the first evaluation's time includes the list
     launch_list_begin(e->cap_cases, e->dconst, e->ddyn, e->ctl, 0.f, 1, e->cstart, e->cells_hw,
@@ -687,7 +688,8 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
                          e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
-                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
+                         e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
+                         e->cap_cases == 1);
   } else {
     launch_list_begin(e->cap_cases, e->dconst, e->ddyn, e->ctl, 0.f, 1, e->cstart, e->cells_hw,
                       s);
@@ -728,7 +730,8 @@ void enqueue_list_half(sph_engine e, cudaEvent_t *ev, float *mu) {
   launch_interact_list(nl, e->nvalid, e->keysC, e->walk, Y.cid, e->cstart, e->cells_hw,
                        e->nbits, e->dconst, e->ddyn, e->ace, 0, e->nlist, e->list_cap, e->ncount,
                        e->ext, e->sps ? e->tau4 : nullptr, e->tau2, s, mu, e->opt.pi_block,
-                       e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu);
+                       e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
+                         e->cap_cases == 1);
   if (ev) cudaEventRecord(ev[3], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysC, Z.posc, Y.cid, e->dconst, e->nbits, e->nlist,

@@ -703,13 +703,26 @@ __global__ void k_need_all(int ncases, CaseDyn *__restrict__ dyn) {
 
 // Turns the records (first index, mask) that each lane of the warp wrote for
 // its target into the target's flat list: the candidate indices in record
-// order, 32 bits each, in the same segment (2 cap of them).  The warp takes
-// its 32 targets one by one: the records go to registers, then each record's
+// order, 32 bits each, in the same segment (2 cap of them), padded with the target
+// itself to a multiple of 16.  In a block of 16 entries the e-th candidate sits at
+// flat_slot(e), so that of eight lanes that read two entries side by side (one
+// 64-bit load) each takes candidates e and e + 8, and a warp's gathers go to
+// neighbouring records (walk of 1.48M particles 527 us; 544 with two 32-bit index
+// loads, 631 with candidates e and e + 1).  The warp takes its 32 targets one by one: the records go to registers, then each record's
 // candidates are written side by side by the lanes whose bit is set.  A target
 // whose candidates do not fit, or with more than 128 records, keeps its records
 // (kListRecords in its count).  Cost: about 11 warp-instructions per record,
 // paid once per build, against a list walk without masks, rows or bit scans.
 constexpr int kFlatRounds = 4;  // of 32 records
+__device__ __forceinline__ int flat_slot(int e) {
+  return (e & ~15) | ((e << 1) & 14) | ((e >> 3) & 1);
+}
+// *p = v where on, as one predicated store: a branch around it would keep the
+// unrolled candidates' arithmetic from overlapping.
+__device__ __forceinline__ void store_if(bool on, uint32_t *p, uint32_t v) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.global.u32 [%0], %1;\n}"
+               :: "l"(p), "r"(v), "r"((unsigned)on) : "memory");
+}
 __device__ __forceinline__ void flatten_records(int i, bool build, int nrec,
                                                 uint2 *__restrict__ list, int cap,
                                                 uint16_t *__restrict__ count) {
@@ -742,22 +755,32 @@ __device__ __forceinline__ void flatten_records(int i, bool build, int nrec,
       off[h] = total + x - c;
       total += __shfl_sync(full, x, 31);
     }
-    const bool flat = nr <= 32 * kFlatRounds && total <= 2 * cap;
-    if (lane == t) mine = flat ? total : (int)kListRecords | nr;
+    const int n16 = (total + 15) & ~15;
+    const bool flat = nr <= 32 * kFlatRounds && n16 <= 2 * cap;
+    if (lane == t) mine = flat ? n16 : (int)kListRecords | nr;
     if (!flat) continue;
     __syncwarp();  // every record is in registers before its memory is overwritten
     uint32_t *dst = reinterpret_cast<uint32_t *>(rec);
 #pragma unroll
     for (int h = 0; h < kFlatRounds; h++) {
       const int m = min(32, nr - 32 * h);
-#pragma unroll 4
-      for (int q = 0; q < m; q++) {
-        const uint32_t b = __shfl_sync(full, r[h].x, q);
-        const unsigned mask = __shfl_sync(full, r[h].y, q);
-        const int o = __shfl_sync(full, off[h], q);
-        if ((mask >> lane) & 1u) dst[o + __popc(mask & lt)] = b + (uint32_t)lane;
+      for (int q = 0; q < m; q += 4) {  // (records past the last are empty)
+        uint32_t b[4];
+        unsigned mask[4];
+        int o[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          b[u] = __shfl_sync(full, r[h].x, q + u);
+          mask[u] = __shfl_sync(full, r[h].y, q + u);
+          o[u] = __shfl_sync(full, off[h], q + u);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+          store_if((mask[u] >> lane) & 1u, dst + flat_slot(o[u] + __popc(mask[u] & lt)),
+                   b[u] + (uint32_t)lane);
       }
     }
+    if (lane < n16 - total) dst[flat_slot(total + lane)] = (uint32_t)(i - lane + t);
   }
   if (build) count[i] = (uint16_t)mine;
 }
@@ -1929,6 +1952,7 @@ struct ListArgs {
   const float4 *tau4;
   const float2 *tau2;
   float *mu_out;
+  int one_case;  // the engine has one case slot: every target is of case 0
   int per;  // targets that a group of G lanes takes one after another (<= G)
 };
 
@@ -1944,6 +1968,10 @@ __device__ __forceinline__ float walk_r2(const float4 &a, const float4 &b, float
   return fmaf(rx, rx, fmaf(ry, ry, rz * rz));
 }
 
+// Density in the record of a particle that left the domain at the half step: it
+// is still in the lists, but in no pair.
+constexpr float kGone = -INFINITY;
+
 // One 32-byte walk record in one 256-bit load.
 __device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j, float4 &p,
                                           float4 &b) {
@@ -1953,13 +1981,19 @@ __device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j
 }
 
 // The candidates of target i (all 32 lanes of the warp call it together, G
-// lanes with the same i; sub: the lane's rank among them).  Lane sub takes the
-// list entries sub, sub + G, ..., so the lanes of a target read neighbouring
-// entries and, the list being in cell order, mostly neighbouring candidates;
-// two candidates per iteration with their loads issued together, the next two
-// indices loaded ahead.  body(rx, ry, rz, r2, b, j) runs for every candidate
+// lanes with the same i; sub: the lane's rank among them).  In every iteration
+// lane sub takes two of the next 2 G entries (side by side in the list, one 64-bit
+// load an iteration ahead; see flatten_records) and gathers both records before it uses either: the lanes of
+// a target read neighbouring entries and, the list being in cell order, mostly
+// neighbouring records.  body(rx, ry, rz, r2, b, Qb, j) runs for every candidate
 // inside the support; positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
 // A lane without an entry takes the target itself (r2 = 0: no pair).
+// What bounds it (1.48M particles, 530 us): L1 gathers (data pipe 78 % of its
+// peak) and issue (68 %) together.  Measured and left out, per evaluation: records
+// double-buffered in registers 608 us, one candidate per iteration 634, no branch
+// around the pair terms 588 (against 562), targets taken by bricks of cells 535
+// (L1 hits 52 -> 72 %, same time), list entries dealt to lanes by index modulo 8,
+// free of bank conflicts, 541 but a build of 1.42 instead of 1.08 ms.
 template <int G, class Body>
 __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const int sub,
                                           const unsigned cw, const float4 &pa,
@@ -1969,25 +2003,24 @@ __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const 
   const bool rec = (cw & kListRecords) != 0u;
   const int cnt = rec ? 0 : (int)cw;
   const int kmax = (int)__reduce_max_sync(full, (unsigned)cnt);
-  const uint32_t *__restrict__ mine =
-      reinterpret_cast<const uint32_t *>(a.list + (int64_t)i * a.cap);
-  int j1 = sub < cnt ? (int)mine[sub] : i;
-  int j2 = sub + G < cnt ? (int)mine[sub + G] : i;
+  // (a list's length is a multiple of 16: both entries of a lane exist or none)
+  const uint2 *__restrict__ mine = a.list + (int64_t)i * a.cap + sub;
+  const uint2 none = make_uint2((unsigned)i, (unsigned)i);
+  uint2 j = cnt > 0 ? *mine : none;
 #pragma unroll 1
-  for (int k = sub; k - sub < kmax; k += 2 * G) {
+  for (int k = 2 * G; k - 2 * G < kmax; k += 2 * G) {
     float4 p1, b1, p2, b2;
-    load_walk(walk, j1, p1, b1);
-    load_walk(walk, j2, p2, b2);
-    const int i1 = j1, i2 = j2;
-    j1 = k + 2 * G < cnt ? (int)mine[k + 2 * G] : i;
-    j2 = k + 3 * G < cnt ? (int)mine[k + 3 * G] : i;
+    load_walk(walk, (int)j.x, p1, b1);
+    load_walk(walk, (int)j.y, p2, b2);
+    const int i1 = (int)j.x, i2 = (int)j.y;
+    mine += G;
+    j = k < cnt ? *mine : none;
 #pragma unroll
     for (int u = 0; u < 2; u++) {
       float rx, ry, rz;
       const float r2 = walk_r2(pa, u ? p2 : p1, rx, ry, rz);
       const float4 &b = u ? b2 : b1;
-      // (a particle that left at the half step has no density)
-      if (__float_as_uint(r2) - 1u < r2max_u && b.w > 0.f)
+      if (__float_as_uint(r2) - 1u < r2max_u && b.w != kGone)
         body(rx, ry, rz, r2, b, u ? p2.w : p1.w, u ? i2 : i1);
     }
   }
@@ -2004,7 +2037,7 @@ __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const 
         const float4 p = walk[2 * (int64_t)j], b = walk[2 * (int64_t)j + 1];
         float rx, ry, rz;
         const float r2 = walk_r2(pa, p, rx, ry, rz);
-        if (__float_as_uint(r2) - 1u < r2max_u && b.w > 0.f) body(rx, ry, rz, r2, b, p.w, j);
+        if (__float_as_uint(r2) - 1u < r2max_u && b.w != kGone) body(rx, ry, rz, r2, b, p.w, j);
       }
     }
     __syncwarp();
@@ -2097,15 +2130,14 @@ struct WalkTarget {
   unsigned cw;  // count word of its list (0: nothing to walk)
   float4 pa, va;
 };
-__device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int nvalid) {
+__device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int nvalid,
+                                                  int jb) {
   WalkTarget t;
-  const uint32_t key = i < nvalid ? a.keys[i] : key_out(a.nbits);
-  t.has = key < key_out(a.nbits);  // not frozen at this state
-  t.afluid = t.has && !key_boundary(key, a.nbits);
-  t.cidx = i < a.n ? (int)a.cid[i] : 0;
+  load_walk(a.walk, i, t.pa, t.va);  // (readable past the last particle)
+  t.has = i < nvalid && t.va.w != kGone;
+  t.afluid = t.has && i < jb;
+  t.cidx = a.one_case || i >= a.n ? 0 : (int)a.cid[i];
   t.cw = t.has ? (unsigned)a.count[i] : 0u;
-  t.pa = a.walk[2 * (int64_t)i];  // (readable past the last particle)
-  t.va = t.has ? a.walk[2 * (int64_t)i + 1] : make_float4(0.f, 0.f, 0.f, 1.f);
   return t;
 }
 
@@ -2117,7 +2149,7 @@ __device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int 
 // consecutive targets), then lane q of the group finishes its q-th target, so
 // that the closing arithmetic runs on as many lanes as there are targets.
 template <int EXT, int G>
-__global__ void __launch_bounds__(EXT == 0 ? 1024 : 256, EXT == 0 ? 1 : 0)
+__global__ void __launch_bounds__(256, EXT == 0 ? 4 : 0)
 k_interact_list(const ListArgs a) {
   const int lane = threadIdx.x & 31;
   const int sub = lane % G;
@@ -2126,15 +2158,15 @@ k_interact_list(const ListArgs a) {
   const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
   const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
-  Acc K = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};  // sums of the lane's own target
+  __shared__ float s_k[8][32][6];  // the targets' sums, by the lane that finishes them
   unsigned npairs = 0u, nfb = 0u, nbf = 0u;
   int ccase = -1;  // case of the counts and of the constants below
-  float hih = 0.f, eta2 = 0.f, kvc = 0.f, unit = 0.f, inv_unit = 0.f;
+  float hih = 0.f, eta2 = 0.f, kvc = 0.f;
   unsigned r2max_u = 0u;
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
-    WalkTarget t = walk_target(a, i, nvalid);
+    WalkTarget t = walk_target(a, i, nvalid, jb);
     const CaseConst &C = a.cc[t.cidx];
     // (the list of an mDBC boundary particle is its ghost node's)
     if (!t.afluid && C.bmode == 1) t.cw = 0u;
@@ -2146,9 +2178,7 @@ k_interact_list(const ListArgs a) {
       ccase = t.cidx;
       hih = C.walk_hih;
       eta2 = C.walk_eta2;
-      unit = C.unit;
-      inv_unit = C.inv_unit;
-      kvc = C.kvisc * inv_unit;
+      kvc = C.kvisc * C.inv_unit;
       r2max_u = __float_as_uint(C.walk_r2max) - 1u;
     }
     Acc A = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u};
@@ -2158,10 +2188,10 @@ k_interact_list(const ListArgs a) {
       Ext X;
       if (EXT >= 1) {
         X.C = &C;
-        X.unit = unit;
+        X.unit = C.unit;
         X.hyd = C.ddt == 2;
         X.sps = EXT == 2 && C.visc == 1 && t.afluid;
-        X.kl = -4.f * C.nu0 * t.va.w * inv_unit;
+        X.kl = -4.f * C.nu0 * t.va.w * C.inv_unit;
         X.tau4 = a.tau4;
         X.tau2 = a.tau2;
         const float4 t4 = X.sps ? a.tau4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2209,24 +2239,30 @@ k_interact_list(const ListArgs a) {
       A.s2 = group_sum<G>(A.s2);
       A.mur = group_max<G>(A.mur);
     }
-    if (sub == q) {  // the sums back from units of cs / 2^29
-      K.ax = unit * A.ax;
-      K.ay = unit * A.ay;
-      K.az = unit * A.az;
-      K.s1 = unit * A.s1;
-      K.s2 = A.s2;
-      K.mur = inv_unit * A.mur;
+    if (sub == 0) {
+      float *k = s_k[threadIdx.x >> 5][(lane & ~(G - 1)) + q];
+      k[0] = A.ax;
+      k[1] = A.ay;
+      k[2] = A.az;
+      k[3] = A.s1;
+      k[4] = A.s2;
+      k[5] = A.mur;
     }
   }
+  __syncwarp();
   const int i = first + sub * NG;
-  const bool own = sub < a.per && i < nvalid && a.keys[i] < key_out(a.nbits);
+  const float rho = sub < a.per && i < nvalid ? a.walk[2 * (int64_t)i + 1].w : kGone;
+  const bool own = rho != kGone;
   unsigned dtbits = kFloatInfBits;
   bool bad = false;
   int cidx = ccase;
   if (own) {
-    cidx = (int)a.cid[i];
-    finish_values(a.cc[cidx], i, !key_boundary(a.keys[i], a.nbits), a.walk[2 * (int64_t)i + 1].w,
-                  K, a.want_dt, a.ace, a.mu_out, dtbits, bad);
+    cidx = a.one_case ? 0 : (int)a.cid[i];
+    const float *k = s_k[threadIdx.x >> 5][lane];
+    const float unit = a.cc[cidx].unit;  // the sums back from units of cs / 2^29
+    const Acc K = {unit * k[0], unit * k[1], unit * k[2], unit * k[3], k[4],
+                   a.cc[cidx].inv_unit * k[5], 0u, 0u};
+    finish_values(a.cc[cidx], i, i < jb, rho, K, a.want_dt, a.ace, a.mu_out, dtbits, bad);
     if (cidx != ccase) {  // the lane's counts and its own target differ in case
       if (dtbits < kFloatInfBits) atomicMin(&a.dyn[cidx].dtmin_bits, dtbits);
       if (bad) atomicOr(&a.dyn[cidx].flags, kFlagNaN);
@@ -2268,7 +2304,7 @@ k_interact_sym(const ListArgs a, float4 *__restrict__ sum, unsigned *__restrict_
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
-    const WalkTarget t = walk_target(a, i, nvalid);
+    const WalkTarget t = walk_target(a, i, nvalid, jb);
     if (ccase != t.cidx) {  // the counts so far belong to another case
       if (nall) atomicAdd(&a.dyn[ccase].pairs, 2ull * nall);
       if (nfb) {
@@ -2475,10 +2511,11 @@ k_strain_list(const ListArgs a, float4 *__restrict__ tau4, float2 *__restrict__ 
   constexpr int NG = 32 / G;
   const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
+  const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
 #pragma unroll 1
   for (int q = 0; q < a.per; q++) {
     const int i = first + q * NG;
-    const WalkTarget t = walk_target(a, i, nvalid);
+    const WalkTarget t = walk_target(a, i, nvalid, jb);
     const CaseConst &C = a.cc[t.cidx];
     const bool act = t.afluid && C.visc == 1;
     const float hih = C.walk_hih;
@@ -2553,7 +2590,7 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
       const float dy = unit * (float)(qy - __float_as_int(p.y));
       const float dz = unit * (float)(qz - __float_as_int(p.z));
       const float rr2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      if (rr2 < r2max && b.w > 0.f) S.add(C, hih, dx, dy, dz, rr2, b);
+      if (rr2 < r2max && b.w != kGone) S.add(C, hih, dx, dy, dz, rr2, b);
     };
     const unsigned cw = count[i];
     const uint2 *__restrict__ seg = list + (int64_t)i * cap;
@@ -2564,9 +2601,13 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
           if ((q.y >> k) & 1u) visit((int)q.x + k);
       }
     } else {
-      const uint32_t *__restrict__ mine = reinterpret_cast<const uint32_t *>(seg);
-#pragma unroll 2
-      for (int k = sub; k < (int)cw; k += G) visit((int)mine[k]);
+      const uint2 *__restrict__ mine = seg + sub;
+      // (two entries per lane and iteration, as the walks; i: the list's padding)
+      for (int k = 0; k < (int)cw; k += 2 * G) {
+        const uint2 j = mine[k >> 1];
+        if ((int)j.x != i) visit((int)j.x);
+        if ((int)j.y != i) visit((int)j.y);
+      }
     }
   }
   __syncwarp();
@@ -2638,7 +2679,7 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
     posc_out[i] = make_float4(1e30f, 1e30f, 1e30f, p.w);
     velrho_out[i] = v;
     keys_out[i] = key_out(nbits);
-    walk[2 * (int64_t)i + 1] = make_float4(0.f, 0.f, 0.f, -1.f);  // no density: in no pair
+    walk[2 * (int64_t)i + 1] = make_float4(0.f, 0.f, 0.f, kGone);  // in no pair
     atomicAdd(&dyn[cidx].n_out, 1);
     return;
   }
@@ -2814,7 +2855,7 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
   auto inside = [&](int j) {
     float rx, ry, rz;
     const float r2 = walk_r2(wa, walk[2 * (int64_t)j], rx, ry, rz);
-    return __float_as_uint(r2) - 1u < r2max_u && walk[2 * (int64_t)j + 1].w > 0.f;
+    return __float_as_uint(r2) - 1u < r2max_u && walk[2 * (int64_t)j + 1].w != kGone;
   };
   for (int j = 0; j < nvalid; j++) {
     const uint32_t kj = keys[j];
@@ -3338,15 +3379,15 @@ void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const 
                           int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
                           float4 *tau4, float2 *tau2, cudaStream_t s, float *mu, int block,
-                          int lanes, float4 *sym_sum, unsigned *sym_mu) {
+                          int lanes, float4 *sym_sum, unsigned *sym_mu, bool one_case) {
   if (n <= 0) return;
   const int G = lanes == 1 || lanes == 2 || lanes == 4 ? lanes : 8;
   const int per = walk_targets(n, G);
   const ListArgs a{n,    nvalid, keys, walk, cid,   cstart, (uint32_t)(cap_cells + 1),
-                   nbits, cc,    dyn,  ace,  want_dt, list, cap, count, tau4, tau2, mu, per};
+                   nbits, cc,    dyn,  ace,  want_dt, list, cap, count, tau4, tau2, mu, one_case ? 1 : 0, per};
   // block size of the default kernel as asked for (pi_block); its default 256,
   // and always for the others (registers)
-  const int b0 = block >= 128 && block <= 1024 && block % 32 == 0 ? block : 256;
+  const int b0 = block == 128 ? 128 : 256;
   const int64_t threads = (n + (int64_t)per * (32 / G) - 1) / (per * (32 / G)) * 32;
 #define SPH_LANES(CALL) \
   switch (G) {          \

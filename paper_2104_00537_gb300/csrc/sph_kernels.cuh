@@ -105,7 +105,7 @@ void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const 
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
                           float4 *tau4, float2 *tau2, cudaStream_t s, float *mu = nullptr,
                           int block = 0, int lanes = 0, float4 *sym_sum = nullptr,
-                          unsigned *sym_mu = nullptr);
+                          unsigned *sym_mu = nullptr, bool one_case = false);
 // The walk records of a state (posc, velrho, press in the cells of keys).
 void launch_pack_walk(int n, const uint32_t *keys, const float4 *posc, const float4 *velrho,
                       const float *press, const uint16_t *cid, const CaseConst *cc, int nbits,

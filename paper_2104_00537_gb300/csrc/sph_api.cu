@@ -882,8 +882,12 @@ void enqueue_reuse_rebuild(sph_engine e, cudaEvent_t *ev) {
   auto nl_part = [=](cudaStream_t q) { enqueue_rebuild_sort(e, q); };
   auto list_part = [=](cudaStream_t q) { enqueue_rebuild_list(e, extra, q); };
   if (e->capturing) {
-    capture_if_rebuild(e, nl_part);
-    capture_if_rebuild(e, list_part);
+    // one IF node around both parts: a node that is not taken costs about 5 us
+    // with the kernel before it, every step
+    capture_if_rebuild(e, [=](cudaStream_t q) {
+      enqueue_rebuild_sort(e, q);
+      enqueue_rebuild_list(e, extra, q);
+    });
   } else {
     eager_if_rebuild(e, 0, nl_part);
     if (ev) cudaEventRecord(ev[0], e->s);
@@ -1111,7 +1115,7 @@ int sph_step(sph_engine e, int64_t nsteps) {
     t1 = e->evs[4 * nsteps + 1];
     CUDA_TRY(cudaEventRecord(t0, e->s));
   }
-  int64_t k = 0;
+  int64_t k = 0, decides = 2;  // k_decide launches per kept-list step
   const bool reuse = use_list(e) && e->opt.pi_variant == 5;
   if (reuse) {
     if (!e->s2) CUDA_TRY(cudaStreamCreateWithFlags(&e->s2, cudaStreamNonBlocking));
@@ -1147,6 +1151,7 @@ int sph_step(sph_engine e, int64_t nsteps) {
       e->graph_ext = graph_key(e);
     }
     for (; k < nsteps; k++) CUDA_TRY(cudaGraphLaunch(e->gexec, e->s));
+    decides = 1;
   }
   // per Symplectic step: 2 sorts (3 kernels per 8-bit pass), 2 reorders, 2
   // cell tables (4 kernels), 2 interactions, dt, predictor, corrector, end of
@@ -1156,11 +1161,11 @@ int sph_step(sph_engine e, int64_t nsteps) {
   const int64_t passes = std::max(1, (e->nbits + 7) / 8);
   const int64_t pis = e->integrator == 1 ? 1 : 2;
   const bool listed = use_list(e);
-  // (the list kept across steps: 2 decide kernels, 2 interactions, dt,
-  // predictor, corrector, end per step; the sort, reorder, cell table, skin
+  // (the list kept across steps: 2 decide kernels, 1 in a captured graph, 2
+  // interactions, dt, predictor, corrector, end per step; the sort, reorder, cell table, skin
   // and list per build, counted from the device's build counter)
-  const int64_t per_step = (e->integrator == 1 ? (reuse ? 2 + 1 + 3 : 3 * passes + 1 + 4 + 1 + 3)
-                            : reuse            ? 2 + 2 + 4
+  const int64_t per_step = (e->integrator == 1 ? (reuse ? decides + 1 + 3 : 3 * passes + 1 + 4 + 1 + 3)
+                            : reuse            ? decides + 2 + 4
                             : listed           ? 3 * passes + 1 + 4 + 1 + 2 + 4 +
                                                      (e->opt.pi_variant == 4 ? 1 : 0)
                                                : 6 * passes + 2 + 8 + 2 + 4) +

@@ -1699,13 +1699,17 @@ __device__ __forceinline__ double motion_vel(const CaseConst &C, int g, double t
   return C.mot_amp[g] * C.mot_omega[g] * cos(C.mot_omega[g] * t + C.mot_phase[g]);
 }
 
-__global__ void k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncases) return;
+// One block per case.  The imposed motion's FP64 sines and cosines bound it (five
+// per motion, one after another, when one thread took the case: 8.4 us): a thread
+// for each displacement and velocity of each motion.
+__global__ void __launch_bounds__(4 * kMaxMotions)
+k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn) {
+  const int c = blockIdx.x;
   const CaseConst &C = cc[c];
   CaseDyn &D = dyn[c];
   if (!C.active) return;
-  unsigned bits = D.dtmin_bits;
+  const unsigned bits = D.dtmin_bits;
+  const double t = D.t;
   double dt;
   if (C.dt_fixed > 0.0) {
     dt = C.dt_fixed;
@@ -1714,17 +1718,18 @@ __global__ void k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__re
   } else {
     dt = C.cfl * (double)__uint_as_float(bits);
   }
-  if (dt < C.dt_min) D.flags |= kFlagDtMin;
-  if (C.t_end > 0.0 && D.t >= C.t_end) dt = 0.0;  // finished cases stay put
-  D.dt = dt;
-  D.dtmin_bits = kFloatInfBits;
-  for (int g = 0; g < C.nmot; g++) {
-    double d0 = motion_disp(C, g, D.t);
-    D.mot[g][0] = motion_disp(C, g, D.t + 0.5 * dt) - d0;
-    D.mot[g][1] = motion_vel(C, g, D.t + 0.5 * dt);
-    D.mot[g][2] = motion_disp(C, g, D.t + dt) - d0;
-    D.mot[g][3] = motion_vel(C, g, D.t + dt);
+  const bool small = dt < C.dt_min;
+  if (C.t_end > 0.0 && t >= C.t_end) dt = 0.0;  // finished cases stay put
+  __syncthreads();  // every thread has read the case's values
+  if (threadIdx.x == 0) {
+    if (small) D.flags |= kFlagDtMin;
+    D.dt = dt;
+    D.dtmin_bits = kFloatInfBits;
   }
+  const int g = threadIdx.x >> 2, w = threadIdx.x & 3;
+  if (g >= C.nmot) return;
+  const double te = w < 2 ? t + 0.5 * dt : t + dt;
+  D.mot[g][w] = w & 1 ? motion_vel(C, g, te) : motion_disp(C, g, te) - motion_disp(C, g, t);
 }
 
 __global__ void k_end_step(int ncases, const CaseConst *__restrict__ cc,
@@ -3311,7 +3316,7 @@ void launch_interact(int margin, int variant, int n, const int *nvalid, const ui
 }
 
 void launch_dt(int ncases, const CaseConst *cc, CaseDyn *dyn, cudaStream_t s) {
-  k_dt<<<nblk(ncases, 64), 64, 0, s>>>(ncases, cc, dyn);
+  if (ncases > 0) k_dt<<<ncases, 4 * kMaxMotions, 0, s>>>(ncases, cc, dyn);
 }
 
 void launch_end_step(int ncases, const CaseConst *cc, CaseDyn *dyn, cudaStream_t s) {

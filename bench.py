@@ -631,10 +631,11 @@ def main():
                           args.warmup, args.warmup + args.steps),
                       "neighbour_list": (
                           {"builds_per_step": builds / args.steps,
-                           "records": "wide (32-bit index)" if n_particles >= (1 << 25)
-                           else "narrow (25-bit index + row code)",
+                           "records": "candidate indices (32 bits)",
                            "skin": "list_k |v|max + 1e-3 h + %g x 2h" % (
-                               args.list_skin if args.list_skin >= 0 else 0.04)}
+                               args.list_skin if args.list_skin >= 0 else
+                               0.04 if args.visc_mode == 1 or args.boundary_mode == 1 else
+                               0.08 if n_particles < 32768 else 0.055)}
                           if eff_var == 5 else
                           {"builds_per_step": builds / args.steps} if eff_var in (3, 4)
                           else None),

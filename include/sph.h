@@ -169,7 +169,9 @@ typedef struct {
                        * steps then run without the captured step graph   */
   float list_skin;    /* pi_variant 5: skin added for the steps the list is
                        * kept, as a fraction of 2h, in [0, 0.25]; < 0: the
-                       * default (0.04)                                    */
+                       * default (per case: 0.04 with laminar + SPS or
+                       * mDBC, else 0.08 below 32,768 particles, 0.055 from
+                       * there on)                                         */
   int32_t check_list; /* 1: after every list evaluation, count the pairs of
                        * every target by brute force and compare (tests;
                        * sph_list_info reports the result)                */

@@ -127,6 +127,16 @@ void fill_const(const sph_case_params &p, const sph_particles &parts, const Grid
   C.cw = (float)(-5.0 * aD / (p.h * p.h));
   C.wk = (float)aD;
   C.list_k = (float)(1.25 * (p.dt_fixed > 0 ? p.dt_fixed : p.cfl * p.h / p.cs0));
+  // The kept list's default skin.  A wider one is rebuilt less often and walked
+  // longer.  Measured at 0.04 / 0.055 / 0.07 / 0.09 (us per step): 6k particles
+  // 89 / 84 / 80 / 78, 28k 72 / 68 / 66 / 64, 167k 249 / 244 / 244 / 250, 410k Verlet
+  // 244 / 235 / 237 / 244, 1.5M 1377 / 1372 / 1410 / 1513, batch of 420k 769 / 737 /
+  // 744 / 764; SPS 270k 563 / 572 / 588 / 627, mDBC 190k 347 / 354 / 358 / 375 (their
+  // evaluations cost more beside a build).  By the case alone, so that it takes the
+  // same steps in any engine.
+  C.list_extra = p.visc_mode == 1 || p.boundary_mode == 1 ? 0.04f
+                 : parts.n < 32768                        ? 0.08f
+                                                          : 0.055f;
   C.half_inv_h = (float)(0.5 / p.h);
   // artificial viscosity only in visc_mode 0; laminar + SPS constants otherwise
   C.kvisc = p.visc_mode == 0 ? (float)(-2.0 * p.alpha * p.cs0 * p.h) : 0.f;
@@ -878,7 +888,7 @@ void eager_if_rebuild(sph_engine e, int which, F fn) {
 // then sits between the two parts, so that the first evaluation's time
 // includes the list build).
 void enqueue_reuse_rebuild(sph_engine e, cudaEvent_t *ev) {
-  const float extra = e->opt.list_skin >= 0.f ? e->opt.list_skin : 0.04f;
+  const float extra = e->opt.list_skin;  // (< 0: each case's default)
   auto nl_part = [=](cudaStream_t q) { enqueue_rebuild_sort(e, q); };
   auto list_part = [=](cudaStream_t q) { enqueue_rebuild_list(e, extra, q); };
   if (e->capturing) {

@@ -60,6 +60,7 @@ struct CaseConst {
   // 1/2h in that unit
   float unit, inv_unit, fix_hi, fix_lo;
   float walk_r2max, walk_eta2, walk_hih;
+  float list_extra;  // the kept list's default skin beyond one step's need, x 2h
   float list_k;   // 1.25 x the Eq 35 bound on dt (or the fixed dt): skin = list_k |v|max + 1e-3 h
 };
 

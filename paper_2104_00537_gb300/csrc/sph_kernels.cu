@@ -650,7 +650,7 @@ __device__ __forceinline__ void finish_target(const CaseConst &C, int i, int n, 
 // its records from its build positions with its old skin, and the rest keep
 // their records.  Clears the rebuild request and counts the build.
 __global__ void k_list_begin(int ncases, const CaseConst *__restrict__ cc,
-                             CaseDyn *__restrict__ dyn, ListCtl *__restrict__ ctl, float extra,
+                             CaseDyn *__restrict__ dyn, ListCtl *__restrict__ ctl, float extra_opt,
                              int fresh_all, const uint32_t *__restrict__ cstart, uint32_t cap1) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c == 0 && ctl) {
@@ -666,6 +666,7 @@ __global__ void k_list_begin(int ncases, const CaseConst *__restrict__ cc,
     const float need = fmaf(C.list_k, sqrtf(__uint_as_float(D.v2max_bits)), 1e-3f * C.h);
     const float smax = 0.95f * C.csf;
     if (need > smax) D.flags |= kFlagSkin;
+    const float extra = extra_opt >= 0.f ? extra_opt : C.list_extra;
     D.skin = fminf(fmaf(extra, 2.f * C.h, need), smax);
     D.lmode = 1u;
   } else {

@@ -334,11 +334,11 @@ class Engine:
         a neighbour list: kept across steps, 5; else the compacted loop, 0;
         4, one list per step, keeps batch and pool cases equal to their runs
         alone bit for bit); list_skin:
-        variant 5's added skin as a fraction of 2h (< 0: the default, 0.04);
+        variant 5's added skin as a fraction of 2h (< 0: the default, per case);
         check_list: brute-force check of every list evaluation (list_info);
         pi_lanes: threads per target of the list walk (0: the default);
         pair_once: evaluate each pair once (atomic sums, not bit-reproducible);
-        wide_records: 32-bit list records at any size (else beyond 2^25 only)."""
+        wide_records: of no effect (lists hold 32-bit indices at every size)."""
         o = Options(pi_block, pi_variant, use_graph, timing, list_skin, check_list, pi_lanes,
                     pair_once, wide_records)
         check(self.lib.sph_set_options(self.h, C.byref(o)))

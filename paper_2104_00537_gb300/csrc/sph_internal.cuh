@@ -82,6 +82,7 @@ struct CaseDyn {
   // state, 2 rebuild from the build positions after an index shift);
   // startF / startB = first fluid / boundary index of the case at its build
   unsigned int need, lmode, startF, startB;
+  float dts[2], hdt[2], hdt2[2];  // dt, dt / 2 and dt^2 / 2, each in two FP32 parts
   double mot[kMaxMotions][4];  // displacement and velocity at t+dt/2 and t+dt
 };
 

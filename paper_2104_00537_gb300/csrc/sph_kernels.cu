@@ -47,18 +47,54 @@ __device__ __forceinline__ float below(float cs) {  // largest float < cs
   return __int_as_float(__float_as_int(cs) - 1);
 }
 
-// New offset after adding disp (FP64) to a float offset in [0, cs); returns
-// the cell shift.  The sum is formed in FP64; when its float rounding stays
-// inside the cell (the common case) that rounding is the new offset, and
-// only a particle that changes cell takes the FP64 floor / shift path.
-__device__ __forceinline__ int shift_axis(float off, double disp, const CaseConst &C,
+// A displacement as the unevaluated sum of two FP32 numbers (48 bits; products of
+// dt, itself split, with FP32 velocities).  FP64 runs at 1/74 of the FP32 rate here
+// and, with its conversions, bound the predictor (60 us for 1.48M particles) and the
+// corrector (65 us); an error-free FP32 sum of offset and displacement takes ten
+// FP32 operations.
+struct Disp {
+  float hi, lo;
+};
+__device__ __forceinline__ Disp disp_scaled(const float (&c)[2], float v) {  // (c[0] + c[1]) v
+  Disp d;
+  d.hi = __fmul_rn(c[0], v);
+  d.lo = fmaf(c[1], v, fmaf(c[0], v, -d.hi));
+  return d;
+}
+__device__ __forceinline__ Disp disp_sum(const Disp &a, const Disp &b) {
+  Disp d;
+  d.hi = __fadd_rn(a.hi, b.hi);
+  const float t = __fsub_rn(d.hi, a.hi);
+  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(d.hi, t)), __fsub_rn(b.hi, t));
+  d.lo = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
+  return d;
+}
+__device__ __forceinline__ Disp disp_of(double x) {
+  Disp d;
+  d.hi = (float)x;
+  d.lo = (float)(x - (double)d.hi);
+  return d;
+}
+// off + d, rounded once to FP32 (the sum of off and d.hi with its exact error,
+// Knuth's two-sum)
+__device__ __forceinline__ float add_disp(float off, const Disp &d) {
+  const float s = __fadd_rn(off, d.hi), t = __fsub_rn(s, off);
+  const float e = __fadd_rn(__fsub_rn(off, __fsub_rn(s, t)), __fsub_rn(d.hi, t));
+  return __fadd_rn(s, __fadd_rn(e, d.lo));
+}
+
+// New offset after adding disp to a float offset in [0, cs); returns the cell
+// shift.  When the sum's float rounding stays inside the cell (the common case)
+// that rounding is the new offset, and only a particle that changes cell takes the
+// FP64 floor / shift path.
+__device__ __forceinline__ int shift_axis(float off, const Disp &disp, const CaseConst &C,
                                           float &off_out) {
-  double x = (double)off + disp;
-  const float xf = (float)x;
+  const float xf = add_disp(off, disp);
   if (xf >= 0.f && xf < C.csf) {
     off_out = xf;
     return 0;
   }
+  double x = (double)off + ((double)disp.hi + (double)disp.lo);
   double k = floor(x * C.inv_cs);
   x = fma(-k, C.cs, x);
   if (x < 0.0) {
@@ -1700,6 +1736,11 @@ __device__ __forceinline__ double motion_vel(const CaseConst &C, int g, double t
   return C.mot_amp[g] * C.mot_omega[g] * cos(C.mot_omega[g] * t + C.mot_phase[g]);
 }
 
+__device__ __forceinline__ void split(double x, float (&f)[2]) {
+  f[0] = (float)x;
+  f[1] = (float)(x - (double)f[0]);
+}
+
 // One block per case.  The imposed motion's FP64 sines and cosines bound it (five
 // per motion, one after another, when one thread took the case: 8.4 us): a thread
 // for each displacement and velocity of each motion.
@@ -1726,6 +1767,9 @@ k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn) {
     if (small) D.flags |= kFlagDtMin;
     D.dt = dt;
     D.dtmin_bits = kFloatInfBits;
+    split(dt, D.dts);
+    split(0.5 * dt, D.hdt);
+    split(0.5 * dt * dt, D.hdt2);
   }
   const int g = threadIdx.x >> 2, w = threadIdx.x & 3;
   if (g >= C.nmot) return;
@@ -1749,7 +1793,7 @@ __global__ void k_end_step(int ncases, const CaseConst *__restrict__ cc,
 
 // Moves a particle by disp (FP64, per axis) from the cell of key k; returns
 // the new key (or key_out) and writes the new offsets.
-__device__ __forceinline__ uint32_t move_particle(uint32_t k, const float4 &p, const double disp[3],
+__device__ __forceinline__ uint32_t move_particle(uint32_t k, const float4 &p, const Disp disp[3],
                                                   const CaseConst &C, bool boundary, int nbits,
                                                   float4 &pout, bool &left) {
   int cx, cy, cz;
@@ -1776,13 +1820,12 @@ __device__ __forceinline__ uint32_t move_particle(uint32_t k, const float4 &p, c
 // displaced by Eq 37 at t + dt/2.
 __device__ __forceinline__ void predictor_core(const CaseConst &C, const CaseDyn &D,
                                                uint8_t code, const float4 &v, const float4 &a,
-                                               double disp[3], float4 &vn) {
-  const double hdt = 0.5 * D.dt;
-  const float hdtf = (float)hdt;
+                                               Disp disp[3], float4 &vn) {
+  const float hdtf = D.hdt[0];
   if (code == 0) {
-    disp[0] = hdt * (double)v.x;
-    disp[1] = hdt * (double)v.y;
-    disp[2] = hdt * (double)v.z;
+    disp[0] = disp_scaled(D.hdt, v.x);
+    disp[1] = disp_scaled(D.hdt, v.y);
+    disp[2] = disp_scaled(D.hdt, v.z);
     vn = make_float4(fmaf(hdtf, a.x, v.x), fmaf(hdtf, a.y, v.y), fmaf(hdtf, a.z, v.z),
                      fmaf(hdtf, a.w, v.w));
   } else {
@@ -1792,12 +1835,12 @@ __device__ __forceinline__ void predictor_core(const CaseConst &C, const CaseDyn
       const int g = code - 2;
       const double d = D.mot[g][0];
       const float vm = (float)D.mot[g][1];
-      disp[0] = d * C.mot_axis[g][0];
-      disp[1] = d * C.mot_axis[g][1];
-      disp[2] = d * C.mot_axis[g][2];
+      disp[0] = disp_of(d * C.mot_axis[g][0]);
+      disp[1] = disp_of(d * C.mot_axis[g][1]);
+      disp[2] = disp_of(d * C.mot_axis[g][2]);
       vn = make_float4(vm * C.mot_axis[g][0], vm * C.mot_axis[g][1], vm * C.mot_axis[g][2], rho);
     } else {
-      disp[0] = disp[1] = disp[2] = 0.0;
+      disp[0] = disp[1] = disp[2] = Disp{0.f, 0.f};
       vn = make_float4(v.x, v.y, v.z, rho);
     }
   }
@@ -1822,7 +1865,7 @@ __global__ void k_predictor(int n, const uint32_t *__restrict__ keys_in, State s
   const uint8_t code = src.code[i];
   const CaseConst &C = cc[cidx];
   const CaseDyn &D = dyn[cidx];
-  double disp[3];
+  Disp disp[3];
   float4 vn;
   predictor_core(C, D, code, v, ace[i], disp, vn);
   float4 pn;
@@ -1850,34 +1893,32 @@ __device__ __forceinline__ uint32_t corrector_core(const CaseConst &C, const Cas
                                                    const float4 &vn, float rhoh, const float4 &a,
                                                    int nbits, int cidx, CaseDyn *dyn,
                                                    float4 &pnew, float4 &vnew,
-                                                   double *disp_out = nullptr) {
-  const double dt = D.dt;
-  const float dtf = (float)dt;
+                                                   Disp *disp_out = nullptr) {
+  const float dtf = D.dts[0];
   // Eq 34: rho^{n+1} = rho^n (2 - eps) / (2 + eps), eps = -(R / rho^{n+1/2}) dt
   const float eps = -(a.w / rhoh) * dtf;
   float rho = vn.w * (2.f - eps) / (2.f + eps);
-  double disp[3];
+  Disp disp[3];
   if (code == 0) {
     vnew = make_float4(fmaf(dtf, a.x, vn.x), fmaf(dtf, a.y, vn.y), fmaf(dtf, a.z, vn.z), rho);
     // r^{n+1} = r^n + dt (v^{n+1} + v^n) / 2: the FP32 sum of two FP32
-    // velocities is exact to within one rounding; dt multiplies in FP64
-    const double hdt = 0.5 * dt;
-    disp[0] = hdt * (double)(vnew.x + vn.x);
-    disp[1] = hdt * (double)(vnew.y + vn.y);
-    disp[2] = hdt * (double)(vnew.z + vn.z);
+    // velocities is exact to within one rounding; dt multiplies split
+    disp[0] = disp_scaled(D.hdt, vnew.x + vn.x);
+    disp[1] = disp_scaled(D.hdt, vnew.y + vn.y);
+    disp[2] = disp_scaled(D.hdt, vnew.z + vn.z);
   } else {
     if (C.clamp && rho < C.rho0) rho = C.rho0;
     if (code >= 2) {
       const int g = code - 2;
       const double d = D.mot[g][2];
       const float vm = (float)D.mot[g][3];
-      disp[0] = d * C.mot_axis[g][0];
-      disp[1] = d * C.mot_axis[g][1];
-      disp[2] = d * C.mot_axis[g][2];
+      disp[0] = disp_of(d * C.mot_axis[g][0]);
+      disp[1] = disp_of(d * C.mot_axis[g][1]);
+      disp[2] = disp_of(d * C.mot_axis[g][2]);
       vnew = make_float4(vm * C.mot_axis[g][0], vm * C.mot_axis[g][1], vm * C.mot_axis[g][2],
                          rho);
     } else {
-      disp[0] = disp[1] = disp[2] = 0.0;
+      disp[0] = disp[1] = disp[2] = Disp{0.f, 0.f};
       vnew = make_float4(vn.x, vn.y, vn.z, rho);
     }
   }
@@ -2667,15 +2708,17 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
     return;
   }
   const CaseDyn &D = dyn[cidx];
-  double disp[3];
+  Disp disp[3];
   float4 vn;
   predictor_core(C, D, code, v, a, disp, vn);
   const float hs = 0.5f * D.skin;
-  float dx = (float)disp[0], dy = (float)disp[1], dz = (float)disp[2];
+  const float4 ph = make_float4(add_disp(p.x, disp[0]), add_disp(p.y, disp[1]),
+                                add_disp(p.z, disp[2]), p.w);
+  float dx = disp[0].hi, dy = disp[1].hi, dz = disp[2].hi;
   if (REF) {
-    dx = (float)((double)p.x + disp[0]) - r.x;
-    dy = (float)((double)p.y + disp[1]) - r.y;
-    dz = (float)((double)p.z + disp[2]) - r.z;
+    dx = ph.x - r.x;
+    dy = ph.y - r.y;
+    dz = ph.z - r.z;
   }
   if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > hs * hs) atomicOr(&dyn[cidx].flags, kFlagSkin);
   float4 ptmp;
@@ -2689,8 +2732,6 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
     atomicAdd(&dyn[cidx].n_out, 1);
     return;
   }
-  const float4 ph = make_float4((float)((double)p.x + disp[0]), (float)((double)p.y + disp[1]),
-                                (float)((double)p.z + disp[2]), p.w);
   const float Q = tait_pressure(C, vn.w) / vn.w;  // P/rho of Eq 28 at n+1/2
   posc_out[i] = ph;
   velrho_out[i] = vn;
@@ -2796,7 +2837,7 @@ __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
   }
   const CaseDyn &D = dyn[cidx];
   float4 pnew, vnew;
-  double disp[3];
+  Disp disp[3];
   const uint32_t kn = corrector_core(C, D, code, k, pn, vn, rho_half, a, nbits,
                                      cidx, dyn, pnew, vnew, disp);
   x.posc[i] = pnew;
@@ -2808,8 +2849,8 @@ __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
     ctl->rebuild = 1u;
     return;
   }
-  const float4 pu = make_float4((float)((double)pn.x + disp[0]), (float)((double)pn.y + disp[1]),
-                                (float)((double)pn.z + disp[2]), pn.w);
+  const float4 pu = make_float4(add_disp(pn.x, disp[0]), add_disp(pn.y, disp[1]),
+                                add_disp(pn.z, disp[2]), pn.w);
   y.posc[i] = pu;
   y.velrho[i] = vnew;
   const float Q = tait_pressure(C, vnew.w) / vnew.w;
@@ -2934,32 +2975,31 @@ __global__ void k_verlet(int n, const uint32_t *__restrict__ keys_in, State src,
     return;
   }
   const bool eq31 = (D.step % C.verlet_steps) == 0;
-  const float dtf = (float)dt;
+  const float dtf = D.dts[0];
   const float4 a = ace[i];
   const float4 base = eq31 ? v : vp;  // v, rho at n (Eq 31) or n-1 (Eq 30)
   const float fdt = eq31 ? dtf : 2.f * dtf;
   float rho = fmaf(fdt, a.w, base.w);
-  double disp[3];
+  Disp disp[3];
   float4 vnew;
   if (code == 0) {
     vnew = make_float4(fmaf(fdt, a.x, base.x), fmaf(fdt, a.y, base.y), fmaf(fdt, a.z, base.z), rho);
-    const double hdt2 = 0.5 * dt * dt;
-    disp[0] = fma(hdt2, (double)a.x, dt * (double)v.x);
-    disp[1] = fma(hdt2, (double)a.y, dt * (double)v.y);
-    disp[2] = fma(hdt2, (double)a.z, dt * (double)v.z);
+    disp[0] = disp_sum(disp_scaled(D.dts, v.x), disp_scaled(D.hdt2, a.x));
+    disp[1] = disp_sum(disp_scaled(D.dts, v.y), disp_scaled(D.hdt2, a.y));
+    disp[2] = disp_sum(disp_scaled(D.dts, v.z), disp_scaled(D.hdt2, a.z));
   } else {
     if (C.clamp && rho < C.rho0) rho = C.rho0;
     if (code >= 2) {
       const int g = code - 2;
       const double d = D.mot[g][2];
       const float vm = (float)D.mot[g][3];
-      disp[0] = d * C.mot_axis[g][0];
-      disp[1] = d * C.mot_axis[g][1];
-      disp[2] = d * C.mot_axis[g][2];
+      disp[0] = disp_of(d * C.mot_axis[g][0]);
+      disp[1] = disp_of(d * C.mot_axis[g][1]);
+      disp[2] = disp_of(d * C.mot_axis[g][2]);
       vnew = make_float4(vm * C.mot_axis[g][0], vm * C.mot_axis[g][1], vm * C.mot_axis[g][2],
                          rho);
     } else {
-      disp[0] = disp[1] = disp[2] = 0.0;
+      disp[0] = disp[1] = disp[2] = Disp{0.f, 0.f};
       vnew = make_float4(v.x, v.y, v.z, rho);
     }
   }
@@ -2978,8 +3018,8 @@ __global__ void k_verlet(int n, const uint32_t *__restrict__ keys_in, State src,
       ctl->rebuild = 1u;
       return;
     }
-    const float4 pu = make_float4((float)((double)p.x + disp[0]), (float)((double)p.y + disp[1]),
-                                  (float)((double)p.z + disp[2]), p.w);
+    const float4 pu = make_float4(add_disp(p.x, disp[0]), add_disp(p.y, disp[1]),
+                                  add_disp(p.z, disp[2]), p.w);
     src.posc[i] = pu;
     src.velrho[i] = vnew;
     src.vrprev[i] = v;

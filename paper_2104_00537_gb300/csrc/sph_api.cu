@@ -920,8 +920,8 @@ void enqueue_step_reuse(sph_engine e, cudaEvent_t *ev) {
   enqueue_list_first(e, ev, nullptr);
   enqueue_list_half(e, ev, nullptr);
   launch_corrector_reuse(nl, e->keysB, e->keysC, Y, Z.velrho, e->ace, e->posc_ref, e->dconst,
-                         e->ddyn, e->nbits, X, e->keysA, e->press, e->ctl, e->walk, e->s);
-  launch_end_step(e->cap_cases, e->dconst, e->ddyn, e->s);
+                         e->ddyn, e->nbits, X, e->keysA, e->press, e->ctl, e->walk,
+                         e->cap_cases, e->s);
 }
 
 // One Verlet step over the list kept across steps: the guarded sort +
@@ -1172,10 +1172,10 @@ int sph_step(sph_engine e, int64_t nsteps) {
   const int64_t pis = e->integrator == 1 ? 1 : 2;
   const bool listed = use_list(e);
   // (the list kept across steps: 2 decide kernels, 1 in a captured graph, 2
-  // interactions, dt, predictor, corrector, end per step; the sort, reorder, cell table, skin
+  // interactions, dt, predictor, corrector per step; the sort, reorder, cell table, skin
   // and list per build, counted from the device's build counter)
   const int64_t per_step = (e->integrator == 1 ? (reuse ? decides + 1 + 3 : 3 * passes + 1 + 4 + 1 + 3)
-                            : reuse            ? decides + 2 + 4
+                            : reuse            ? decides + 2 + 3
                             : listed           ? 3 * passes + 1 + 4 + 1 + 2 + 4 +
                                                      (e->opt.pi_variant == 4 ? 1 : 0)
                                                : 6 * passes + 2 + 8 + 2 + 4) +

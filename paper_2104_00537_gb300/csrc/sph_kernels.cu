@@ -1730,22 +1730,16 @@ k_mdbc(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__ key
 
 // ---- time step and motion ----------------------------------------------------
 
-__device__ __forceinline__ double motion_disp(const CaseConst &C, int g, double t) {
-  return C.mot_amp[g] * (sin(C.mot_omega[g] * t + C.mot_phase[g]) - sin(C.mot_phase[g]));
-}
-__device__ __forceinline__ double motion_vel(const CaseConst &C, int g, double t) {
-  return C.mot_amp[g] * C.mot_omega[g] * cos(C.mot_omega[g] * t + C.mot_phase[g]);
-}
-
 __device__ __forceinline__ void split(double x, float (&f)[2]) {
   f[0] = (float)x;
   f[1] = (float)(x - (double)f[0]);
 }
 
-// One block per case.  The imposed motion's FP64 sines and cosines bound it (five
-// per motion, one after another, when one thread took the case: 8.4 us): a thread
-// for each displacement and velocity of each motion.
-__global__ void __launch_bounds__(4 * kMaxMotions)
+// One block per case.  The imposed motion's FP64 sines and cosines bound it (8.4 us
+// with one motion when one thread took them in turn): of each motion's eight
+// threads, 0 to 3 take the sine and cosine at t + dt/2 and at t + dt, 4 the sine
+// at t, so that each waits for one.
+__global__ void __launch_bounds__(8 * kMaxMotions)
 k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn) {
   const int c = blockIdx.x;
   const CaseConst &C = cc[c];
@@ -1772,22 +1766,33 @@ k_dt(int ncases, const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn) {
     split(0.5 * dt, D.hdt);
     split(0.5 * dt * dt, D.hdt2);
   }
-  const int g = threadIdx.x >> 2, w = threadIdx.x & 3;
-  if (g >= C.nmot) return;
-  const double te = w < 2 ? t + 0.5 * dt : t + dt;
-  D.mot[g][w] = w & 1 ? motion_vel(C, g, te) : motion_disp(C, g, te) - motion_disp(C, g, t);
+  if (C.nmot == 0) return;
+  const int g = threadIdx.x >> 3, w = threadIdx.x & 7;
+  const bool on = g < C.nmot && w < 5;
+  const double te = w < 2 ? t + 0.5 * dt : (w < 4 ? t + dt : t);
+  const double x = on ? C.mot_omega[g] * te + C.mot_phase[g] : 0.0;
+  const double f = on ? (w == 1 || w == 3 ? cos(x) : sin(x)) : 0.0;
+  const double f0 = __shfl_sync(0xffffffffu, f, 4, 8);  // sin at t
+  if (on && w < 4)
+    D.mot[g][w] = w & 1 ? C.mot_amp[g] * C.mot_omega[g] * f : C.mot_amp[g] * (f - f0);
 }
 
-__global__ void k_end_step(int ncases, const CaseConst *__restrict__ cc,
-                           CaseDyn *__restrict__ dyn) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncases || !cc[c].active) return;
+// t += dt (FP64) and the step count of case c, and its |v|max for the next reorder.
+__device__ __forceinline__ void end_step(int c, const CaseConst *__restrict__ cc,
+                                         CaseDyn *__restrict__ dyn) {
+  if (!cc[c].active) return;
   CaseDyn &D = dyn[c];
   if (D.dt > 0.0) {
     D.t += D.dt;
     D.step += 1;
   }
   D.v2max_bits = 0u;
+}
+
+__global__ void k_end_step(int ncases, const CaseConst *__restrict__ cc,
+                           CaseDyn *__restrict__ dyn) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < ncases) end_step(c, cc, dyn);
 }
 
 // ---- Symplectic predictor / corrector ------------------------------------------
@@ -2792,7 +2797,7 @@ __global__ void k_corrector_list(int n, const uint32_t *__restrict__ keys_n,
 // |r - r_build| + 1.25 (dt_max / 2) |v| <= (skin - 1e-3 h) / 2 (dt_max the
 // Eq 35 bound: the displacement at n+1 and the most the next half step
 // adds); otherwise, or when a particle leaves the domain, the corrector
-// requests a rebuild.
+// requests a rebuild.  It also ends the step (end_step): a launch less.
 __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
                                   const uint32_t *__restrict__ keys_half, State y,
                                   const float4 *__restrict__ velrho_half,
@@ -2800,8 +2805,10 @@ __global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
                                   const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
                                   int nbits, State x, uint32_t *__restrict__ keys_next,
                                   float *__restrict__ press, ListCtl *__restrict__ ctl,
-                                  float4 *__restrict__ walk) {
+                                  float4 *__restrict__ walk, int ncases) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  // the end of the step, which nothing else in this kernel reads or writes
+  for (int c = i; c < ncases; c += gridDim.x * blockDim.x) end_step(c, cc, dyn);
   if (i >= n) return;
   // every load of the particle first (independent: one memory latency)
   const uint32_t k = keys_n[i];
@@ -3358,7 +3365,7 @@ void launch_interact(int margin, int variant, int n, const int *nvalid, const ui
 }
 
 void launch_dt(int ncases, const CaseConst *cc, CaseDyn *dyn, cudaStream_t s) {
-  if (ncases > 0) k_dt<<<ncases, 4 * kMaxMotions, 0, s>>>(ncases, cc, dyn);
+  if (ncases > 0) k_dt<<<ncases, 8 * kMaxMotions, 0, s>>>(ncases, cc, dyn);
 }
 
 void launch_end_step(int ncases, const CaseConst *cc, CaseDyn *dyn, cudaStream_t s) {
@@ -3590,11 +3597,11 @@ void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_
                             const float4 *velrho_half, const float4 *ace, const float4 *ref,
                             const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
                             uint32_t *keys_next, float *press, ListCtl *ctl, float4 *walk,
-                            cudaStream_t s) {
+                            int ncases, cudaStream_t s) {
   if (n > 0)
     k_corrector_reuse<<<nblk(n, 256), 256, 0, s>>>(n, keys_n, keys_half, y, velrho_half, ace,
                                                    ref, cc, dyn, nbits, x, keys_next, press,
-                                                   ctl, walk);
+                                                   ctl, walk, ncases);
 }
 
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s) {

@@ -116,12 +116,13 @@ void launch_predictor_list(int n, const uint32_t *keys_in, State src, const floa
                            const float4 *ref, float4 *walk, cudaStream_t s);
 // Corrector of the list kept across steps: state n+1 to x (normalised, keys)
 // and in place to y (the build's cells, P/rho to press); requests a rebuild
-// through ctl when the next step could leave the skin.
+// through ctl when the next step could leave the skin; ends the step of the
+// ncases cases (as launch_end_step).
 void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_half, State y,
                             const float4 *velrho_half, const float4 *ace, const float4 *ref,
                             const CaseConst *cc, CaseDyn *dyn, int nbits, State x,
                             uint32_t *keys_next, float *press, ListCtl *ctl, float4 *walk,
-                            cudaStream_t s);
+                            int ncases, cudaStream_t s);
 // One-thread kernel: sets conditional handle h to ctl->rebuild != 0.
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s);
 // Brute-force check of the list against the evaluated state (tests).

@@ -578,7 +578,7 @@ def main():
     # the committed capture is of the default physics and launch shape
     captured = ((args.ddt_mode, args.integrator, args.visc_mode, args.boundary_mode) ==
                 (1, "symplectic", 0, 0) and eff_var in (4, 5) and
-                args.pi_block in (0, 128) and args.pi_lanes in (0, 1) and args.list_skin < 0)
+                args.pi_block in (0, 256) and args.pi_lanes in (0, 8) and args.list_skin < 0)
     roofline = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak,
                 "flop_basis": "48 / 45 / 25 FLOP per directed fluid-fluid / fluid-boundary / "

@@ -138,15 +138,16 @@ typedef void (*sph_free_fn)(void *ptr, size_t bytes, void *stream, void *ctx);
 /* Engine-wide launch options (the autotuner's knobs). */
 typedef struct {
   int32_t pi_block;   /* threads per block of the list walk of the default
-                       * physics: 0 (default: 128), 128, 256, 512 or 1024;
-                       * the other interaction kernels use 128 */
+                       * physics: 0 (default: 256), 128, 256, or 512 and
+                       * 1024 (run as 256: the walk keeps blocks small);
+                       * the other interaction kernels choose their own */
   int32_t pi_variant; /* interaction pair loop: -1 the engine default (5 where
                        * a list is supported, else 0); 0 compacted hit
                        * masks; 1 test
                        * and evaluate inline; 2 hit masks queued per lane
                        * across rows (same sums as 0, bit for bit); 3, 4
                        * and 5 a neighbour list: candidates within 2h + skin
-                       * of state n in chunk records, walked by both
+                       * of state n as index lists, walked by both
                        * evaluations of a Symplectic step, no re-sort for
                        * the half step; 3 writes the list during the first
                        * evaluation, 4 builds it alone, once per step; 5
@@ -285,7 +286,7 @@ int sph_eval_forces(sph_engine e, int32_t icase, float *acc, float *drho,
  * 21-22, 35-36), without advancing the engine.  stage 0: the step's first
  * evaluation, on state n; stage 1: its second, on the half-step state of
  * Eq 33-34 (dt of Eq 35 from stage 0, then the predictor).  With a neighbour
- * list (pi_variant 3-5) both walk the list's chunk records, and with the list
+ * list (pi_variant 3-5) both walk the lists, and with the list
  * kept across steps (5) state n and state n+1/2 are those kept in the order
  * and cells of the list's build (cell offsets up to half the skin outside
  * [0, cs)).  The part of the next step before its first evaluation runs for

@@ -204,8 +204,8 @@ struct sph_engine_t {
   // neighbour list (pi_variant 3-5): a segment of list_cap chunk records (2
   // list_cap candidate indices) per target
   bool list_ok = false;
-  bool list_wide = false;  // wide records: beyond 2^25 particles (default physics only)
-  bool list_wide_needed = false;  // (then always; else as sph_options.wide_records)
+  bool list_wide = false;  // pi_variant 3 runs as 4: beyond 2^25 particles (lists of the
+  bool list_wide_needed = false;  // default physics only), or sph_options.wide_records
   int list_cap = 0;
   int64_t list_ld = 0;
   uint2 *nlist = nullptr;
@@ -370,7 +370,7 @@ bool sym_on(sph_engine e) {
 
 int resolve_variant(sph_engine e, int v) {
   if (v == -1) v = e->list_ok ? e->list_default : 0;
-  if (v == 3 && e->list_wide) v = 4;  // variant 3's records are narrow
+  if (v == 3 && e->list_wide) v = 4;
   if (v >= 3 && v <= 5 && (!e->list_ok || (e->integrator == 1 && v != 5))) v = 0;
   return v;
 }
@@ -590,8 +590,8 @@ int create_engine(const sph_case_params *params, const sph_particles *parts, int
     e->mdbc = e->mdbc || params[c].boundary_mode == 1;
   }
   // the neighbour list serves every physics option (the Verlet scheme only
-  // with the list kept across steps); beyond 2^25 particles its records are
-  // wide (the default physics only: the other walks keep the narrow form)
+  // with the list kept across steps); beyond 2^25 particles the default physics
+  // only, built alone (pi_variant 4, 5)
   e->list_ok = np < kListMaxParticles;
   if (!e->list_ok && !e->ext && !e->sps && !e->mdbc && np < ((int64_t)1 << 31)) {
     e->list_ok = true;
@@ -792,7 +792,7 @@ void enqueue_rebuild_sort(sph_engine e, cudaStream_t q) {
 
 // The list: per-case skin and build mode, then the build (a case that needs
 // it from its state, one whose indices moved from its build positions, the
-// rest keep their records).
+// rest keep their lists).
 void enqueue_rebuild_list(sph_engine e, float extra, cudaStream_t q) {
   const int nl = (int)(e->n_phys - e->n_dead);
   State &Y = e->S[1];
@@ -1098,7 +1098,6 @@ int sph_set_options(sph_engine e, const sph_options *opt) {
   if (opt->list_skin > (float)kListExtraMax)
     return fail(SPH_ERR_ARG, "list_skin must be at most 0.25 (or < 0 for the default)");
   e->opt = *opt;
-  // wide records where needed, or where asked for and the physics allows them
   e->list_wide = e->list_wide_needed ||
                  (opt->wide_records && e->list_ok && !e->ext && !e->sps && !e->mdbc && !e->pool);
   e->opt.pi_variant = resolve_variant(e, opt->pi_variant);

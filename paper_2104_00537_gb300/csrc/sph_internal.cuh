@@ -87,7 +87,7 @@ struct CaseDyn {
 };
 
 constexpr unsigned kFlagNaN = 1u, kFlagDtMin = 2u, kFlagQuota = 4u;
-// neighbour-list path: a target had more records than its list segment
+// neighbour-list path: a target had more chunk records than its list segment
 // holds; a displacement since the list's build exceeded half its skin (or
 // one step's need exceeded the largest skin the rows cover)
 constexpr unsigned kFlagListFull = 8u, kFlagSkin = 16u;

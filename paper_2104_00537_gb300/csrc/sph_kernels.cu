@@ -683,8 +683,8 @@ __device__ __forceinline__ void finish_target(const CaseConst &C, int i, int n, 
 // case builds from its state; else a case that needs a rebuild does (and
 // takes a new skin), one whose particles moved in the sorted order (another
 // case's particle left the domain, a case was admitted or released) rebuilds
-// its records from its build positions with its old skin, and the rest keep
-// their records.  Clears the rebuild request and counts the build.
+// its list from its build positions with its old skin, and the rest keep
+// their lists.  Clears the rebuild request and counts the build.
 __global__ void k_list_begin(int ncases, const CaseConst *__restrict__ cc,
                              CaseDyn *__restrict__ dyn, ListCtl *__restrict__ ctl, float extra_opt,
                              int fresh_all, const uint32_t *__restrict__ cstart, uint32_t cap1) {
@@ -744,12 +744,14 @@ __global__ void k_need_all(int ncases, CaseDyn *__restrict__ dyn) {
 // itself to a multiple of 16.  In a block of 16 entries the e-th candidate sits at
 // flat_slot(e), so that of eight lanes that read two entries side by side (one
 // 64-bit load) each takes candidates e and e + 8, and a warp's gathers go to
-// neighbouring records (walk of 1.48M particles 527 us; 544 with two 32-bit index
-// loads, 631 with candidates e and e + 1).  The warp takes its 32 targets one by one: the records go to registers, then each record's
-// candidates are written side by side by the lanes whose bit is set.  A target
-// whose candidates do not fit, or with more than 128 records, keeps its records
-// (kListRecords in its count).  Cost: about 11 warp-instructions per record,
-// paid once per build, against a list walk without masks, rows or bit scans.
+// neighbouring particles (walk of 1.48M particles 527 us; 544 with two 32-bit index
+// loads, 631 with candidates e and e + 1).  The warp takes its 32 targets one by
+// one: the records go to registers, then each record's candidates are written by
+// the lanes whose bit is set.  A target whose candidates do not fit, or with more
+// than 128 records, keeps its records (kListRecords in its count).  Issue-bound,
+// some 16 warp-instructions per record: the whole-list build of 1.48M particles
+// takes 1.24 ms with it and 0.74 without, once in eight to twelve steps, for a walk
+// without masks, rows and bit scans (733 to 527 us, twice a step).
 constexpr int kFlatRounds = 4;  // of 32 records
 __device__ __forceinline__ int flat_slot(int e) {
   return (e & ~15) | ((e << 1) & 14) | ((e >> 3) & 1);
@@ -1972,18 +1974,15 @@ __global__ void k_corrector(int n, const uint32_t *__restrict__ perm2,
 //
 // The Symplectic step evaluates the interaction on state n and on state n+1/2.
 // Instead of sorting again for n+1/2, the candidate test runs on state n with
-// radius 2h + skin and writes every chunk of candidates that passes as a
-// record (first index | row code, mask) into a per-target list; both
-// evaluations walk the records and keep the pairs with 0 < r^2 < (2h)^2 at
-// their own state.  The half-step state keeps the cells of state n (offsets
-// may leave [0, cs) by a half-step displacement), so relative positions stay
-// cell + offset in FP32.  The skin covers twice the largest displacement since
-// the build, which the predictor checks (kFlagSkin).  Variants 3 and 4 build
+// radius 2h + skin and leaves every target's candidates as a list of indices; both
+// evaluations walk the lists and keep the pairs with 0 < r^2 < (2h)^2 at their own
+// state.  The half-step state keeps the cells of state n (offsets may leave [0, cs)
+// by a half-step displacement).  The skin covers twice the largest displacement
+// since the build, which the predictor checks (kFlagSkin).  Variants 3 and 4 build
 // the list every step; 5 keeps it, with the particle order and cells, until a
-// particle of the case could leave the skin.  The pair set of each evaluation
-// is the same as with a fresh neighbour list; only the order of the sums
-// differs.
-
+// particle of the case could leave the skin.  The pair set of each evaluation is
+// that of a fresh neighbour list up to FP32 rounding at the cut-off; only the order
+// of the sums differs.
 
 // Arguments of the interaction over the neighbour list.
 struct ListArgs {
@@ -2036,17 +2035,18 @@ __device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j
 // The candidates of target i (all 32 lanes of the warp call it together, G
 // lanes with the same i; sub: the lane's rank among them).  In every iteration
 // lane sub takes two of the next 2 G entries (side by side in the list, one 64-bit
-// load an iteration ahead; see flatten_records) and gathers both records before it uses either: the lanes of
-// a target read neighbouring entries and, the list being in cell order, mostly
-// neighbouring records.  body(rx, ry, rz, r2, b, Qb, j) runs for every candidate
-// inside the support; positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
+// load an iteration ahead; see flatten_records) and gathers both walk records
+// before it uses either: the lanes of a target take neighbouring entries and, the
+// list being in cell order, mostly neighbouring particles.
+// body(rx, ry, rz, r2, b, Qb, j) runs for every candidate inside the support; positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
 // A lane without an entry takes the target itself (r2 = 0: no pair).
-// What bounds it (1.48M particles, 530 us): L1 gathers (data pipe 78 % of its
-// peak) and issue (68 %) together.  Measured and left out, per evaluation: records
-// double-buffered in registers 608 us, one candidate per iteration 634, no branch
-// around the pair terms 588 (against 562), targets taken by bricks of cells 535
-// (L1 hits 52 -> 72 %, same time), list entries dealt to lanes by index modulo 8,
-// free of bank conflicts, 541 but a build of 1.42 instead of 1.08 ms.
+// What bounds it (1.48M particles, 0.53 ms): L1 gathers (data pipe 78 % of its peak)
+// and issue (68 %) together.  Measured and left out, per evaluation: the records
+// double-buffered in registers 608 us, one candidate per iteration 634, 40 warps per
+// SM with spills 542, targets taken by bricks of cells 535 (L1 hits 52 to 72 %, same
+// time), no branch around the pair terms 588 (against 562 then), list entries dealt
+// to the lanes by index modulo 8, free of bank conflicts, 541, with a build of 1.42
+// instead of 1.08 ms.
 template <int G, class Body>
 __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const int sub,
                                           const unsigned cw, const float4 &pa,

@@ -91,7 +91,7 @@ void launch_mdbc_list(int n, const int *nvalid, const uint32_t *keys, State st, 
                       const CaseDyn *dyn, int stage, float4 *walk, const uint2 *list, int cap,
                       const uint16_t *count, cudaStream_t s);
 // First evaluation of the list step: the compacted pair loop on state n that
-// also writes every target's list (chunk records, radius 2h + skin) and count.
+// also writes every target's list (radius 2h + skin) and count.
 void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t *keys,
                            const float4 *posc, const float4 *velrho, const float *press,
                            const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,

@@ -174,7 +174,8 @@ typedef struct {
                        * mDBC, else 0.08 below 32,768 particles, 0.055 from
                        * there on)                                         */
   int32_t check_list; /* 1: after every list evaluation, count the pairs of
-                       * every target by brute force and compare (tests;
+                       * every target, and the fluid around every ghost node
+                       * of an mDBC case, by brute force and compare (tests;
                        * sph_list_info reports the result)                */
   int32_t pi_lanes;   /* threads that share one target in the list walk
                        * (pi_variant 3-5): 0 (default: 8), 1, 2, 4 or 8;

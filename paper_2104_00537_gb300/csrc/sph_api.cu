@@ -712,7 +712,8 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
   if (ev) cudaEventRecord(ev[1], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysB, Y.posc, Y.cid, e->dconst, e->nbits, e->nlist,
-                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk);
+                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk,
+                      e->mdbc && e->opt.pi_variant != 3 ? Y.ghost : nullptr);
 }
 
 // The rest of a list step up to its second evaluation: dt (Eq 35), the half
@@ -745,7 +746,8 @@ void enqueue_list_half(sph_engine e, cudaEvent_t *ev, float *mu) {
   if (ev) cudaEventRecord(ev[3], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysC, Z.posc, Y.cid, e->dconst, e->nbits, e->nlist,
-                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk);
+                      e->list_cap, e->ncount, e->ctl, s, sym_on(e), e->walk,
+                      e->mdbc && e->opt.pi_variant != 3 ? Y.ghost : nullptr);
 }
 
 // One Symplectic step with the per-step neighbour list: NL on state n (Y),

@@ -886,7 +886,6 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
     r2l = R * R;
     if (has) decode_cell((uint32_t)gc - C.cellbase, nx, C.ny, tcx, tcy, tcz);
   }
-  const unsigned r2l_u = __float_as_uint(r2l) - 1u;
   const float r2prune = r2l * 1.0001f;  // conservative: pruning never drops a pair
   int lcnt = 0;                          // LIST: records written
   const int lmode = (LIST >= 2 && ref) ? (int)dyn[cidx].lmode : 1;
@@ -903,6 +902,10 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
   constexpr bool HALF = LIST == 3;
   const bool node = LIST == 2 && ghost && has && !afluid && C.bmode == 1 && lmode != 0;
   const bool work = (has && (afluid || C.bmode == 0) && lmode != 0 && (!HALF || afluid)) || node;
+  // 0 < r2 < r2l, or, for a ghost node (a fluid particle on it is no pair with
+  // itself but the neighbour of the largest weight), 0 <= r2 < r2l
+  const unsigned r2l_lo = LIST == 2 && node ? 0u : 1u;
+  const unsigned r2l_u = __float_as_uint(r2l) - r2l_lo;
   Ext X;
   X.C = &C;
   X.unit = 1.f;
@@ -1007,7 +1010,7 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
               const float ry = sy - pb.y, rz = sz - pb.z;
               const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
               if (__float_as_uint(r2) - 1u < r2max_u) m |= 1u << k;
-              if (LIST && __float_as_uint(r2) - 1u < r2l_u) ml |= 1u << k;
+              if (LIST && __float_as_uint(r2) - r2l_lo < r2l_u) ml |= 1u << k;
             }
           }
           if (HALF) {  // half list: only candidates of larger index than the target
@@ -2602,6 +2605,14 @@ k_strain_list(const ListArgs a, float4 *__restrict__ tau4, float2 *__restrict__ 
   }
 }
 
+// Walk coordinate of a ghost node: that of its particle (p) and the offset d (whole
+// cells first: d may exceed 4 of them).
+__device__ __forceinline__ int node_coord(const CaseConst &C, float p, float d) {
+  const float u = floorf(d * C.inv_csf);
+  return (int)((unsigned)__float_as_int(p) +
+               (unsigned)walk_coord(C, (int)u, fmaf(-u, C.csf, d)));
+}
+
 // The mDBC boundary values (as k_mdbc) over the ghost nodes' lists, which the
 // list build wrote into the boundary particles' segments: no search of rows and
 // cells, only the fluid within 2h + skin of the node.  G lanes share a node and
@@ -2630,11 +2641,8 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
   if (act) {
     // the node's position in walk coordinates
     const float4 pb = walk[2 * (int64_t)i], g = st.ghost[i];
-    auto coord = [&](float p, float d) {  // (whole cells first: d may exceed 4 of them)
-      const float u = floorf(d * C.inv_csf);
-      return (int)((unsigned)__float_as_int(p) + (unsigned)walk_coord(C, (int)u, fmaf(-u, C.csf, d)));
-    };
-    const int qx = coord(pb.x, g.x), qy = coord(pb.y, g.y), qz = coord(pb.z, g.z);
+    const int qx = node_coord(C, pb.x, g.x), qy = node_coord(C, pb.y, g.y),
+              qz = node_coord(C, pb.z, g.z);
     const float unit = C.unit, r2max = C.r2max, hih = C.half_inv_h;
     auto visit = [&](int j) {
       float4 p, b;
@@ -2885,13 +2893,16 @@ __global__ void k_decide(cudaGraphConditionalHandle h, const ListCtl *__restrict
 // are counted with the list walk's own arithmetic (walk_r2; the cells of the
 // keys rule out what its wrapping positions alias) and compared with the pairs
 // its list yields.  Adds the brute-force pairs to ctl->check_pairs and every
-// mismatching target to ctl->check_bad.
+// mismatching target to ctl->check_bad.  ghost (or null): an mDBC boundary
+// target's list is that of the fluid around its ghost node, checked alike (no
+// pairs: not in check_pairs).
 __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
                              const uint32_t *__restrict__ keys, const float4 *__restrict__ posc,
                              const uint16_t *__restrict__ cid, const CaseConst *__restrict__ cc,
                              int nbits, const uint2 *__restrict__ list, int cap,
                              const uint16_t *__restrict__ count, ListCtl *__restrict__ ctl,
-                             int half, const float4 *__restrict__ walk) {
+                             int half, const float4 *__restrict__ walk,
+                             const float4 *__restrict__ ghost) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int nvalid = *nvalid_p;
   if (i >= nvalid || i >= n) return;
@@ -2900,17 +2911,26 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
   const bool afluid = !key_boundary(k, nbits);
   const int cidx = cid[i];
   const CaseConst &C = cc[cidx];
-  if (!afluid && C.bmode == 1) return;  // mDBC boundary: no pair terms (Eq 38 instead)
+  const bool node = !afluid && C.bmode == 1;  // mDBC boundary: no pair terms (Eq 38 instead)
+  if (node && !ghost) return;
   const float cs = C.csf;
-  const unsigned r2max_u = __float_as_uint(C.walk_r2max) - 1u;
-  const float4 pa = posc[i], wa = walk[2 * (int64_t)i];
+  const unsigned r2lo = node ? 0u : 1u, r2max_u = __float_as_uint(C.walk_r2max) - r2lo;
+  float4 pa = posc[i], wa = walk[2 * (int64_t)i];
+  if (node) {
+    const float4 g = ghost[i];
+    pa = make_float4(pa.x + g.x, pa.y + g.y, pa.z + g.z, pa.w);
+    wa = make_float4(__int_as_float(node_coord(C, wa.x, g.x)),
+                     __int_as_float(node_coord(C, wa.y, g.y)),
+                     __int_as_float(node_coord(C, wa.z, g.z)), wa.w);
+  }
   int cx, cy, cz;
   decode_cell(key_cell(k, nbits) - C.cellbase, C.nx, C.ny, cx, cy, cz);
   unsigned nb = 0u, nl = 0u;
   auto inside = [&](int j) {
+    if (j == i) return false;  // (a list's padding)
     float rx, ry, rz;
     const float r2 = walk_r2(wa, walk[2 * (int64_t)j], rx, ry, rz);
-    return __float_as_uint(r2) - 1u < r2max_u && walk[2 * (int64_t)j + 1].w != kGone;
+    return __float_as_uint(r2) - r2lo < r2max_u && walk[2 * (int64_t)j + 1].w != kGone;
   };
   for (int j = 0; j < nvalid; j++) {
     const uint32_t kj = keys[j];
@@ -2934,7 +2954,7 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
     for (int r = 0; r < (int)cw; r++)
       if (inside((int)reinterpret_cast<const uint32_t *>(seg)[r])) nl++;
   }
-  atomicAdd(&ctl->check_pairs, (unsigned long long)nb);
+  if (!node) atomicAdd(&ctl->check_pairs, (unsigned long long)nb);
   if (nb != nl) atomicAdd(&ctl->check_bad, 1ull);
 }
 
@@ -3611,10 +3631,10 @@ void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_
 void launch_list_check(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
                        const uint16_t *cid, const CaseConst *cc, int nbits, const uint2 *list,
                        int cap, const uint16_t *count, ListCtl *ctl, cudaStream_t s, bool half,
-                       const float4 *walk) {
+                       const float4 *walk, const float4 *ghost) {
   if (n > 0)
     k_list_check<<<nblk(n, 128), 128, 0, s>>>(n, nvalid, keys, posc, cid, cc, nbits, list, cap,
-                                              count, ctl, half ? 1 : 0, walk);
+                                              count, ctl, half ? 1 : 0, walk, ghost);
 }
 
 void launch_corrector_list(int n, const uint32_t *keys_n, const uint32_t *keys_half, State sn,

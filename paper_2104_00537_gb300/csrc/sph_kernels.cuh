@@ -125,11 +125,12 @@ void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_
                             int ncases, cudaStream_t s);
 // One-thread kernel: sets conditional handle h to ctl->rebuild != 0.
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s);
-// Brute-force check of the list against the evaluated state (tests).
+// Brute-force check of the list against the evaluated state (tests).  ghost (or
+// null): also of the ghost nodes' lists.
 void launch_list_check(int n, const int *nvalid, const uint32_t *keys, const float4 *posc,
                        const uint16_t *cid, const CaseConst *cc, int nbits, const uint2 *list,
                        int cap, const uint16_t *count, ListCtl *ctl, cudaStream_t s,
-                       bool half, const float4 *walk);
+                       bool half, const float4 *walk, const float4 *ghost = nullptr);
 void launch_corrector_list(int n, const uint32_t *keys_n, const uint32_t *keys_half, State sn,
                            const float4 *velrho_half, const float4 *ace, const CaseConst *cc,
                            CaseDyn *dyn, int nbits, State x, uint32_t *keys_next,

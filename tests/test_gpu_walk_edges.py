@@ -1,0 +1,62 @@
+"""Edges of the walks over flat lists that the ordinary cases do not reach."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2104_00537_gb300 import cases, sph
+from tests.test_gpu_list_eval import check_step_eval
+
+pytestmark = pytest.mark.gpu
+
+
+def check_boundary(case, g):
+    """Boundary values of an evaluated state (fixed walls) against the oracle's
+    Eq 38-39 on it, with the tolerances of test_gpu_mdbc."""
+    vel = g["vel"].astype(np.float64)
+    rho, vel_o, dets = oracle.mdbc(case, g["pos"], vel, g["rho"].astype(np.float64),
+                                   with_dets=True)
+    b = case.ptype == 1
+    ad = np.abs(dets)
+    sel = b & (np.abs(ad / 1e-3 - 1.0) >= 1e-3)  # (at the threshold either branch)
+    d = np.abs(g["rho"].astype(np.float64) - rho)
+    assert d[sel & (ad < 1e-3)].max(initial=0) < 1e-3
+    assert d[sel & (ad >= 1e-3) & (ad < 1e-2)].max(initial=0) < 0.1
+    assert d[sel & (ad >= 1e-2)].max(initial=0) < 0.01
+    vscale = max(np.abs(vel[~b]).max(), 1e-3)
+    assert np.abs(g["vel"][sel] - vel_o[sel]).max() < 1e-5 * vscale
+
+
+def lattice_at_ghosts(cell_mode):
+    """An mDBC dam break on the bare lattice, with noise in velocity (0.1 m/s) and
+    density (3 kg/m^3): the walls' mirror points fall on fluid particles.  Returns
+    it and the number of ghost nodes that lie on one to within 1e-9 dp."""
+    c = cases.dam_break(0.02, boundary_mode=1, mdbc_slip=1, cell_mode=cell_mode)
+    f = c.ptype == 0
+    dp = c.params["dp"]
+    c.pos[f] = np.round(c.pos[f] / dp) * dp
+    u = cases.uniform01(7, 4 * c.n_fluid).reshape(-1, 4) - 0.5
+    c.vel[f] = (0.2 * u[:, :3]).astype(np.float32)
+    c.rho[f] += (6.0 * u[:, 3]).astype(np.float32)
+    site = lambda x: set(map(tuple, np.round(x / dp).astype(int)))
+    b = ~f
+    node = c.pos[b] + c.ghost[b]
+    on = np.abs(node / dp - np.round(node / dp)).max(1) < 1e-9
+    return c, len(site(node[on]) & site(c.pos[f]))
+
+
+@pytest.mark.parametrize("cell_mode", [0, 1, 2])
+@pytest.mark.parametrize("variant", [5, 4, 3])
+def test_ghost_node_on_a_fluid_particle(variant, cell_mode):
+    """A fluid particle exactly on a ghost node has the largest weight of Eq 38-39
+    there: both evaluations of the first step against the oracle, and the nodes'
+    lists by brute force."""
+    c, hits = lattice_at_ghosts(cell_mode)
+    assert hits > 100
+    eng = sph.Engine.create(c)
+    eng.set_options(pi_variant=variant, check_list=1)
+    for stage in (0, 1):
+        g = eng.eval_step(stage)
+        check_boundary(c, g)
+    eng.step(3)
+    assert eng.list_info()["check_bad"] == 0
+    eng.destroy()

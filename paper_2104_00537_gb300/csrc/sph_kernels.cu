@@ -121,6 +121,12 @@ __device__ __forceinline__ int walk_coord(const CaseConst &C, int c, float off) 
   return (int)(((uint32_t)c << 29) + (uint32_t)__float2int_rn(p) + (uint32_t)__float2int_rn(e));
 }
 
+// Density bits in the record of a particle that left the domain at the half step:
+// it is still in the lists, but in no pair.  A NaN that put_walk writes for no
+// density, so that a case whose density is not finite is evaluated and reported.
+constexpr unsigned kGone = 0xffffdeadu;
+__device__ __forceinline__ bool walk_gone(float rho) { return __float_as_uint(rho) == kGone; }
+
 // The record the list walks gather for particle i (32 bytes, one sector):
 // {position as three walk_coord integers, P/rho}, {v, rho}.
 __device__ __forceinline__ void put_walk(float4 *walk, int i, const CaseConst &C, uint32_t key,
@@ -130,7 +136,7 @@ __device__ __forceinline__ void put_walk(float4 *walk, int i, const CaseConst &C
   walk[2 * (int64_t)i] = make_float4(__int_as_float(walk_coord(C, cx, p.x)),
                                      __int_as_float(walk_coord(C, cy, p.y)),
                                      __int_as_float(walk_coord(C, cz, p.z)), Q);
-  walk[2 * (int64_t)i + 1] = v;
+  walk[2 * (int64_t)i + 1] = make_float4(v.x, v.y, v.z, walk_gone(v.w) ? NAN : v.w);
 }
 
 // ---- upload ------------------------------------------------------------------
@@ -2023,10 +2029,6 @@ __device__ __forceinline__ float walk_r2(const float4 &a, const float4 &b, float
   return fmaf(rx, rx, fmaf(ry, ry, rz * rz));
 }
 
-// Density in the record of a particle that left the domain at the half step: it
-// is still in the lists, but in no pair.
-constexpr float kGone = -INFINITY;
-
 // One 32-byte walk record in one 256-bit load.
 __device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j, float4 &p,
                                           float4 &b) {
@@ -2076,7 +2078,7 @@ __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const 
       float rx, ry, rz;
       const float r2 = walk_r2(pa, u ? p2 : p1, rx, ry, rz);
       const float4 &b = u ? b2 : b1;
-      if (__float_as_uint(r2) - 1u < r2max_u && b.w != kGone)
+      if (__float_as_uint(r2) - 1u < r2max_u && !walk_gone(b.w))
         body(rx, ry, rz, r2, b, u ? p2.w : p1.w, u ? i2 : i1);
     }
   }
@@ -2093,7 +2095,7 @@ __device__ __forceinline__ void walk_list(const ListArgs &a, const int i, const 
         const float4 p = walk[2 * (int64_t)j], b = walk[2 * (int64_t)j + 1];
         float rx, ry, rz;
         const float r2 = walk_r2(pa, p, rx, ry, rz);
-        if (__float_as_uint(r2) - 1u < r2max_u && b.w != kGone) body(rx, ry, rz, r2, b, p.w, j);
+        if (__float_as_uint(r2) - 1u < r2max_u && !walk_gone(b.w)) body(rx, ry, rz, r2, b, p.w, j);
       }
     }
     __syncwarp();
@@ -2190,7 +2192,7 @@ __device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int 
                                                   int jb) {
   WalkTarget t;
   load_walk(a.walk, i, t.pa, t.va);  // (readable past the last particle)
-  t.has = i < nvalid && t.va.w != kGone;
+  t.has = i < nvalid && !walk_gone(t.va.w);
   t.afluid = t.has && i < jb;
   t.cidx = a.one_case || i >= a.n ? 0 : (int)a.cid[i];
   t.cw = t.has ? (unsigned)a.count[i] : 0u;
@@ -2307,8 +2309,9 @@ k_interact_list(const ListArgs a) {
   }
   __syncwarp();
   const int i = first + sub * NG;
-  const float rho = sub < a.per && i < nvalid ? a.walk[2 * (int64_t)i + 1].w : kGone;
-  const bool own = rho != kGone;
+  bool own = sub < a.per && i < nvalid;
+  const float rho = own ? a.walk[2 * (int64_t)i + 1].w : 0.f;
+  own = own && !walk_gone(rho);
   unsigned dtbits = kFloatInfBits;
   bool bad = false;
   int cidx = ccase;
@@ -2651,7 +2654,7 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
       const float dy = unit * (float)(qy - __float_as_int(p.y));
       const float dz = unit * (float)(qz - __float_as_int(p.z));
       const float rr2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      if (rr2 < r2max && b.w != kGone) S.add(C, hih, dx, dy, dz, rr2, b);
+      if (rr2 < r2max && !walk_gone(b.w)) S.add(C, hih, dx, dy, dz, rr2, b);
     };
     const unsigned cw = count[i];
     const uint2 *__restrict__ seg = list + (int64_t)i * cap;
@@ -2742,7 +2745,7 @@ __global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, St
     posc_out[i] = make_float4(1e30f, 1e30f, 1e30f, p.w);
     velrho_out[i] = v;
     keys_out[i] = key_out(nbits);
-    walk[2 * (int64_t)i + 1] = make_float4(0.f, 0.f, 0.f, kGone);  // in no pair
+    walk[2 * (int64_t)i + 1] = make_float4(0.f, 0.f, 0.f, __uint_as_float(kGone));  // in no pair
     atomicAdd(&dyn[cidx].n_out, 1);
     return;
   }
@@ -2930,7 +2933,7 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
     if (j == i) return false;  // (a list's padding)
     float rx, ry, rz;
     const float r2 = walk_r2(wa, walk[2 * (int64_t)j], rx, ry, rz);
-    return __float_as_uint(r2) - r2lo < r2max_u && walk[2 * (int64_t)j + 1].w != kGone;
+    return __float_as_uint(r2) - r2lo < r2max_u && !walk_gone(walk[2 * (int64_t)j + 1].w);
   };
   for (int j = 0; j < nvalid; j++) {
     const uint32_t kj = keys[j];

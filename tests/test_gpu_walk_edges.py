@@ -60,3 +60,19 @@ def test_ghost_node_on_a_fluid_particle(variant, cell_mode):
     eng.step(3)
     assert eng.list_info()["check_bad"] == 0
     eng.destroy()
+
+
+@pytest.mark.parametrize("variant,pair_once", [(5, 0), (4, 0), (3, 0), (5, 1), (4, 1), (0, 0)])
+@pytest.mark.parametrize("value", [-np.inf, np.inf, np.nan,
+                                   np.uint32(0xffffdead).view(np.float32)])
+def test_nonfinite_density_is_reported(variant, pair_once, value):
+    """A density that is not finite makes the evaluation fail on every path, also
+    the NaN that marks a record of a particle outside the domain."""
+    c = cases.dam_break(0.04)
+    f = np.nonzero(c.ptype == 0)[0]
+    c.rho[f[len(f) // 2]] = value
+    eng = sph.Engine.create(c)
+    eng.set_options(pi_variant=variant, pair_once=pair_once)
+    with pytest.raises(sph.SphError, match="NaN/Inf"):
+        eng.eval_step(0)
+    eng.destroy()

@@ -91,6 +91,11 @@ constexpr unsigned kFlagNaN = 1u, kFlagDtMin = 2u, kFlagQuota = 4u;
 // holds; a displacement since the list's build exceeded half its skin (or
 // one step's need exceeded the largest skin the rows cover)
 constexpr unsigned kFlagListFull = 8u, kFlagSkin = 16u;
+// a - b of two list-walk coordinates, modulo 2^32 (they change sign between the
+// cells 3 and 4 of every eight: a signed subtraction would overflow there).
+__host__ __device__ inline int walk_delta(int a, int b) {
+  return (int)((uint32_t)a - (uint32_t)b);
+}
 // A target's list: its candidates' indices (32 bits each; count = their
 // number), or, where they do not fit its segment, chunk records (first
 // candidate index, 32-bit mask) with count = kListRecords | their number.

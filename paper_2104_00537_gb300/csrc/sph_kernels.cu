@@ -2017,15 +2017,15 @@ struct ListArgs {
   int per;  // targets that a group of G lanes takes one after another (<= G)
 };
 
-// Relative position of two walk records, in units of cs / 2^29: the integer
-// differences wrap (period 8 cs), so cells and rows need no bookkeeping.
+// Relative position of two walk records, in units of cs / 2^29: the differences
+// wrap (walk_delta, period 8 cs), so cells and rows need no bookkeeping.
 // Listed particles lie within 2h + 2 skin < 5 cs of each other on every axis;
 // what aliases (beyond 4 cs) stays beyond 3 cs >= 2h, so it is no pair.
 __device__ __forceinline__ float walk_r2(const float4 &a, const float4 &b, float &rx, float &ry,
                                          float &rz) {
-  rx = (float)(__float_as_int(a.x) - __float_as_int(b.x));
-  ry = (float)(__float_as_int(a.y) - __float_as_int(b.y));
-  rz = (float)(__float_as_int(a.z) - __float_as_int(b.z));
+  rx = (float)walk_delta(__float_as_int(a.x), __float_as_int(b.x));
+  ry = (float)walk_delta(__float_as_int(a.y), __float_as_int(b.y));
+  rz = (float)walk_delta(__float_as_int(a.z), __float_as_int(b.z));
   return fmaf(rx, rx, fmaf(ry, ry, rz * rz));
 }
 
@@ -2650,9 +2650,9 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
     auto visit = [&](int j) {
       float4 p, b;
       load_walk(walk, j, p, b);
-      const float dx = unit * (float)(qx - __float_as_int(p.x));
-      const float dy = unit * (float)(qy - __float_as_int(p.y));
-      const float dz = unit * (float)(qz - __float_as_int(p.z));
+      const float dx = unit * (float)walk_delta(qx, __float_as_int(p.x));
+      const float dy = unit * (float)walk_delta(qy, __float_as_int(p.y));
+      const float dz = unit * (float)walk_delta(qz, __float_as_int(p.z));
       const float rr2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
       if (rr2 < r2max && !walk_gone(b.w)) S.add(C, hih, dx, dy, dz, rr2, b);
     };

@@ -138,9 +138,9 @@ typedef void (*sph_free_fn)(void *ptr, size_t bytes, void *stream, void *ctx);
 /* Engine-wide launch options (the autotuner's knobs). */
 typedef struct {
   int32_t pi_block;   /* threads per block of the list walk of the default
-                       * physics: 0 (default: 256), 128, 256, or 512 and
-                       * 1024 (run as 256: the walk keeps blocks small);
-                       * the other interaction kernels choose their own */
+                       * physics: 0 (default: 256), 128, 256, 512 or 1024;
+                       * the other interaction kernels (pair_once among
+                       * them) choose their own                           */
   int32_t pi_variant; /* interaction pair loop: -1 the engine default (5 where
                        * a list is supported, else 0); 0 compacted hit
                        * masks; 1 test

@@ -2205,9 +2205,12 @@ __device__ __forceinline__ WalkTarget walk_target(const ListArgs &a, int i, int 
 // from k_strain_list), for the cases that use them.  G lanes share a target;
 // a group takes a.per targets one after another (a warp covers 32 / G x per
 // consecutive targets), then lane q of the group finishes its q-th target, so
-// that the closing arithmetic runs on as many lanes as there are targets.
+// that the closing arithmetic runs on as many lanes as there are targets.  Blocks
+// of any number of warps (pi_block; EXT 1 and 2 take 256 threads): shared memory
+// by the launch, kWalkSums floats per thread.
+constexpr int kWalkSums = 6;
 template <int EXT, int G>
-__global__ void __launch_bounds__(256, EXT == 0 ? 4 : 0)
+__global__ void __launch_bounds__(EXT == 0 ? 1024 : 256, EXT == 0 ? 1 : 0)
 k_interact_list(const ListArgs a) {
   const int lane = threadIdx.x & 31;
   const int sub = lane % G;
@@ -2216,7 +2219,7 @@ k_interact_list(const ListArgs a) {
   const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (NG * a.per) + lane / G;
   const int nvalid = *a.nvalid_p;
   const int jb = (int)a.cstart[a.cap1 - 1];  // first boundary particle of the key order
-  __shared__ float s_k[8][32][6];  // the targets' sums, by the lane that finishes them
+  extern __shared__ float s_k[];  // the targets' sums, by the thread that finishes them
   unsigned npairs = 0u, nfb = 0u, nbf = 0u;
   int ccase = -1;  // case of the counts and of the constants below
   float hih = 0.f, eta2 = 0.f, kvc = 0.f;
@@ -2298,7 +2301,7 @@ k_interact_list(const ListArgs a) {
       A.mur = group_max<G>(A.mur);
     }
     if (sub == 0) {
-      float *k = s_k[threadIdx.x >> 5][(lane & ~(G - 1)) + q];
+      float *k = s_k + kWalkSums * ((threadIdx.x & ~(G - 1)) + q);
       k[0] = A.ax;
       k[1] = A.ay;
       k[2] = A.az;
@@ -2317,7 +2320,7 @@ k_interact_list(const ListArgs a) {
   int cidx = ccase;
   if (own) {
     cidx = a.one_case ? 0 : (int)a.cid[i];
-    const float *k = s_k[threadIdx.x >> 5][lane];
+    const float *k = s_k + kWalkSums * threadIdx.x;
     const float unit = a.cc[cidx].unit;  // the sums back from units of cs / 2^29
     const Acc K = {unit * k[0], unit * k[1], unit * k[2], unit * k[3], k[4],
                    a.cc[cidx].inv_unit * k[5], 0u, 0u};
@@ -3464,7 +3467,8 @@ void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const 
                    nbits, cc,    dyn,  ace,  want_dt, list, cap, count, tau4, tau2, mu, one_case ? 1 : 0, per};
   // block size of the default kernel as asked for (pi_block); its default 256,
   // and always for the others (registers)
-  const int b0 = block == 128 ? 128 : 256;
+  const int b0 = block == 128 || block == 512 || block == 1024 ? block : 256;
+  const size_t sh0 = sizeof(float) * kWalkSums * b0, sh = sizeof(float) * kWalkSums * 256;
   const int64_t threads = (n + (int64_t)per * (32 / G) - 1) / (per * (32 / G)) * 32;
 #define SPH_LANES(CALL) \
   switch (G) {          \
@@ -3485,15 +3489,15 @@ void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const 
 #define SPH_STR(GG) k_strain_list<GG><<<nblk(threads, 256), 256, 0, s>>>(a, tau4, tau2)
     SPH_LANES(SPH_STR)
 #undef SPH_STR
-#define SPH_L2(GG) k_interact_list<2, GG><<<nblk(threads, 256), 256, 0, s>>>(a)
+#define SPH_L2(GG) k_interact_list<2, GG><<<nblk(threads, 256), 256, sh, s>>>(a)
     SPH_LANES(SPH_L2)
 #undef SPH_L2
   } else if (ext) {
-#define SPH_L1(GG) k_interact_list<1, GG><<<nblk(threads, 256), 256, 0, s>>>(a)
+#define SPH_L1(GG) k_interact_list<1, GG><<<nblk(threads, 256), 256, sh, s>>>(a)
     SPH_LANES(SPH_L1)
 #undef SPH_L1
   } else {
-#define SPH_L0(GG) k_interact_list<0, GG><<<nblk(threads, b0), b0, 0, s>>>(a)
+#define SPH_L0(GG) k_interact_list<0, GG><<<nblk(threads, b0), b0, sh0, s>>>(a)
     SPH_LANES(SPH_L0)
 #undef SPH_L0
   }

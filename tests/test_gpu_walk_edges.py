@@ -76,3 +76,42 @@ def test_nonfinite_density_is_reported(variant, pair_once, value):
     with pytest.raises(sph.SphError, match="NaN/Inf"):
         eng.eval_step(0)
     eng.destroy()
+
+
+def walk_blocks(eng):
+    """Threads per block of the list walk's launches in one evaluation, from its
+    trace (the second session's: a process's first one misses launches, as does one
+    in which the list is built, by a conditional graph)."""
+    import json
+    import os
+    import tempfile
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            g = eng.eval_step(0)
+            torch.cuda.synchronize()
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "trace.json")
+        prof.export_chrome_trace(path)
+        with open(path) as f:
+            events = json.load(f)["traceEvents"]
+    kernels = [e for e in events if e.get("cat") == "kernel"]
+    if not kernels:
+        pytest.skip("no kernel trace on this machine")
+    return g, {e["args"]["block"][0] for e in kernels if "k_interact_list" in e["name"]}
+
+
+def test_pi_block_is_the_walk_s_block():
+    """pi_block threads per block (0: 256), the same sums bit for bit."""
+    eng = sph.Engine.create(cases.dam_break(0.03))
+    ref = None
+    for block in (0, 128, 256, 512, 1024):
+        eng.set_options(pi_block=block)
+        g, used = walk_blocks(eng)
+        assert used == {block or 256}
+        if ref is None:
+            ref = g
+        for k in ("acc", "drho", "mumax", "dt", "pairs"):
+            assert np.array_equal(g[k], ref[k]), (block, k)
+    eng.destroy()

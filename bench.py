@@ -277,15 +277,15 @@ def measure_batched(ncases, steps, warmup, tune, clock_index=0, pair_once=0, fix
     time the same steps (warmup .. warmup + steps of every case from rest)
     with CUDA events on the engines' stream.  tune: pick cell size and
     interaction variant and list-walk block size with the autotuner (else
-    cells of h, kept list, 128 threads).  pair_once: both paths evaluate each
+    cells of h, kept list, the engine's block size).  pair_once: both paths evaluate each
     pair once (atomic sums: the two paths then agree to rounding, not bit for
     bit, and their pair counts may differ by the pairs at the cut-off)."""
     import torch
     from paper_2104_00537_gb300 import autotune, cases, sph
     stream = torch.cuda.Stream()
     cs = cases.batch_dam_breaks(ncases, seed=0)
-    cm, var, block, tune_ms = 1, 5, 128, None
-    if fixed:  # (cell_mode, pi_variant, pi_block) of an earlier tuning
+    cm, var, block, tune_ms = 1, 5, 0, None
+    if fixed:  # (cell_mode, pi_variant, pi_block)
         cm, var, block = fixed
     elif tune:
         mk = lambda cc: sph.Engine.batch(cc, stream=stream)
@@ -695,8 +695,9 @@ def main():
         b = out["batched"]
         out["batched_" + other] = measure_batched(
             256, 500, 3, tune=False, clock_index=local, pair_once=1 - po,
-            fixed=(b["cell_mode"], b["pi_variant"], b["pi_block"]))
-        out["batched_" + other]["note"] = "as batched, both paths with pair_once = %d" % (1 - po)
+            fixed=(b["cell_mode"], b["pi_variant"], 0))  # (a block tuned for the other mode)
+        out["batched_" + other]["note"] = "as batched, both paths with pair_once = %d and the engine's " \
+                                           "block size" % (1 - po)
         out["served"] = measure_served(48, 20.0, 200000, 0.1, 10, pair_once=po)
         out["served"]["note"] = ("C4 scaled to fit the run: 48 requests, fluid <= 200k, "
                                  "0.1 s simulated (C4: 100+ requests, <= 2M, 1 s; run with "

@@ -4,8 +4,9 @@ For a set of cases it times a few Symplectic steps of each candidate
 configuration on the device (CUDA events inside libsph) and keeps the fastest.
 The search has two stages: the cell size (cells of 2h, h or 2h/3, i.e. the
 cells a target's support spans per axis) crossed with the interaction
-variant, then, for the winner if it walks a neighbour list, the thread-block
-size of that walk.  Results are cached in a JSON file keyed by (GPU name,
+variant, then, for the winner if it walks a neighbour list whose launches take
+it (the default physics, each target its own pairs), the thread-block size of
+that walk.  Every entry is timed with the block size of its name.  Results are cached in a JSON file keyed by (GPU name,
 case count bucket, particle count bucket) so that later runs on the same kind
 of GPU and workload skip the search.
 """
@@ -17,6 +18,7 @@ import os
 CANDIDATES = [(1, 4), (1, 5), (2, 4), (2, 5), (0, 4), (1, 3), (1, 0), (2, 0), (1, 1), (0, 0)]
 # threads per block of the list walk (pi_variant 3-5)
 BLOCKS = (128, 256, 512)
+BLOCK0 = 128  # the first stage's
 
 
 def cache_path() -> str:
@@ -86,17 +88,21 @@ def tune(cases, make_engine, gpu_name: str, steps=3, warmup=2, candidates=CANDID
     list walk applies).  The cases' cell_mode is restored afterwards."""
     key = bucket_key(gpu_name, cases, pair_once)
     cache = _load() if use_cache else {}
-    if key in cache and len(cache[key].get("best", ())) == 3:
+    # (entries without a block0 were timed at another block size than they name)
+    if (key in cache and len(cache[key].get("best", ())) == 3
+            and cache[key].get("block0") == BLOCK0):
         return tuple(cache[key]["best"]), cache[key].get("times", {})
     times = {}
     saved = [c.params.get("cell_mode", 0) for c in cases]
     try:
         for cm, var in candidates:
-            times["%d,%d,128" % (cm, var)] = _time(cases, make_engine, cm, var, 0, steps, warmup,
-                                                   pair_once)
+            times["%d,%d,%d" % (cm, var, BLOCK0)] = _time(cases, make_engine, cm, var, BLOCK0,
+                                                          steps, warmup, pair_once)
         best_s = min(times, key=times.get)
         cm, var, _ = (int(x) for x in best_s.split(","))
-        if var in (3, 4, 5):
+        plain = not any(c.params.get("visc_mode") == 1 or c.params.get("ddt_mode") == 2
+                        for c in cases)
+        if var in (3, 4, 5) and plain and not pair_once:
             for b in blocks:
                 k = "%d,%d,%d" % (cm, var, b)
                 if k not in times:
@@ -107,6 +113,6 @@ def tune(cases, make_engine, gpu_name: str, steps=3, warmup=2, candidates=CANDID
     best_s = min(times, key=times.get)
     best = tuple(int(x) for x in best_s.split(","))
     if use_cache:
-        cache[key] = {"best": list(best), "times": times}
+        cache[key] = {"best": list(best), "times": times, "block0": BLOCK0}
         _store(cache)
     return best, times

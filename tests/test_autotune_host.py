@@ -5,6 +5,8 @@ size of its list walk, restores the cases' cell size, and caches the result
 per (GPU, case-count bucket, particle-count bucket)."""
 import json
 
+import pytest
+
 from paper_2104_00537_gb300 import autotune
 
 
@@ -81,3 +83,42 @@ def test_configuration_that_cannot_run_is_skipped(tmp_path, monkeypatch):
                                 candidates=[(2, 5), (1, 4)], use_cache=False)
     assert times["2,5,128"] == float("inf")
     assert best[:2] == (1, 4)
+
+
+class RecordingEngine(FakeEngine):
+    """Notes the block size of every run under (cell mode, variant)."""
+    ran = []
+
+    def step(self, n):
+        RecordingEngine.ran.append((self.cm, self.var, self.block))
+        super().step(n)
+
+
+def test_every_entry_is_timed_at_its_own_block(tmp_path, monkeypatch):
+    monkeypatch.setenv("SPH_AUTOTUNE_CACHE", str(tmp_path / "cache.json"))
+    RecordingEngine.ran.clear()
+    _, times = autotune.tune([FakeCase(5000)], RecordingEngine, "GB300")
+    assert {"%d,%d,%d" % r for r in RecordingEngine.ran} == set(times)
+    assert {"1,5,128", "1,5,256", "1,5,512"} <= set(times)
+
+
+@pytest.mark.parametrize("pair_once,params", [(1, {}), (0, {"visc_mode": 1}),
+                                              (0, {"ddt_mode": 2})])
+def test_no_block_search_where_the_walk_has_its_own(tmp_path, monkeypatch, pair_once, params):
+    """pi_block is for the default physics' walk of each target's own pairs."""
+    monkeypatch.setenv("SPH_AUTOTUNE_CACHE", str(tmp_path / "cache.json"))
+    case = FakeCase(5000)
+    case.params.update(params)
+    best, times = autotune.tune([case], FakeEngine, "GB300", pair_once=pair_once)
+    assert best == (1, 5, 128)
+    assert all(k.endswith(",128") for k in times)
+
+
+def test_entries_of_an_earlier_search_are_not_reused(tmp_path, monkeypatch):
+    """A cached entry that does not say which block size its first stage ran with."""
+    monkeypatch.setenv("SPH_AUTOTUNE_CACHE", str(tmp_path / "cache.json"))
+    cases = [FakeCase(5000)]
+    key = autotune.bucket_key("GB300", cases)
+    (tmp_path / "cache.json").write_text(json.dumps({key: {"best": [0, 4, 128], "times": {}}}))
+    best, _ = autotune.tune(cases, FakeEngine, "GB300")
+    assert best == (1, 5, 256)

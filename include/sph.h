@@ -195,9 +195,11 @@ typedef struct {
                        * admitted a case with other physics) evaluate as
                        * with 0.  0 (default): every target sums its own
                        * pairs, deterministically                         */
-  int32_t wide_records; /* 0 or 1, of no effect: lists hold 32-bit indices
-                       * at every size (it once chose between two record
-                       * forms, with the same results bit for bit)        */
+  int32_t wide_records; /* 0 or 1.  1: pi_variant 3 of an engine with the
+                       * default physics (not a pool) runs as 4, with
+                       * pair_once too.  No other effect: lists hold 32-bit
+                       * indices at every size (it once chose between two
+                       * record forms, of which 3 wrote only one)          */
 } sph_options;
 
 /* Last error message of the calling thread ("" if none). */

@@ -338,7 +338,8 @@ class Engine:
         check_list: brute-force check of every list evaluation (list_info);
         pi_lanes: threads per target of the list walk (0: the default);
         pair_once: evaluate each pair once (atomic sums, not bit-reproducible);
-        wide_records: of no effect (lists hold 32-bit indices at every size)."""
+        wide_records: 1 takes variant 3 to 4 (default physics, not in pools), else of
+        no effect."""
         o = Options(pi_block, pi_variant, use_graph, timing, list_skin, check_list, pi_lanes,
                     pair_once, wide_records)
         check(self.lib.sph_set_options(self.h, C.byref(o)))

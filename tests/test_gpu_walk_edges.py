@@ -115,3 +115,18 @@ def test_pi_block_is_the_walk_s_block():
         for k in ("acc", "drho", "mumax", "dt", "pairs"):
             assert np.array_equal(g[k], ref[k]), (block, k)
     eng.destroy()
+
+
+def test_wide_records_takes_variant_3_to_4():
+    """wide_records 1 changes one thing: pi_variant 3 runs as 4."""
+    eng = sph.Engine.create(cases.dam_break(0.03))
+    runs = {}
+    for variant in (3, 4, 5):
+        for wide in (0, 1):
+            eng.set_options(pi_variant=variant, wide_records=wide)
+            runs[variant, wide] = eng.eval_step(0)["acc"]
+    assert np.array_equal(runs[3, 1], runs[4, 0])
+    assert not np.array_equal(runs[3, 0], runs[4, 0])  # (sums in another order)
+    for v in (4, 5):
+        assert np.array_equal(runs[v, 1], runs[v, 0])
+    eng.destroy()

@@ -3629,6 +3629,8 @@ void launch_corrector_reuse(int n, const uint32_t *keys_n, const uint32_t *keys_
     k_corrector_reuse<<<nblk(n, 256), 256, 0, s>>>(n, keys_n, keys_half, y, velrho_half, ace,
                                                    ref, cc, dyn, nbits, x, keys_next, press,
                                                    ctl, walk, ncases);
+  else  // (only cases without particles: they step all the same)
+    launch_end_step(ncases, cc, dyn, s);
 }
 
 void launch_decide(cudaGraphConditionalHandle h, const ListCtl *ctl, cudaStream_t s) {

@@ -130,3 +130,22 @@ def test_wide_records_takes_variant_3_to_4():
     for v in (4, 5):
         assert np.array_equal(runs[v, 1], runs[v, 0])
     eng.destroy()
+
+
+def test_empty_case_keeps_its_time():
+    """A pool whose only particles belong to a case just released still steps its
+    case without particles: no pair bounds dt, so t advances by cfl h / cs0."""
+    c = cases.dam_break(0.04)
+    e = cases.dam_break(0.04)
+    for k in ("pos", "vel", "rho", "ptype", "group", "ghost"):
+        setattr(e, k, getattr(e, k)[:0])
+    pool = sph.Engine.pool(50000, 400000, 2)
+    a = pool.admit(c, t_end=1.0)
+    b = pool.admit(e, t_end=1.0)
+    pool.pool_step(1)
+    t0 = pool.stats(b)["t"]
+    assert t0 > 0
+    pool.release(a)
+    pool.pool_step(3)
+    assert pool.stats(b)["t"] == pytest.approx(4 * t0, rel=1e-12)
+    pool.destroy()

@@ -197,6 +197,7 @@ struct sph_engine_t {
   int cap_cases = 0;
   int nbits = 0;
   int margin = 0;  // shared by all cases (0: not set yet)
+  int sms = 0;         // SMs of the device
   int integrator = 0;  // 0 Symplectic (Eq 33-34), 1 Verlet (Eq 30-31), all cases
   bool ext = false;    // a case uses Eq 19-20 diffusion or laminar + SPS viscosity
   bool sps = false;    // a case uses laminar + SPS viscosity (tau buffers below)
@@ -459,6 +460,9 @@ int init_engine(sph_engine e, void *stream, sph_alloc_fn alloc, sph_free_fn free
   e->alloc = alloc;
   e->freefn = freefn;
   e->ctx = ctx;
+  int dev = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&e->sms, cudaDevAttrMultiProcessorCount, dev));
   if (stream) {
     e->s = (cudaStream_t)stream;
   } else {
@@ -684,7 +688,7 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
                        e->dconst, e->ddyn, 0, e->walk, e->nlist, e->list_cap, e->ncount, s);
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
-                         e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
+                         e->ncount, e->ext, tau4, e->tau2, s, e->sms, mu, e->opt.pi_block,
                          e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
                          e->cap_cases == 1);
   } else if (e->opt.pi_variant == 4) {  // list alone, then both evaluations over it
@@ -697,7 +701,7 @@ void enqueue_list_first(sph_engine e, cudaEvent_t *ev, float *mu) {
                       e->mdbc ? Y.ghost : nullptr);
     launch_interact_list(nl, e->nvalid, e->keysB, e->walk, Y.cid, e->cstart, e->cells_hw,
                          e->nbits, e->dconst, e->ddyn, e->ace, 1, e->nlist, e->list_cap,
-                         e->ncount, e->ext, tau4, e->tau2, s, mu, e->opt.pi_block,
+                         e->ncount, e->ext, tau4, e->tau2, s, e->sms, mu, e->opt.pi_block,
                          e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
                          e->cap_cases == 1);
   } else {
@@ -740,9 +744,9 @@ void enqueue_list_half(sph_engine e, cudaEvent_t *ev, float *mu) {
   if (ev) cudaEventRecord(ev[2], s);
   launch_interact_list(nl, e->nvalid, e->keysC, e->walk, Y.cid, e->cstart, e->cells_hw,
                        e->nbits, e->dconst, e->ddyn, e->ace, 0, e->nlist, e->list_cap, e->ncount,
-                       e->ext, e->sps ? e->tau4 : nullptr, e->tau2, s, mu, e->opt.pi_block,
-                       e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr, e->sym_mu,
-                         e->cap_cases == 1);
+                       e->ext, e->sps ? e->tau4 : nullptr, e->tau2, s, e->sms, mu,
+                       e->opt.pi_block, e->opt.pi_lanes, sym_on(e) ? e->sym_sum : nullptr,
+                       e->sym_mu, e->cap_cases == 1);
   if (ev) cudaEventRecord(ev[3], s);
   if (e->opt.check_list)
     launch_list_check(nl, e->nvalid, e->keysC, Z.posc, Y.cid, e->dconst, e->nbits, e->nlist,

@@ -3433,14 +3433,14 @@ void launch_mdbc(int margin, int n, const int *nvalid, const uint32_t *keys, Sta
 }
 
 // Targets that a group of G lanes takes one after another: as many (at most G)
-// as leave 128 warps per SM, some five rounds of its resident ones.  More
+// as leave 128 warps per SM (sms of them), some five rounds of its resident ones.  More
 // targets per group share the closing arithmetic, but fewer, longer warps leave
 // the last round emptier.  Measured per evaluation at 1 / 2 / 4 / 8 targets
 // (G = 8): 28k particles 12 / 16 / 27 / 47 us, 167k 91 / 81 / 82 / 91, batch of
 // 420k 305 / 260 / 246 / 248, 1.5M 736 / 635 / 598 / 586.
-static inline int walk_targets(int n, int G) {
+static inline int walk_targets(int n, int G, int sms) {
   int per = 1;
-  while (per < G && (int64_t)n * G / 32 / (2 * per) >= 152 * 128) per *= 2;
+  while (per < G && (int64_t)n * G / 32 / (2 * per) >= sms * 128) per *= 2;
   return per;
 }
 
@@ -3458,11 +3458,11 @@ void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const 
                           const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,
                           int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
-                          float4 *tau4, float2 *tau2, cudaStream_t s, float *mu, int block,
+                          float4 *tau4, float2 *tau2, cudaStream_t s, int sms, float *mu, int block,
                           int lanes, float4 *sym_sum, unsigned *sym_mu, bool one_case) {
   if (n <= 0) return;
   const int G = lanes == 1 || lanes == 2 || lanes == 4 ? lanes : 8;
-  const int per = walk_targets(n, G);
+  const int per = walk_targets(n, G, sms);
   const ListArgs a{n,    nvalid, keys, walk, cid,   cstart, (uint32_t)(cap_cells + 1),
                    nbits, cc,    dyn,  ace,  want_dt, list, cap, count, tau4, tau2, mu, one_case ? 1 : 0, per};
   // block size of the default kernel as asked for (pi_block); its default 256,

@@ -98,13 +98,14 @@ void launch_interact_build(int margin, int n, const int *nvalid, const uint32_t 
                            int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace,
                            uint2 *list, int cap, uint16_t *count, bool ext, float4 *tau4,
                            float2 *tau2, cudaStream_t s, float *mu = nullptr);
-// The interaction over the lists of the state whose records are in walk.
+// The interaction over the lists of the state whose records are in walk; sms: the
+// device's SM count.
 void launch_interact_list(int n, const int *nvalid, const uint32_t *keys, const float4 *walk,
                           const uint16_t *cid, const uint32_t *cstart, int64_t cap_cells,
                           int nbits, const CaseConst *cc, CaseDyn *dyn, float4 *ace, int want_dt,
                           const uint2 *list, int cap, const uint16_t *count, bool ext,
-                          float4 *tau4, float2 *tau2, cudaStream_t s, float *mu = nullptr,
-                          int block = 0, int lanes = 0, float4 *sym_sum = nullptr,
+                          float4 *tau4, float2 *tau2, cudaStream_t s, int sms,
+                          float *mu = nullptr, int block = 0, int lanes = 0, float4 *sym_sum = nullptr,
                           unsigned *sym_mu = nullptr, bool one_case = false);
 // The walk records of a state (posc, velrho, press in the cells of keys).
 void launch_pack_walk(int n, const uint32_t *keys, const float4 *posc, const float4 *velrho,

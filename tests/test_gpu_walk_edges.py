@@ -149,3 +149,115 @@ def test_empty_case_keeps_its_time():
     pool.pool_step(3)
     assert pool.stats(b)["t"] == pytest.approx(4 * t0, rel=1e-12)
     pool.destroy()
+
+
+def targets_per_group(n, lanes=8, sms=152):
+    """The walk's rule: as many targets (at most the lanes) one after another as
+    leave 128 warps per SM."""
+    per = 1
+    while per < lanes and n * lanes // 32 // (2 * per) >= sms * 128:
+        per *= 2
+    return per
+
+
+@pytest.mark.parametrize("dp,per", [(0.0097, 1), (0.0095, 2), (0.0072, 4), (0.0055, 8)])
+@pytest.mark.parametrize("pair_once", [0, 1])
+def test_several_targets_per_group(dp, per, pair_once):
+    """Either side of every size at which a lane group takes more targets: both
+    evaluations against the oracle."""
+    case = cases.dam_break(dp)
+    assert targets_per_group(case.n) == per
+    eng = sph.Engine.create(case)
+    eng.set_options(use_graph=1, pair_once=pair_once)
+    eng.step(2)
+    for stage in (0, 1):
+        check_step_eval(case, eng, stage, exact_pairs=False)
+    eng.destroy()
+
+
+@pytest.mark.parametrize("kw", [dict(visc_mode=1, nu0=1e-3), dict(ddt_mode=2),
+                                dict(boundary_mode=1), dict(integrator=1)])
+def test_several_targets_per_group_of_other_physics(kw):
+    case = cases.dam_break(0.0085, **kw)
+    assert targets_per_group(case.n) > 1
+    eng = sph.Engine.create(case)
+    eng.step(2)
+    for stage in (0,) if "integrator" in kw else (0, 1):
+        check_step_eval(case, eng, stage, exact_pairs=False)
+    eng.destroy()
+
+
+@pytest.mark.parametrize("lanes", [0, 4, 2, 1])
+def test_groups_across_cases(lanes):
+    """Groups whose targets belong to different cases (fluid and boundary ranges
+    of 14 uneven cases, few of them a multiple of 32): every case bit for bit as alone,
+    where its groups take one target each, with its own pair counts and dt."""
+    cs = cases.batch_dam_breaks(14, seed=5, n_min=5000, n_max=60000)
+    assert targets_per_group(sum(c.n for c in cs)) == 8
+    assert all(targets_per_group(c.n) == 1 for c in cs)
+    bat = sph.Engine.batch(cs)
+    bat.set_options(use_graph=1, pi_lanes=lanes)
+    once = sph.Engine.batch(cs)
+    once.set_options(use_graph=1, pair_once=1, pi_lanes=lanes)
+    first = [once.eval_step(0, i) for i in range(len(cs))]
+    bat.step(4)
+    for i, c in enumerate(cs):
+        e = sph.Engine.create(c)
+        e.set_options(use_graph=1, pi_lanes=lanes)
+        g = e.eval_step(0)
+        assert first[i]["pairs"] == g["pairs"], i
+        assert first[i]["dt"] == pytest.approx(g["dt"], rel=1e-5), i
+        scale = np.abs(g["acc"]).max()
+        assert np.abs(first[i]["acc"] - g["acc"]).max() < 1e-5 * scale, i
+        e.step(4)
+        a, b = e.get_state(), bat.get_state(i)
+        for k in ("pos", "vel", "rho", "t"):
+            assert np.array_equal(a[k], b[k]), (i, k)
+        sa, sb = e.stats(), bat.stats(i)
+        for k in ("interactions", "interactions_fb", "interactions_bf", "last_dt", "flags"):
+            assert sa[k] == sb[k], (i, k)
+        e.destroy()
+    bat.destroy()
+    once.destroy()
+
+
+def crowded_wall(cell_mode=1, **kw):
+    """A dam break whose fluid near the middle of the x = 0 wall is drawn together:
+    more candidates around it than a list segment holds as indices (256 at cells
+    of 2h and h), so that fluid targets, and the ghost nodes of an mDBC wall, keep
+    chunk records."""
+    from scipy.spatial import cKDTree
+    c = cases.dam_break(0.04, cell_mode=cell_mode, **kw)
+    f = c.ptype == 0
+    h = c.params["h"]
+    mid = c.pos[f].mean(0)
+    mid[0] = c.pos[f][:, 0].min()
+    d = c.pos - mid
+    near = f & (np.linalg.norm(d, axis=1) < 3.5 * h)
+    c.pos[near] = mid + 0.62 * d[near]
+    u = cases.uniform01(11, 3 * c.n_fluid).reshape(-1, 3) - 0.5
+    c.vel[f] = (0.2 * u).astype(np.float32)
+    tree = cKDTree(c.pos[f])
+    where = c.pos[c.ptype == 1] + c.ghost[c.ptype == 1] if kw.get("boundary_mode") else c.pos[f]
+    most = max(len(x) for x in tree.query_ball_point(where, 2.0 * h))
+    assert most > 256, most
+    return c
+
+
+@pytest.mark.parametrize("cell_mode", [0, 1])
+@pytest.mark.parametrize("kw", [dict(visc_mode=1, nu0=1e-3), dict(ddt_mode=2),
+                                dict(boundary_mode=1, mdbc_slip=1), dict(integrator=1)])
+def test_kept_records_of_other_physics(kw, cell_mode):
+    """Targets that keep chunk records in the walks of laminar + SPS (with its
+    strain pass), Fourtakas diffusion, mDBC (whose ghost nodes keep records too)
+    and Verlet, against the oracle and by brute force."""
+    c = crowded_wall(cell_mode, **kw)
+    eng = sph.Engine.create(c)
+    eng.set_options(pi_variant=5, check_list=1)
+    for stage in (0,) if "integrator" in kw else (0, 1):
+        g = check_step_eval(c, eng, stage)
+        if "boundary_mode" in kw:
+            check_boundary(c, g)
+    eng.step(1)
+    assert eng.list_info()["check_bad"] == 0
+    eng.destroy()

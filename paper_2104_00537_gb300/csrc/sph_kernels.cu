@@ -16,6 +16,7 @@
 
 #include "sph_internal.cuh"
 #include "sph_kernels.cuh"
+#include "sph_disp.cuh"
 
 namespace sph {
 
@@ -45,42 +46,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 __device__ __forceinline__ float below(float cs) {  // largest float < cs
   return __int_as_float(__float_as_int(cs) - 1);
-}
-
-// A displacement as the unevaluated sum of two FP32 numbers (48 bits; products of
-// dt, itself split, with FP32 velocities).  FP64 runs at 1/74 of the FP32 rate here
-// and, with its conversions, bound the predictor (60 us for 1.48M particles) and the
-// corrector (65 us); an error-free FP32 sum of offset and displacement takes ten
-// FP32 operations.
-struct Disp {
-  float hi, lo;
-};
-__device__ __forceinline__ Disp disp_scaled(const float (&c)[2], float v) {  // (c[0] + c[1]) v
-  Disp d;
-  d.hi = __fmul_rn(c[0], v);
-  d.lo = fmaf(c[1], v, fmaf(c[0], v, -d.hi));
-  return d;
-}
-__device__ __forceinline__ Disp disp_sum(const Disp &a, const Disp &b) {
-  Disp d;
-  d.hi = __fadd_rn(a.hi, b.hi);
-  const float t = __fsub_rn(d.hi, a.hi);
-  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(d.hi, t)), __fsub_rn(b.hi, t));
-  d.lo = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-  return d;
-}
-__device__ __forceinline__ Disp disp_of(double x) {
-  Disp d;
-  d.hi = (float)x;
-  d.lo = (float)(x - (double)d.hi);
-  return d;
-}
-// off + d, rounded once to FP32 (the sum of off and d.hi with its exact error,
-// Knuth's two-sum)
-__device__ __forceinline__ float add_disp(float off, const Disp &d) {
-  const float s = __fadd_rn(off, d.hi), t = __fsub_rn(s, off);
-  const float e = __fadd_rn(__fsub_rn(off, __fsub_rn(s, t)), __fsub_rn(d.hi, t));
-  return __fadd_rn(s, __fadd_rn(e, d.lo));
 }
 
 // New offset after adding disp to a float offset in [0, cs); returns the cell
@@ -114,7 +79,13 @@ __device__ __forceinline__ int shift_axis(float off, const Disp &disp, const Cas
 // Position of the list walks along one axis: the cell index modulo 8 and the
 // offset in units of cs / 2^29, as one wrapping 32-bit integer.  The offset's
 // product with 2^29 / cs is formed in two FP32 parts, so the integer is within
-// one unit (2^-29 cs) of it: the FP32 offset itself is rounded to 2^-25 cs.
+// one unit of it.  FP32 offsets are spaced 2^-25 cs and more above cs / 2, finer
+// below 2^-5 cs.  Over random pairs the component error of r_ab against the exact
+// one, in cs (largest / rms; FP32 offsets and cell differences in brackets):
+// 3.2e-8 / 1.5e-8 (7.7e-8 / 2.4e-8) at cells of 2h, 6.2e-8 / 2.9e-8 (1.7e-7 /
+// 4.2e-8) of h, 1.2e-7 / 4.8e-8 (2.6e-7 / 7.6e-8) of 2h/3; below 2e-4 h apart the
+// FP32 form is the finer one, and particles closer than a unit on every axis
+// (2^-29 cs) count as coincident: no pair, as at distance zero.
 __device__ __forceinline__ int walk_coord(const CaseConst &C, int c, float off) {
   const float p = off * C.fix_hi;
   const float e = fmaf(off, C.fix_lo, fmaf(off, C.fix_hi, -p));
@@ -1808,7 +1779,7 @@ __global__ void k_end_step(int ncases, const CaseConst *__restrict__ cc,
 
 // ---- Symplectic predictor / corrector ------------------------------------------
 
-// Moves a particle by disp (FP64, per axis) from the cell of key k; returns
+// Moves a particle by disp (two FP32 parts per axis) from the cell of key k; returns
 // the new key (or key_out) and writes the new offsets.
 __device__ __forceinline__ uint32_t move_particle(uint32_t k, const float4 &p, const Disp disp[3],
                                                   const CaseConst &C, bool boundary, int nbits,
@@ -1832,7 +1803,7 @@ __device__ __forceinline__ uint32_t move_particle(uint32_t k, const float4 &p, c
   return key_make(C.cellbase + lin, boundary, nbits);
 }
 
-// Eq 33-34 half step of one particle: displacement dt/2 v^n (FP64) and
+// Eq 33-34 half step of one particle: displacement dt/2 v^n (48 bits) and
 // v, rho at n+1/2; boundary particles: density only (clamped), moving ones
 // displaced by Eq 37 at t + dt/2.
 __device__ __forceinline__ void predictor_core(const CaseConst &C, const CaseDyn &D,
@@ -1904,7 +1875,7 @@ __global__ void k_predictor(int n, const uint32_t *__restrict__ keys_in, State s
 
 // Eq 33-34 full step of one particle from state n (key k, pn, vn), the
 // half-step density rhoh and F, R at n+1/2 (a): the new position (cell +
-// offset, FP64 displacement), velocity and density; returns the new key.
+// offset, rounded once), velocity and density; returns the new key.
 __device__ __forceinline__ uint32_t corrector_core(const CaseConst &C, const CaseDyn &D,
                                                    uint8_t code, uint32_t k, const float4 &pn,
                                                    const float4 &vn, float rhoh, const float4 &a,
@@ -2701,9 +2672,10 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
 // cells as state n (Eq 33-34 as k_predictor); a particle that leaves the
 // domain is frozen at state n and moved out of every list's reach.  The
 // displacement since the list's build (from ref, else the half step alone)
-// must stay within half the skin (kFlagSkin).
+// must stay within half the skin (kFlagSkin).  Five blocks per SM: 48 registers (50,
+// and four blocks, without the bound; times at add_disp).
 template <bool REF>
-__global__ void k_predictor_list(int n, const uint32_t *__restrict__ keys_in, State src,
+__global__ void __launch_bounds__(256, 5) k_predictor_list(int n, const uint32_t *__restrict__ keys_in, State src,
                                  const float4 *__restrict__ ace,
                                  const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
                                  int nbits, float4 *__restrict__ posc_out,
@@ -2811,8 +2783,9 @@ __global__ void k_corrector_list(int n, const uint32_t *__restrict__ keys_n,
 // |r - r_build| + 1.25 (dt_max / 2) |v| <= (skin - 1e-3 h) / 2 (dt_max the
 // Eq 35 bound: the displacement at n+1 and the most the next half step
 // adds); otherwise, or when a particle leaves the domain, the corrector
-// requests a rebuild.  It also ends the step (end_step): a launch less.
-__global__ void k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
+// requests a rebuild.  It also ends the step (end_step): a launch less.  Five blocks
+// per SM, as the predictor.
+__global__ void __launch_bounds__(256, 5) k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
                                   const uint32_t *__restrict__ keys_half, State y,
                                   const float4 *__restrict__ velrho_half,
                                   const float4 *__restrict__ ace, const float4 *__restrict__ ref,
@@ -2969,7 +2942,7 @@ __global__ void k_list_check(int n, const int *__restrict__ nvalid_p,
 // One Verlet step (Eq 30, or Eq 31 when the case's count of completed steps
 // is a multiple of N_S) from the sorted state n (src, with v^{n-1}, rho^{n-1}
 // in src.vrprev) and F^n, R^n (ace) to state n+1 in dst, same order:
-//   r^{n+1} = r^n + dt v^n + dt^2 F^n / 2            (FP64 displacement)
+//   r^{n+1} = r^n + dt v^n + dt^2 F^n / 2            (48 bits, rounded once)
 //   v^{n+1} = v^{n-1} + 2 dt F^n   |  v^n + dt F^n    (Eq 30 | Eq 31)
 //   rho^{n+1} = rho^{n-1} + 2 dt R^n | rho^n + dt R^n
 // and v^n, rho^n become dst.vrprev.  Boundary particles: density as above

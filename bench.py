@@ -337,7 +337,7 @@ def measure_served(requests, rate, max_fluid, t_end, chunk, cell_mode=1, pi_vari
     for _, c, _ in trace:
         c.params["cell_mode"] = cell_mode
     free, _ = torch.cuda.mem_get_info()
-    # about 200 B of state and 1.5 KB of per-step list per particle slot
+    # about 240 B of state and 1.5 KB of list per particle slot
     max_p = int(min(free * 0.3 / 1800, max_particles or 16_000_000))
     max_cells = int(min(free * 0.05 / 8, 200_000_000))
     results = {}
@@ -496,7 +496,7 @@ def main():
                     pi_lanes=args.pi_lanes, pair_once=args.pair_once)
     n_particles = sum(c.n for c in cs)
     # the pi_variant the engine runs (its default: 5, the list kept across
-    # steps; beyond 2^25 particles with wide records, for the default physics)
+    # steps; beyond 2^25 particles for the default physics only)
     default_physics = (args.ddt_mode != 2 and args.visc_mode == 0 and args.boundary_mode == 0)
     list_ok = n_particles < (1 << 25) or default_physics
     default_var = 5
@@ -696,8 +696,8 @@ def main():
         out["batched_" + other] = measure_batched(
             256, 500, 3, tune=False, clock_index=local, pair_once=1 - po,
             fixed=(b["cell_mode"], b["pi_variant"], 0))  # (a block tuned for the other mode)
-        out["batched_" + other]["note"] = "as batched, both paths with pair_once = %d and the engine's " \
-                                           "block size" % (1 - po)
+        out["batched_" + other]["note"] = ("as batched, both paths with pair_once = %d and the "
+                                           "engine's block size" % (1 - po))
         out["served"] = measure_served(48, 20.0, 200000, 0.1, 10, pair_once=po)
         out["served"]["note"] = ("C4 scaled to fit the run: 48 requests, fluid <= 200k, "
                                  "0.1 s simulated (C4: 100+ requests, <= 2M, 1 s; run with "

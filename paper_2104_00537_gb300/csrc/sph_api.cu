@@ -128,12 +128,16 @@ void fill_const(const sph_case_params &p, const sph_particles &parts, const Grid
   C.wk = (float)aD;
   C.list_k = (float)(1.25 * (p.dt_fixed > 0 ? p.dt_fixed : p.cfl * p.h / p.cs0));
   // The kept list's default skin.  A wider one is rebuilt less often and walked
-  // longer.  Measured at 0.04 / 0.055 / 0.07 / 0.09 (us per step): 6k particles
-  // 89 / 84 / 80 / 78, 28k 72 / 68 / 66 / 64, 167k 249 / 244 / 244 / 250, 410k Verlet
-  // 244 / 235 / 237 / 244, 1.5M 1377 / 1372 / 1410 / 1513, batch of 420k 769 / 737 /
-  // 744 / 764; SPS 270k 563 / 572 / 588 / 627, mDBC 190k 347 / 354 / 358 / 375 (their
-  // evaluations cost more beside a build).  By the case alone, so that it takes the
-  // same steps in any engine.
+  // longer.  us per step at 0.04 / 0.055 / 0.07 / 0.08, dam breaks of 31k particles
+  // 62 / 59 / 58 / 56, 35k 68 / 63 / 62 / 60, 55k 82 / 77 / 77 / 75, 90k 106 / 102 /
+  // 101 / 100, 125k 134 / 129 / 130 / 131; at 0.04 / 0.055 / 0.07 / 0.09 6k 89 / 84 /
+  // 80 / 78, 167k 249 / 244 / 244 / 250, 410k Verlet 244 / 235 / 237 / 244, 1.5M
+  // 1377 / 1372 / 1410 / 1513, batch of 420k 769 / 737 / 744 / 764.  (0.08 wins up to
+  // about 100k: below 32,768 the gain is 5 %, above it falls to 3 % and ends.)
+  // Evaluations that cost more beside a build, at 0.03 / 0.04 / 0.055 / 0.08: SPS 28k
+  // 93 / 89 / 86 / 85, 83k 179 / 174 / 173 / 174, 427k 847 / 857 / 873 / 937; mDBC 51k
+  // 121 / 119 / 117 / 118, 109k 189 / 183 / 186 / 186, 430k 576 / 579 / 596 / 618.  By
+  // the case alone, so that it takes the same steps in any engine.
   C.list_extra = p.visc_mode == 1 || p.boundary_mode == 1 ? 0.04f
                  : parts.n < 32768                        ? 0.08f
                                                           : 0.055f;

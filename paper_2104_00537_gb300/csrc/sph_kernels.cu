@@ -2014,7 +2014,8 @@ __device__ __forceinline__ void load_walk(const float4 *__restrict__ walk, int j
 // load an iteration ahead; see flatten_records) and gathers both walk records
 // before it uses either: the lanes of a target take neighbouring entries and, the
 // list being in cell order, mostly neighbouring particles.
-// body(rx, ry, rz, r2, b, Qb, j) runs for every candidate inside the support; positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
+// body(rx, ry, rz, r2, b, Qb, j) runs for every candidate inside the support;
+// positions in units of cs / 2^29, b = {v, rho}, Qb = P/rho.
 // A lane without an entry takes the target itself (r2 = 0: no pair).
 // What bounds it (1.48M particles, 0.53 ms): L1 gathers (data pipe 78 % of its peak)
 // and issue (68 %) together.  Measured and left out, per evaluation: the records
@@ -2675,13 +2676,13 @@ k_mdbc_list(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict_
 // must stay within half the skin (kFlagSkin).  Five blocks per SM: 48 registers (50,
 // and four blocks, without the bound; times at add_disp).
 template <bool REF>
-__global__ void __launch_bounds__(256, 5) k_predictor_list(int n, const uint32_t *__restrict__ keys_in, State src,
-                                 const float4 *__restrict__ ace,
-                                 const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
-                                 int nbits, float4 *__restrict__ posc_out,
-                                 float4 *__restrict__ velrho_out, uint32_t *__restrict__ keys_out,
-                                 float *__restrict__ press, const float4 *__restrict__ ref,
-                                 float4 *__restrict__ walk) {
+__global__ void __launch_bounds__(256, 5)
+k_predictor_list(int n, const uint32_t *__restrict__ keys_in, State src,
+                 const float4 *__restrict__ ace, const CaseConst *__restrict__ cc,
+                 CaseDyn *__restrict__ dyn, int nbits, float4 *__restrict__ posc_out,
+                 float4 *__restrict__ velrho_out, uint32_t *__restrict__ keys_out,
+                 float *__restrict__ press, const float4 *__restrict__ ref,
+                 float4 *__restrict__ walk) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   // every load of the particle first (independent: one memory latency)
@@ -2785,14 +2786,14 @@ __global__ void k_corrector_list(int n, const uint32_t *__restrict__ keys_n,
 // adds); otherwise, or when a particle leaves the domain, the corrector
 // requests a rebuild.  It also ends the step (end_step): a launch less.  Five blocks
 // per SM, as the predictor.
-__global__ void __launch_bounds__(256, 5) k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
-                                  const uint32_t *__restrict__ keys_half, State y,
-                                  const float4 *__restrict__ velrho_half,
-                                  const float4 *__restrict__ ace, const float4 *__restrict__ ref,
-                                  const CaseConst *__restrict__ cc, CaseDyn *__restrict__ dyn,
-                                  int nbits, State x, uint32_t *__restrict__ keys_next,
-                                  float *__restrict__ press, ListCtl *__restrict__ ctl,
-                                  float4 *__restrict__ walk, int ncases) {
+__global__ void __launch_bounds__(256, 5)
+k_corrector_reuse(int n, const uint32_t *__restrict__ keys_n,
+                  const uint32_t *__restrict__ keys_half, State y,
+                  const float4 *__restrict__ velrho_half, const float4 *__restrict__ ace,
+                  const float4 *__restrict__ ref, const CaseConst *__restrict__ cc,
+                  CaseDyn *__restrict__ dyn, int nbits, State x,
+                  uint32_t *__restrict__ keys_next, float *__restrict__ press,
+                  ListCtl *__restrict__ ctl, float4 *__restrict__ walk, int ncases) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   // the end of the step, which nothing else in this kernel reads or writes
   for (int c = i; c < ncases; c += gridDim.x * blockDim.x) end_step(c, cc, dyn);
@@ -3405,8 +3406,8 @@ void launch_mdbc(int margin, int n, const int *nvalid, const uint32_t *keys, Sta
 #undef SPH_MD
 }
 
-// Targets that a group of G lanes takes one after another: as many (at most G)
-// as leave 128 warps per SM (sms of them), some five rounds of its resident ones.  More
+// Targets that a group of G lanes takes one after another: as many (at most G) as
+// leave 128 warps for each of the sms SMs, some five rounds of its resident ones.  More
 // targets per group share the closing arithmetic, but fewer, longer warps leave
 // the last round emptier.  Measured per evaluation at 1 / 2 / 4 / 8 targets
 // (G = 8): 28k particles 12 / 16 / 27 / 47 us, 167k 91 / 81 / 82 / 91, batch of

@@ -182,6 +182,7 @@ struct Slot {
   uint32_t cellbase = 0;
   int64_t ncells = 0;
   double t_end = 0;
+  int records = 0;  // list_records_needed of the case (0: no list)
 };
 
 inline size_t align256(size_t b) { return (b + 255) / 256 * 256; }
@@ -352,6 +353,10 @@ int list_records_needed(int cell_mode, double h, double dp) {
       }
   return std::min(4096, ((int)std::ceil(1.2 * worst) + 31) / 32 * 32);
 }
+
+// Candidates up to which a target's list is plain indices: by the case alone.  Twice
+// its list_records_needed (256 or 384).
+int list_entries(int records) { return 2 * std::max(32, records); }
 
 // A neighbour list applies to this step: a list variant chosen (3, 4: one
 // list per Symplectic step; 5: kept across steps, either scheme) and the
@@ -529,7 +534,7 @@ int upload_case(sph_engine e, int slot, const sph_particles *parts, int64_t dst0
 }
 
 int set_slot(sph_engine e, int slot, const sph_case_params *p, const sph_particles *parts,
-             const Grid &g, uint32_t cellbase, double t_end) {
+             const Grid &g, uint32_t cellbase, double t_end, int records) {
   int64_t nf = 0;
   for (int64_t i = 0; i < parts->n; i++) nf += parts->type[i] == 0;
   Slot &S = e->slots[slot];
@@ -540,7 +545,10 @@ int set_slot(sph_engine e, int slot, const sph_case_params *p, const sph_particl
   S.cellbase = cellbase;
   S.ncells = g.ncells;
   S.t_end = t_end;
+  S.records = records;
   fill_const(*p, *parts, g, cellbase, t_end, nf, e->hconst[slot]);
+  e->hconst[slot].flat_max =
+      std::min(2 * e->list_cap, list_entries(records));
   CUDA_TRY(cudaMemcpyAsync(e->dconst + slot, &e->hconst[slot], sizeof(CaseConst),
                            cudaMemcpyHostToDevice, e->s));
   CaseDyn d;
@@ -605,10 +613,13 @@ int create_engine(const sph_case_params *params, const sph_particles *parts, int
     e->list_ok = true;
     e->list_wide = e->list_wide_needed = true;
   }
+  std::vector<int> records(ncases, 0);
   if (e->list_ok) {
     int cap = 32;
-    for (int c = 0; c < ncases; c++)
-      cap = std::max(cap, list_records_needed(params[c].cell_mode, params[c].h, params[c].dp));
+    for (int c = 0; c < ncases; c++) {
+      records[c] = list_records_needed(params[c].cell_mode, params[c].h, params[c].dp);
+      cap = std::max(cap, records[c]);
+    }
     e->list_cap = cap;
     // the list kept across steps (one list per step, 4, makes every case of a
     // batch take the same steps as alone, bit for bit)
@@ -618,7 +629,7 @@ int create_engine(const sph_case_params *params, const sph_particles *parts, int
   rc = allocate(e);
   int64_t cell0 = 0, p0 = 0;
   for (int c = 0; c < ncases && rc == SPH_OK; c++) {
-    rc = set_slot(e, c, params + c, parts + c, grids[c], (uint32_t)cell0, 0.0);
+    rc = set_slot(e, c, params + c, parts + c, grids[c], (uint32_t)cell0, 0.0, records[c]);
     if (rc == SPH_OK) rc = upload_case(e, c, parts + c, p0);
     cell0 += grids[c].ncells;
     p0 += parts[c].n;
@@ -1833,7 +1844,9 @@ int sph_pool_admit(sph_engine e, const sph_case_params *params, const sph_partic
   e->ext = e->ext || params->ddt_mode == 2 || params->visc_mode == 1;
   e->sps = e->sps || params->visc_mode == 1;
   e->mdbc = e->mdbc || params->boundary_mode == 1;
-  if (e->list_ok && list_records_needed(params->cell_mode, params->h, params->dp) > e->list_cap)
+  const int records =
+      e->list_ok ? list_records_needed(params->cell_mode, params->h, params->dp) : 0;
+  if (records > e->list_cap)
     e->list_ok = false;  // from now on the pool runs two neighbour lists per step
   e->opt.pi_variant = resolve_variant(e, e->opt.pi_variant);
   // the half lists of the pair-once walk no longer serve: every case rebuilds
@@ -1859,7 +1872,7 @@ int sph_pool_admit(sph_engine e, const sph_case_params *params, const sph_partic
   e->free_cells[fr].first += g.ncells;
   if (e->free_cells[fr].first == e->free_cells[fr].second)
     e->free_cells.erase(e->free_cells.begin() + fr);
-  rc = set_slot(e, free_slot, params, parts, g, (uint32_t)cb, t_end);
+  rc = set_slot(e, free_slot, params, parts, g, (uint32_t)cb, t_end, records);
   if (rc == SPH_OK) rc = upload_case(e, free_slot, parts, e->n_phys);
   if (rc) return rc;
   e->n_phys += parts->n;

@@ -61,6 +61,7 @@ struct CaseConst {
   float unit, inv_unit, fix_hi, fix_lo;
   float walk_r2max, walk_eta2, walk_hih;
   float list_extra;  // the kept list's default skin beyond one step's need, x 2h
+  int flat_max;      // most candidates of a target kept as plain indices
   float list_k;   // 1.25 x the Eq 35 bound on dt (or the fixed dt): skin = list_k |v|max + 1e-3 h
 };
 
@@ -97,7 +98,7 @@ __host__ __device__ inline int walk_delta(int a, int b) {
   return (int)((uint32_t)a - (uint32_t)b);
 }
 // A target's list: its candidates' indices (32 bits each; count = their
-// number), or, where they do not fit its segment, chunk records (first
+// number), or, where they are more than its case's flat_max, chunk records (first
 // candidate index, 32-bit mask) with count = kListRecords | their number.
 constexpr unsigned kListRecords = 0x8000u;
 // engines beyond this size keep lists for the default physics only

@@ -724,8 +724,10 @@ __global__ void k_need_all(int ncases, CaseDyn *__restrict__ dyn) {
 // neighbouring particles (walk of 1.48M particles 527 us; 544 with two 32-bit index
 // loads, 631 with candidates e and e + 1).  The warp takes its 32 targets one by
 // one: the records go to registers, then each record's candidates are written by
-// the lanes whose bit is set.  A target whose candidates do not fit, or with more
-// than 128 records, keeps its records (kListRecords in its count).  Issue-bound,
+// the lanes whose bit is set.  A target with more candidates than flat_max (its
+// case's, at most 2 cap: a case keeps the same lists in every engine, whatever its
+// segments), or with more than 128 records, keeps its records (kListRecords in its
+// count).  Issue-bound,
 // some 16 warp-instructions per record: the whole-list build of 1.48M particles
 // takes 1.24 ms with it and 0.74 without, once in eight to twelve steps, for a walk
 // without masks, rows and bit scans (733 to 527 us, twice a step).
@@ -740,7 +742,7 @@ __device__ __forceinline__ void store_if(bool on, uint32_t *p, uint32_t v) {
                :: "l"(p), "r"(v), "r"((unsigned)on) : "memory");
 }
 __device__ __forceinline__ void flatten_records(int i, bool build, int nrec,
-                                                uint2 *__restrict__ list, int cap,
+                                                int flat_max, uint2 *__restrict__ list, int cap,
                                                 uint16_t *__restrict__ count) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -772,7 +774,7 @@ __device__ __forceinline__ void flatten_records(int i, bool build, int nrec,
       total += __shfl_sync(full, x, 31);
     }
     const int n16 = (total + 15) & ~15;
-    const bool flat = nr <= 32 * kFlatRounds && n16 <= 2 * cap;
+    const bool flat = nr <= 32 * kFlatRounds && n16 <= __shfl_sync(full, flat_max, t);
     if (lane == t) mine = flat ? n16 : (int)kListRecords | nr;
     if (!flat) continue;
     __syncwarp();  // every record is in registers before its memory is overwritten
@@ -1065,7 +1067,7 @@ k_interact(int n, const int *__restrict__ nvalid_p, const uint32_t *__restrict__
 
   if (LIST) {
     if (has && lcnt > cap) atomicOr(&dyn[cidx].flags, kFlagListFull);
-    flatten_records(i, i < n && lmode != 0, min(lcnt, cap), list, cap, count);
+    flatten_records(i, i < n && lmode != 0, min(lcnt, cap), C.flat_max, list, cap, count);
   }
   if (LIST >= 2) return;
   finish_target(C, i, n, cidx, has, afluid, va, A, want_dt, ace, mu_out, dyn);

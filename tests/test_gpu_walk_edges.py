@@ -261,3 +261,35 @@ def test_kept_records_of_other_physics(kw, cell_mode):
     eng.step(1)
     assert eng.list_info()["check_bad"] == 0
     eng.destroy()
+
+
+@pytest.mark.parametrize("cell_mode", [0, 1])
+@pytest.mark.parametrize("skin", [-1.0, 0.25])
+def test_crowded_case_takes_the_same_steps_in_a_pool(cell_mode, skin):
+    """A pool's list segments are larger than an engine's of the case alone.  Targets
+    whose candidates fit only the larger one (257 to 384 of them) are summed in the
+    same order in both: the same steps bit for bit."""
+    from scipy.spatial import cKDTree
+    c = cases.dam_break(0.04, cell_mode=cell_mode)
+    f = c.ptype == 0
+    h = c.params["h"]
+    mid = c.pos[f].mean(0)
+    d = c.pos - mid
+    near = f & (np.linalg.norm(d, axis=1) < 3.0 * h)
+    c.pos[near] = mid + 0.88 * d[near]
+    most = max(map(len, cKDTree(c.pos).query_ball_point(c.pos[f], 2.16 * h)))  # 2h + skin
+    assert 256 < most < 384, most
+    pool = sph.Engine.pool(60000, 600000, 3)
+    pool.set_options(list_skin=skin)
+    pool.admit(cases.dam_break(0.04, seed=5, cell_mode=cell_mode), t_end=1.0)
+    s = pool.admit(c, t_end=1.0)
+    pool.pool_step(5)
+    alone = sph.Engine.create(c)
+    alone.set_options(list_skin=skin, check_list=1)
+    alone.step(5)
+    assert alone.list_info()["check_bad"] == 0
+    a, b = alone.get_state(), pool.get_state(s)
+    for k in ("pos", "vel", "rho"):
+        assert np.array_equal(a[k], b[k]), k
+    alone.destroy()
+    pool.destroy()

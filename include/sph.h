@@ -172,7 +172,8 @@ typedef struct {
                        * kept, as a fraction of 2h, in [0, 0.25]; < 0: the
                        * default (per case: 0.04 with laminar + SPS or
                        * mDBC, else 0.08 below 32,768 particles, 0.055 from
-                       * there on)                                         */
+                       * there on).  Above 0.1 the engine's list segments
+                       * grow with it (8 bytes per two candidates more)    */
   int32_t check_list; /* 1: after every list evaluation, count the pairs of
                        * every target, and the fluid around every ghost node
                        * of an mDBC case, by brute force and compare (tests;

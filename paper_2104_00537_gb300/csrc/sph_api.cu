@@ -282,6 +282,17 @@ struct sph_engine_t {
     if (p) allocs.push_back({p, bytes});
     return p;
   }
+  void dfree(void *p) {  // a block of dalloc's, with nothing in flight that uses it
+    for (size_t i = 0; i < allocs.size(); i++) {
+      if (allocs[i].first != p) continue;
+      if (freefn)
+        freefn(p, allocs[i].second, (void *)s, ctx);
+      else
+        cudaFree(p);
+      allocs.erase(allocs.begin() + (ptrdiff_t)i);
+      return;
+    }
+  }
   void drop_graphs() {
     if (gexec) cudaGraphExecDestroy(gexec);
     gexec = nullptr;
@@ -354,9 +365,17 @@ int list_records_needed(int cell_mode, double h, double dp) {
   return std::min(4096, ((int)std::ceil(1.2 * worst) + 31) / 32 * 32);
 }
 
-// Candidates up to which a target's list is plain indices: by the case alone.  Twice
-// its list_records_needed (256 or 384).
-int list_entries(int records) { return 2 * std::max(32, records); }
+// Candidates up to which a target's list is plain indices: by the case and the
+// list_skin option alone.  Twice its list_records_needed (256 or 384), which a skin
+// up to 0.1 x 2h fills to some 90 %.  A wider one gets room for the sphere it reaches
+// x 1.25 (0.25: 480): with 256 most targets of 1.48M particles kept chunk records at
+// 0.25, and a step took 4.64 ms instead of 1.80.
+int list_entries(int records, double h, double dp, float skin) {
+  const int base = 2 * std::max(32, records);
+  if (skin <= 0.1f) return base;
+  const double r = (2.0 * h * (1.0 + (double)skin) + 0.05 * h) / dp;
+  return std::max(base, ((int)std::min(1000.0, 1.25 * 4.18879 * r * r * r) + 31) / 16 * 16);
+}
 
 // A neighbour list applies to this step: a list variant chosen (3, 4: one
 // list per Symplectic step; 5: kept across steps, either scheme) and the
@@ -548,7 +567,7 @@ int set_slot(sph_engine e, int slot, const sph_case_params *p, const sph_particl
   S.records = records;
   fill_const(*p, *parts, g, cellbase, t_end, nf, e->hconst[slot]);
   e->hconst[slot].flat_max =
-      std::min(2 * e->list_cap, list_entries(records));
+      std::min(2 * e->list_cap, list_entries(records, p->h, p->dp, e->opt.list_skin));
   CUDA_TRY(cudaMemcpyAsync(e->dconst + slot, &e->hconst[slot], sizeof(CaseConst),
                            cudaMemcpyHostToDevice, e->s));
   CaseDyn d;
@@ -557,6 +576,41 @@ int set_slot(sph_engine e, int slot, const sph_case_params *p, const sph_particl
   d.need = 1u;  // a new case builds its list
   CUDA_TRY(cudaMemcpyAsync(e->ddyn + slot, &d, sizeof(CaseDyn), cudaMemcpyHostToDevice, e->s));
   e->list_dirty = true;
+  CUDA_TRY(cudaStreamSynchronize(e->s));
+  return SPH_OK;
+}
+
+// Longer list segments for a list_skin that asks for them (once: they stay), and
+// every case's flat_max for it.  Where the memory is not to be had the segments stay
+// as they are, and targets with more candidates keep chunk records.
+int grow_list(sph_engine e) {
+  if (!e->list_ok) return SPH_OK;
+  const float skin = e->opt.list_skin;
+  int need = 0;
+  if (e->pool)  // (as its segments at creation)
+    need = list_entries(0, 1.2 * std::sqrt(3.0), 1.0, skin);
+  for (auto &s : e->slots)
+    if (s.used) need = std::max(need, list_entries(s.records, s.params.h, s.params.dp, skin));
+  if (need > 2 * e->list_cap) {
+    const int64_t N = e->cap_p > 0 ? e->cap_p : 1;
+    if (void *p = e->dalloc(sizeof(uint2) * (size_t)(need / 2) * (size_t)N)) {
+      e->dfree(e->nlist);
+      e->nlist = (uint2 *)p;
+      e->list_cap = need / 2;
+    } else {
+      cudaGetLastError();  // (the failed cudaMalloc's)
+    }
+  }
+  for (int c = 0; c < e->cap_cases; c++) {
+    if (!e->slots[c].used) continue;
+    const Slot &S = e->slots[c];
+    const int fm =
+        std::min(2 * e->list_cap, list_entries(S.records, S.params.h, S.params.dp, skin));
+    if (fm == e->hconst[c].flat_max) continue;
+    e->hconst[c].flat_max = fm;
+    CUDA_TRY(cudaMemcpyAsync(e->dconst + c, &e->hconst[c], sizeof(CaseConst),
+                             cudaMemcpyHostToDevice, e->s));
+  }
   CUDA_TRY(cudaStreamSynchronize(e->s));
   return SPH_OK;
 }
@@ -1124,7 +1178,7 @@ int sph_set_options(sph_engine e, const sph_options *opt) {
   e->opt.pi_variant = resolve_variant(e, opt->pi_variant);
   e->list_stale = true;  // another pair loop may have run in between
   e->drop_graphs();
-  return SPH_OK;
+  return grow_list(e);
 }
 
 int sph_step(sph_engine e, int64_t nsteps) {

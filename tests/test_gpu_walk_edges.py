@@ -293,3 +293,32 @@ def test_crowded_case_takes_the_same_steps_in_a_pool(cell_mode, skin):
         assert np.array_equal(a[k], b[k]), k
     alone.destroy()
     pool.destroy()
+
+
+@pytest.mark.parametrize("pooled", [0, 1])
+def test_wide_skin_grows_the_list_segments(pooled):
+    """list_skin above 0.1: longer list segments in the place of the first ones
+    (4 bytes per candidate), kept when the skin narrows again; every pair is found
+    and the evaluations match the oracle throughout."""
+    import torch
+    c = cases.dam_break(0.03)
+    if pooled:
+        eng = sph.Engine.pool(60000, 600000, 2)
+        icase, slots = eng.admit(c, t_end=10.0), 60000
+    else:
+        eng, icase, slots = sph.Engine.create(c), 0, c.n
+    bytes_of = torch.cuda.memory_allocated
+    for skin in (-1.0, 0.25, 0.12, 0.0, -1.0):
+        b0 = bytes_of()
+        eng.set_options(list_skin=skin, check_list=1)
+        grown = (bytes_of() - b0) / slots
+        if skin == 0.25:
+            # 480 entries instead of 256; a pool's (h up to 1.2 sqrt(3) dp) 800 of 384
+            assert abs(grown - (4 * 416 if pooled else 4 * 224)) < 4 * 16, grown
+        else:
+            assert grown == 0
+        eng.step(3)
+        assert eng.list_info()["check_bad"] == 0
+        for stage in (0, 1):
+            check_step_eval(c, eng, stage, icase=icase)
+    eng.destroy()
